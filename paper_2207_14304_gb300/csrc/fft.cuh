@@ -1,10 +1,10 @@
-// Batched 2-D FFTs of square power-of-two tiles (T = 256, 512, 1024) in shared
-// memory: Stockham auto-sort passes of radix 8 (then 4 or 2 to finish), a
-// twiddle table of e^{-2 pi i m / T} built in double precision on the host,
-// one kernel for the rows and one for the columns (the columns are loaded
-// transposed into padded shared rows).  Forward transforms are unnormalised,
-// inverse transforms are unscaled (the caller divides by T^2), as in numpy.
-// The real type is float (image data) or double (PSF transforms).
+// FFTs of square power-of-two tiles (T = 256, 512, 1024): Stockham auto-sort
+// passes of radix 8 (then 4 or 2 to finish) with a twiddle table of
+// e^{-2 pi i m / T} built in double precision on the host.  Forward transforms
+// are unnormalised, inverse transforms are unscaled (the caller divides by T^2),
+// as in numpy.  The real type is float (image data) or double (PSF transforms).
+// The first half states the butterflies and a pass over a sequence in memory
+// (what the CPU tests run); the second half is the register form the kernels run.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -87,31 +87,6 @@ FFT_HD void stockham_pass(const C* a, C* b, const C* tw, int Ns, int lane, int n
     }
 }
 
-// All passes over one sequence: radix 8 while 8 Ns <= T, then 4 or 2.
-// a and b are this sequence's two shared buffers; returns the one holding the
-// result.  Every thread of the CTA calls it (barriers inside).
-template <int T, int S, typename C>
-__device__ __forceinline__ C* stockham(C* a, C* b, const C* tw, int lane, int nlanes) {
-    int Ns = 1;
-    while (Ns < T) {
-        if (Ns * 8 <= T) {
-            stockham_pass<T, 8, S>(a, b, tw, Ns, lane, nlanes);
-            Ns *= 8;
-        } else if (Ns * 4 <= T) {
-            stockham_pass<T, 4, S>(a, b, tw, Ns, lane, nlanes);
-            Ns *= 4;
-        } else {
-            stockham_pass<T, 2, S>(a, b, tw, Ns, lane, nlanes);
-            Ns *= 2;
-        }
-        __syncthreads();
-        C* t = a;
-        a = b;
-        b = t;
-    }
-    return a;
-}
-
 // Sequences per CTA and threads per sequence for a T-point transform.
 template <int T, typename R> struct Shape {
     static constexpr int SEQ = (sizeof(R) == 4 ? 16 : 8) / (T > 512 ? 2 : 1);
@@ -121,47 +96,120 @@ template <int T, typename R> struct Shape {
     static constexpr size_t SMEM = (2 * (size_t)SEQ * PAD + T) * sizeof(typename Cx<R>::T);
 };
 
-// FFT along the rows (COLS = false) or the columns (COLS = true) of n_tiles
-// tiles [n][T][T] of complex values, in place.  S = -1 forward, +1 inverse.
-template <int T, int S, bool COLS, typename R>
-__global__ void __launch_bounds__(Shape<T, R>::THREADS) fft_pass_kernel(typename Cx<R>::T* data, int n_tiles,
-                                                                      const typename Cx<R>::T* tw_global) {
-    using C = typename Cx<R>::T;
-    using Sh = Shape<T, R>;
-    extern __shared__ __align__(16) unsigned char fft_smem[];
-    C* buf = reinterpret_cast<C*>(fft_smem);
-    C* tw = buf + 2 * Sh::SEQ * Sh::PAD;
-    for (int i = threadIdx.x; i < T; i += Sh::THREADS) tw[i] = tw_global[i];
-    const long blocks_per_tile = T / Sh::SEQ;
-    const long tile = blockIdx.x / blocks_per_tile;
-    const int s0 = (int)(blockIdx.x % blocks_per_tile) * Sh::SEQ;   // first row or column
-    if (tile >= n_tiles) return;                                    // uniform per CTA
-    C* base = data + tile * (long)T * T;
-    // load: sequence s of this CTA into buf[s * PAD ...]
-    for (int e = threadIdx.x; e < Sh::SEQ * T; e += Sh::THREADS) {
-        if (COLS) {
-            const int y = e / Sh::SEQ, c = e - y * Sh::SEQ;           // SEQ consecutive columns per row
-            buf[c * Sh::PAD + y] = base[(long)y * T + s0 + c];
-        } else {
-            const int s = e / T, x = e - s * T;
-            buf[s * Sh::PAD + x] = base[(long)(s0 + s) * T + x];
+// ---------------------------------------------------------------------------
+// The transforms the kernels run: one T-point sequence on T / 8 lanes, eight
+// values per lane in registers, lane l holding elements l + m T/8 (m = 0..7)
+// before and after, so a transform can start from and end in global memory with
+// consecutive lanes on consecutive elements, and a forward transform, a
+// pointwise product and an inverse one chain without leaving the registers.
+// Radices 8, 8, 4 (T = 256), 8, 8, 8 (512) and 8, 8, 4, 4 (1024); between two
+// passes the values cross through shared memory once (position p at p + p / 8:
+// the strided writes of a pass then fall on different banks), alternating
+// between two buffers so that a crossing needs one barrier.  The version that
+// kept the sequence in shared memory through all passes (one load, three
+// read-modify-write passes, one store) ran at 1.7 TB/s on 216 tiles of 512^2.
+template <int T> struct Reg {
+    static constexpr int LANES = T / 8;
+    static constexpr int CB = T == 256 ? 8 : 4;           // sequences per CTA and columns per block of the layout
+    static constexpr int THREADS = LANES * CB;
+    static constexpr int PT = T + T / 8;                  // padded shared sequence
+    static constexpr int NTW = T == 256 ? 13 : T == 512 ? 14 : 16;   // twiddles a lane uses
+};
+
+// Index into the twiddle table of slot i of a lane: pass 2 (radix 8, Ns = 8) in
+// slots 0..6, then pass 3 (and 4), per butterfly.
+template <int T> FFT_HD int tw_index(int i, int lane) {
+    if (i < 7) return ((i + 1) * (lane & 7) * (T / 64)) & (T - 1);
+    i -= 7;
+    if (T == 512) return ((i + 1) * lane) & (T - 1);                           // radix 8, Ns = 64
+    if (T == 256) return ((i % 3 + 1) * (lane + (i / 3) * (T / 8))) & (T - 1); // radix 4, Ns = 64
+    if (i < 3) return ((i + 1) * (lane & 63) * (T / 256)) & (T - 1);           // radix 4, Ns = 64
+    i -= 3;
+    return ((i % 3 + 1) * (lane + (i / 3) * (T / 8))) & (T - 1);               // radix 4, Ns = 256
+}
+
+// Twiddles of a lane, held in registers (FP32) or read from the table as they
+// are needed (FP64, where the arithmetic hides the reads).
+template <int T> struct TwReg {
+    float2 w[Reg<T>::NTW];
+    __device__ __forceinline__ TwReg(const float2* tab, int lane) {
+#pragma unroll
+        for (int i = 0; i < Reg<T>::NTW; i++) w[i] = __ldg(tab + tw_index<T>(i, lane));
+    }
+    __device__ __forceinline__ float2 get(int i) const { return w[i]; }
+};
+template <int T> struct TwTab {
+    const double2* tab;
+    int lane;
+    __device__ __forceinline__ double2 get(int i) const { return __ldg(tab + tw_index<T>(i, lane)); }
+};
+
+// Lane values of a pass of radix RAD with Ns points done, to the next pass's
+// lane values; ST the element stride of the sequence in shared memory.
+template <int T, int RAD, int Ns, int ST, typename C>
+__device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
+    constexpr int L = T / 8, NB = 8 / RAD;
+#pragma unroll
+    for (int b = 0; b < NB; b++) {
+        const int j = lane + b * L;
+        const int d = (j / Ns) * Ns * RAD + (j & (Ns - 1));
+#pragma unroll
+        for (int r = 0; r < RAD; r++) {
+            const int p = d + r * Ns;
+            s0[(p + (p >> 3)) * ST] = v[b + NB * r];
         }
     }
     __syncthreads();
-    const int seq = threadIdx.x / Sh::LANES, lane = threadIdx.x - seq * Sh::LANES;
-    // the second buffer of sequence seq is SEQ rows further on
-    C* res = stockham<T, S>(buf + seq * Sh::PAD, buf + (Sh::SEQ + seq) * Sh::PAD, tw, lane, Sh::LANES);
-    const bool in_first = res == buf + seq * Sh::PAD;                // the same for every sequence
-    C* out = in_first ? buf : buf + Sh::SEQ * Sh::PAD;
-    for (int e = threadIdx.x; e < Sh::SEQ * T; e += Sh::THREADS) {
-        if (COLS) {
-            const int y = e / Sh::SEQ, c = e - y * Sh::SEQ;
-            base[(long)y * T + s0 + c] = out[c * Sh::PAD + y];
-        } else {
-            const int s = e / T, x = e - s * T;
-            base[(long)(s0 + s) * T + x] = out[s * Sh::PAD + x];
-        }
+#pragma unroll
+    for (int m = 0; m < 8; m++) {
+        const int p = lane + m * L;
+        v[m] = s0[(p + (p >> 3)) * ST];
     }
+    C* t = s0;
+    s0 = s1;
+    s1 = t;
+}
+
+template <int S, typename C> __device__ __forceinline__ C tmul(C v, C w) { return cmul(v, S < 0 ? w : cconj(w)); }
+
+// One radix-4 pass: butterflies b = 0, 1 on v[b], v[b + 2], v[b + 4], v[b + 6],
+// twiddle slots i0 + (PER ? 3 b : 0) + r - 1.
+template <int S, bool PER, typename C, typename TW>
+__device__ __forceinline__ void radix4(C (&v)[8], const TW& tw, int i0) {
+#pragma unroll
+    for (int b = 0; b < 2; b++) {
+#pragma unroll
+        for (int r = 1; r < 4; r++) v[b + 2 * r] = tmul<S>(v[b + 2 * r], tw.get(i0 + (PER ? 3 * b : 0) + r - 1));
+        dft4<S>(v[b], v[b + 2], v[b + 4], v[b + 6]);
+    }
+}
+
+// Every pass after the first (whose butterflies the caller has done: the PSF
+// transforms skip its zeros).  Every thread of the CTA calls it.
+template <int T, int S, int ST, typename C, typename TW>
+__device__ __forceinline__ void fft_tail(C (&v)[8], const TW& tw, C*& s0, C*& s1, int lane) {
+    cross<T, 8, 1, ST>(v, s0, s1, lane);
+#pragma unroll
+    for (int r = 1; r < 8; r++) v[r] = tmul<S>(v[r], tw.get(r - 1));
+    dft8<S>(v);
+    cross<T, 8, 8, ST>(v, s0, s1, lane);
+    if constexpr (T == 512) {
+#pragma unroll
+        for (int r = 1; r < 8; r++) v[r] = tmul<S>(v[r], tw.get(6 + r));
+        dft8<S>(v);
+    } else if constexpr (T == 256) {
+        radix4<S, true>(v, tw, 7);
+    } else {
+        radix4<S, false>(v, tw, 7);
+        cross<T, 4, 64, ST>(v, s0, s1, lane);
+        radix4<S, true>(v, tw, 10);
+    }
+}
+
+template <int T, int S, int ST, typename C, typename TW>
+__device__ __forceinline__ void fft_reg(C (&v)[8], const TW& tw, C*& s0, C*& s1, int lane) {
+    dft8<S>(v);
+    fft_tail<T, S, ST>(v, tw, s0, s1, lane);
 }
 
 }  // namespace fft

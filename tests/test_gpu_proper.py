@@ -230,3 +230,87 @@ def test_shared_psfs_match_per_tile_copies(ora):
         assert torch.equal(S1, S2) and torch.equal(R1, R2)
     finally:
         B.proper_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("T,nt,J,ps,per_tile", [(256, 1, 41, 63, True),     # pairs in groups, the score carried; odd
+                                                (256, 3, 64, 63, True),     # groups within chunks of one tile
+                                                (256, 3, 64, 31, False),    # the same with shared PSFs
+                                                (256, 8, 5, 31, True)])     # chunks of several tiles
+def test_proper_coadd_cuts(ora, T, nt, J, ps, per_tile):
+    """Every way a coadd is cut into chunks of tiles and groups of pairs, with tiles hanging
+    off the frame and a frame left out (sigma 0), at the bars of test_proper_coadd_parity."""
+    from oracle import proper
+    w, h = T + 90, T + 40
+    rng = np.random.default_rng(T + J)
+    origins = [(-20 + 17 * i, 31 - 13 * i) for i in range(nt)]
+    F = rng.uniform(0.8, 1.2, J).astype(np.float32)
+    sg = rng.uniform(4, 9, J).astype(np.float32)
+    if J > 3:
+        sg[2] = 0.0
+    frames = rng.normal(0, 6, (J, h, w)).astype(np.float32)
+    frames[:, rng.integers(0, h, 40), rng.integers(0, w, 40)] += 3e3
+    half = ps // 2
+    psfs = np.stack([np.stack([_gauss(1.2 + 0.02 * j + 0.05 * t, half) for j in range(J)])
+                     for t in range(nt if per_tile else 1)])
+    pitch = pitch_for(w)
+    stack = torch.zeros((J, h, pitch), device="cuda")
+    stack[:, :, :w] = torch.from_numpy(frames).cuda()
+    S, R, PR = (torch.full((nt, T, T), -7.0, device="cuda") for _ in range(3))
+    FR = torch.zeros(1, dtype=torch.float64, device="cuda")
+    sig = torch.zeros(nt, dtype=torch.float64, device="cuda")
+    plan = B.proper_plan_create(0, T, nt)
+    try:
+        B.argus_proper_coadd(plan, stack, J, B.argus_shape(w, h, pitch),
+                             torch.tensor(origins, dtype=torch.int32, device="cuda"), nt, torch.from_numpy(F).cuda(),
+                             torch.from_numpy(sg).cuda(), torch.from_numpy(psfs).cuda(), ps, 1e-8, S, R, PR, FR, sig,
+                             psf_per_tile=per_tile)
+        torch.cuda.synchronize()
+        S, R, PR, FR, sig = (t.cpu().numpy() for t in (S, R, PR, FR, sig))
+    finally:
+        B.proper_plan_destroy(plan)
+    use = [j for j in range(J) if sg[j] > 0]
+    for i, (x0, y0) in enumerate(origins):
+        Ms = []
+        for j in use:
+            M = np.zeros((T, T), np.float32)
+            xs, ys = slice(max(x0, 0), min(x0 + T, w)), slice(max(y0, 0), min(y0 + T, h))
+            M[ys.start - y0:ys.stop - y0, xs.start - x0:xs.stop - x0] = frames[j, ys, xs]
+            Ms.append(M)
+        Ps = [psfs[i if per_tile else 0, j].astype(np.float64) for j in use]
+        o = proper.proper_coadd(Ms, Ps, [float(F[j]) for j in use], [float(sg[j]) for j in use])
+        lg = F32_EPS * math.log2(T * T) / T
+        eR = lg * sum(np.linalg.norm(M) / sg[j] for M, j in zip(Ms, use))
+        eS = lg * (sum(F[j] / sg[j] ** 2 * np.abs(P).sum() * np.linalg.norm(M) for M, P, j in zip(Ms, Ps, use))
+                   + np.linalg.norm(o["R"]))
+        assert np.abs(R[i] - o["R"]).max() <= 8 * eR
+        assert np.abs(S[i] - o["S"]).max() <= 8 * eS
+        assert np.abs(PR[i] - o["P_R"]).max() <= 64 * F32_EPS * np.abs(o["P_R"]).max()
+        assert abs(FR[0] / o["F_R"] - 1) < 1e-6 and abs(sig[i] / o["sigma_S"] - 1) < 1e-6
+
+
+def test_proper_coadd_1024(ora):
+    """A 1024 tile of five noise frames at the bars of test_proper_coadd_parity."""
+    from oracle import proper
+    T, J = 1024, 5
+    rng = np.random.default_rng(9)
+    F, sg = np.array([1.0, 0.8, 1.2, 0.9, 1.1], np.float32), np.array([5.0, 9.0, 4.0, 7.0, 6.0], np.float32)
+    frames = (rng.normal(0, 1, (J, T, T)) * sg[:, None, None]).astype(np.float32)
+    psfs = np.stack([_gauss(1.2 + 0.2 * j) for j in range(J)])
+    S, R = (torch.empty((1, T, T), device="cuda") for _ in range(2))
+    plan = B.proper_plan_create(0, T, 1)
+    try:
+        B.argus_proper_coadd(plan, torch.from_numpy(frames).cuda(), J, B.argus_shape(T, T, T),
+                             torch.zeros((1, 2), dtype=torch.int32, device="cuda"), 1, torch.from_numpy(F).cuda(),
+                             torch.from_numpy(sg).cuda(), torch.from_numpy(psfs).cuda(), 31, 1e-8, S, R)
+        torch.cuda.synchronize()
+        S, R = S[0].cpu().numpy(), R[0].cpu().numpy()
+    finally:
+        B.proper_plan_destroy(plan)
+    o = proper.proper_coadd(list(frames), [p.astype(np.float64) for p in psfs], [float(f) for f in F],
+                            [float(s) for s in sg])
+    lg = F32_EPS * math.log2(T * T) / T
+    eR = lg * sum(np.linalg.norm(M) / s for M, s in zip(frames, sg))
+    eS = lg * (sum(f / s ** 2 * np.abs(P).sum() * np.linalg.norm(M) for M, P, f, s in zip(frames, psfs, F, sg))
+               + np.linalg.norm(o["R"]))
+    assert np.abs(R - o["R"]).max() <= 8 * eR
+    assert np.abs(S - o["S"]).max() <= 8 * eS
