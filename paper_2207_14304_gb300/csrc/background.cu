@@ -2,15 +2,16 @@
 // background map"; background maps held with the calibration frames, Sec. 3.2).
 //
 //   1. box_median_kernel: one CTA per box x box mesh box; the valid pixels
-//      (flag 0, finite) stay in registers as order-preserving 32-bit keys and
-//      an 8-bit radix select (4 passes over a 256-bin shared histogram) finds
-//      the middle key(s); the box value is their mean in FP64 (exact), or NaN
-//      when fewer than min_frac of the box's pixels are valid.
-//   2. mesh_fill_kernel: one CTA; the median of all box values (the value of
-//      boxes with nothing in reach), by the same radix select on 64-bit keys
-//      of the doubles, reading the mesh from global memory.
-//   3. mesh_filter_kernel: one thread per box; the median of the values that
-//      exist in its filt x filt neighbourhood (clipped at the mesh edges).
+//      (flag 0, finite) stay in registers as order-preserving 32-bit keys and a
+//      bracket around the middle key(s) is narrowed by counting; the box value is
+//      their mean in FP64 (exact), or NaN when fewer than min_frac of the box's
+//      pixels are valid.
+//   2. mesh_filter_kernel: one thread per box; the median of the values that
+//      exist in its filt x filt neighbourhood (clipped at the mesh edges), and the
+//      mesh in FP32 for the map.
+//   3. mesh_fill_kernel: one CTA; if some neighbourhood had no value, the median
+//      of all box values goes there, by radix select on 64-bit keys of the
+//      doubles, reading the mesh from global memory.
 //   4. interp_kernel: the map, bilinear between box centres (mean pixel
 //      coordinate of each box), constant beyond the outermost ones, in FP32,
 //      four pixels per thread.
@@ -29,7 +30,8 @@ struct BgArgs {
     const uint8_t* flags;
     double* raw;        // [ny][nx] box medians (NaN: no value)
     double* mesh;       // [ny][nx] filtered
-    double* fill;       // [1] median of all box values
+    float* meshf;       // [ny][nx] the filtered mesh rounded to FP32
+    int* missing;       // [1] neighbourhoods without a value
     float* map;
     long pitch;
     int w, h, box, filt, nx, ny;
@@ -90,9 +92,11 @@ __host__ __device__ __forceinline__ double unkey64(unsigned long long k) {
     return bits_f64((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k);
 }
 
+// The radix form of a box's selection, one thread of 256 at a time: what the CPU
+// checks run (box_load, box_hist, box_le_min).
 // One thread's share of a box: pixels tid, tid + 256, ... of the box as keys
 // (ok = valid); returns the count of valid pixels.
-__host__ __device__ __forceinline__ int box_load(const BgArgs& a, int bx, int by, int tid, unsigned* key, bool* ok) {
+[[maybe_unused]] __host__ __device__ __forceinline__ int box_load(const BgArgs& a, int bx, int by, int tid, unsigned* key, bool* ok) {
     const int x0 = bx * a.box, y0 = by * a.box;
     const int bw = min(a.box, a.w - x0), bh = min(a.box, a.h - y0);
     const int npx = bw * bh;
@@ -119,7 +123,7 @@ __host__ __device__ __forceinline__ int box_load(const BgArgs& a, int bx, int by
 // One thread's histogram contribution of a radix pass: add(bin) for each of its
 // keys that matches the prefix decided so far.
 template <typename Add>
-__host__ __device__ __forceinline__ void box_hist(const unsigned* key, const bool* ok, unsigned mask, unsigned prefix,
+[[maybe_unused]] __host__ __device__ __forceinline__ void box_hist(const unsigned* key, const bool* ok, unsigned mask, unsigned prefix,
                                                   int shift, Add add) {
 #pragma unroll
     for (int j = 0; j < BM_MAX_PER; j++)
@@ -127,7 +131,7 @@ __host__ __device__ __forceinline__ void box_hist(const unsigned* key, const boo
 }
 
 // One thread's count of keys <= k1 and its smallest key above k1.
-__host__ __device__ __forceinline__ void box_le_min(const unsigned* key, const bool* ok, unsigned k1, int& le,
+[[maybe_unused]] __host__ __device__ __forceinline__ void box_le_min(const unsigned* key, const bool* ok, unsigned k1, int& le,
                                                     unsigned& m) {
     le = 0;
     m = 0xffffffffu;
@@ -197,63 +201,194 @@ __device__ __forceinline__ int pick_bin(const int* hist, int& k, int* sh) {
     return b;
 }
 
-__global__ void __launch_bounds__(BM_THREADS) box_median_kernel(BgArgs a) {
-    __shared__ int hist[256];
-    __shared__ int red[32];
-    __shared__ int sh[2];
-    __shared__ unsigned umin[32];
-    const int bx = blockIdx.x, by = blockIdx.y;
-    const int npx = min(a.box, a.w - bx * a.box) * min(a.box, a.h - by * a.box);
-    unsigned key[BM_MAX_PER];
-    bool ok[BM_MAX_PER];
-    const int n = block_sum(box_load(a, bx, by, threadIdx.x, key, ok), red);
-    double out = __longlong_as_double(0x7ff8000000000000ll);     // NaN: no value
-    if (box_has_value(n, npx, a.min_frac)) {
-        // k-th smallest key for k1 = (n - 1) / 2
-        int k = (n - 1) / 2;
-        unsigned prefix = 0, mask = 0;
-        for (int shift = 24; shift >= 0; shift -= 8) {
-            for (int i = threadIdx.x; i < 256; i += BM_THREADS) hist[i] = 0;
-            __syncthreads();
-            box_hist(key, ok, mask, prefix, shift, [&](int b) { atomicAdd(&hist[b], 1); });
-            __syncthreads();
-            const int b = pick_bin(hist, k, sh);
-            prefix |= (unsigned)b << shift;
-            mask |= 255u << shift;
+// Box medians, one CTA of 128 threads per box, NPL keys per thread (pixel e = tid +
+// 128 j of the box; 0xffffffff, above every valid key, where there is none or it is
+// invalid).  The middle keys are bracketed: (lo, hi] holds the ranks clo .. chi - 1,
+// among them r1 = (n - 1) / 2 and r2 = n / 2.  A pass counts the keys up to two
+// thresholds -- first two order statistics of 32 of the keys, then an interpolated
+// guess with a margin of a few keys either side -- until at most 32 keys are left,
+// which one warp sorts.  Four or five passes of two compares and adds per key and one
+// barrier: 196 us on a 9576 x 6388 frame of 64-pixel boxes (issue slots 69 % busy), against
+// 514 us for an 8-bit radix select, whose first pass is atomics to the few bins that a
+// box's exponents fall in.  After CAREFUL passes the thresholds halve the bracket
+// instead, so every box ends.  One warp per box with all 4096 keys in its registers
+// needed 200 of them and waited on its loads eight warps to an SM.
+constexpr int BOX_THREADS = 128, BOX_WARPS = BOX_THREADS / 32, CAREFUL = 10;
+
+// The lanes' values in ascending order over the lanes (bitonic).
+__device__ __forceinline__ unsigned warp_sort(unsigned v, int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const unsigned o = __shfl_xor_sync(0xffffffffu, v, j);
+            const bool low = ((lane & j) == 0) == ((lane & k) == 0);
+            v = low ? min(v, o) : max(v, o);
         }
-        const unsigned k1 = prefix;
-        unsigned k2 = k1;
-        if ((n & 1) == 0) {
-            // the next order statistic: k1 again if it repeats, else the smallest key above it
-            int le;
-            unsigned m;
-            box_le_min(key, ok, k1, le, m);
-            const int nle = block_sum(le, red);
-            m = __reduce_min_sync(0xffffffffu, m);
-            if ((threadIdx.x & 31) == 0) umin[threadIdx.x >> 5] = m;
-            __syncthreads();
-            unsigned mm = 0xffffffffu;
-            for (int i = 0; i < BM_THREADS / 32; i++) mm = min(mm, umin[i]);
-            k2 = nle >= n / 2 + 1 ? k1 : mm;
-        }
-        out = median_of_keys(k1, k2);
-    }
-    if (threadIdx.x == 0) a.raw[(long)by * a.nx + bx] = out;
+    return v;
 }
 
-// Median of the non-NaN doubles v[0..n) by radix select over global memory
-// (one CTA); 0 if there are none.
+// Sums of c and d over the CTA; `part` alternates between two slots, so one barrier does.
+__device__ __forceinline__ int2 box_sum2(int c, int d, int2 (*part)[BOX_WARPS], int& slot) {
+    c = __reduce_add_sync(0xffffffffu, c);
+    d = __reduce_add_sync(0xffffffffu, d);
+    if ((threadIdx.x & 31) == 0) part[slot][threadIdx.x >> 5] = make_int2(c, d);
+    __syncthreads();
+    int2 s = make_int2(0, 0);
+#pragma unroll
+    for (int i = 0; i < BOX_WARPS; i++) {
+        s.x += part[slot][i].x;
+        s.y += part[slot][i].y;
+    }
+    slot ^= 1;
+    return s;
+}
+
+template <int NPL>
+__global__ void __launch_bounds__(BOX_THREADS) box_median_kernel(BgArgs a) {
+    __shared__ int2 part[2][BOX_WARPS];
+    __shared__ unsigned smp[2], cand[32], kk[2][BOX_WARPS];
+    __shared__ int at;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = blockIdx.x;
+    const int by = b / a.nx, bx = b - by * a.nx;
+    const int bw = min(a.box, a.w - bx * a.box), bh = min(a.box, a.h - by * a.box), npx = bw * bh;
+    unsigned key[NPL];
+    int nv = 0, slot = 0;
+    {
+        const int dq = BOX_THREADS / bw, dr = BOX_THREADS - dq * bw;   // pixel e + 128: dq rows and dr columns on
+        int yy = tid / bw, xx = tid - yy * bw;
+        const long base = (long)by * a.box * a.pitch + bx * a.box;
+        constexpr int LB = NPL < 8 ? NPL : NPL % 8 ? 6 : 8;            // loads in flight per thread and image
+        static_assert(NPL % LB == 0, "whole batches");
+#pragma unroll
+        for (int j0 = 0; j0 < NPL; j0 += LB) {
+            float v[LB];
+            unsigned f[LB];
+#pragma unroll
+            for (int j = 0; j < LB; j++) {
+                const bool in = tid + BOX_THREADS * (j0 + j) < npx;
+                const long p = base + (long)yy * a.pitch + xx;
+                v[j] = in ? __ldg(a.img + p) : __int_as_float(0x7fffffff);
+                f[j] = in && a.flags ? __ldg(a.flags + p) : 0u;
+                yy += dq;
+                xx += dr;
+                if (xx >= bw) { xx -= bw; yy++; }
+            }
+#pragma unroll
+            for (int j = 0; j < LB; j++) {
+                const bool ok = (f[j] == 0u) & (fabsf(v[j]) <= 3.402823466e38f);     // finite
+                key[j0 + j] = ok ? key32(v[j]) : 0xffffffffu;
+                nv += ok ? 1 : 0;
+            }
+        }
+    }
+    if (warp == 0) {
+        const unsigned v = warp_sort(key[0], lane);
+        if (lane == 9) smp[0] = v;
+        if (lane == 22) smp[1] = v;
+        if (lane == 0) at = 0;
+    }
+    const int n = box_sum2(nv, 0, part, slot).x;
+    if (!box_has_value(n, npx, a.min_frac)) {
+        if (tid == 0) a.raw[b] = __longlong_as_double(0x7ff8000000000000ll);     // NaN: no value
+        return;
+    }
+    const int r1 = (n - 1) / 2, r2 = n / 2;
+    unsigned lo = 0u, hi = 0xfffffffeu;                    // no valid key is 0 or above hi
+    int clo = 0, chi = n;
+    unsigned t = smp[0], u = smp[1];
+    bool split = false;
+    unsigned cut = 0u;                                     // split: r1 is the last key <= cut, r2 the first above
+    for (int it = 0;; it++) {                              // the same for every thread
+        if (t > lo && t < hi && u > lo && u < hi) {
+            int c = 0, d = 0;
+#pragma unroll
+            for (int j = 0; j < NPL; j++) {
+                c += key[j] <= t ? 1 : 0;
+                d += key[j] <= u ? 1 : 0;
+            }
+            const int2 s = box_sum2(c, d, part, slot);
+            if (s.x <= r1) { lo = t; clo = s.x; }
+            else if (s.x > r2) { hi = t; chi = s.x; }
+            else { split = true; cut = t; }
+            if (s.y <= r1) { if (u > lo) { lo = u; clo = s.y; } }
+            else if (s.y > r2) { if (u < hi) { hi = u; chi = s.y; } }
+            else { split = true; cut = u; }
+        }
+        if (split || chi - clo <= 32 || hi - lo == 1u) break;
+        const unsigned span = hi - lo;
+        if (it >= CAREFUL) {
+            t = u = lo + span / 2;
+        } else {
+            const float c = (float)(chi - clo), per = (float)span / c;
+            const float g = ((float)(r1 - clo) + 0.75f) * per, m = fmaxf(8.0f, 1.5f * sqrtf(c)) * per;
+            const float top = (float)(span - 1u);
+            t = lo + max(1u, (unsigned)fminf(fmaxf(g - m, 1.0f), top));
+            u = lo + max(1u, (unsigned)fminf(g + m, top));
+            t = min(t, hi - 1u);
+            u = min(u, hi - 1u);
+        }
+    }
+    if (split) {
+        unsigned m1 = 0u, m2 = 0xffffffffu;
+#pragma unroll
+        for (int j = 0; j < NPL; j++) {
+            if (key[j] <= cut) m1 = max(m1, key[j]);
+            else m2 = min(m2, key[j]);
+        }
+        m1 = __reduce_max_sync(0xffffffffu, m1);
+        m2 = __reduce_min_sync(0xffffffffu, m2);
+        if (lane == 0) {
+            kk[0][warp] = m1;
+            kk[1][warp] = m2;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int i = 1; i < BOX_WARPS; i++) {
+                m1 = max(m1, kk[0][i]);
+                m2 = min(m2, kk[1][i]);
+            }
+            a.raw[b] = median_of_keys(m1, m2);
+        }
+    } else if (hi - lo == 1u) {
+        if (tid == 0) a.raw[b] = median_of_keys(hi, hi);   // every key left is hi
+    } else {
+#pragma unroll
+        for (int j = 0; j < NPL; j++)
+            if (key[j] - lo - 1u < hi - lo) cand[atomicAdd(&at, 1)] = key[j];     // lo < key <= hi: at most 32
+        __syncthreads();
+        if (warp == 0) {
+            const unsigned v = warp_sort(lane < at ? cand[lane] : 0xffffffffu, lane);
+            const unsigned k1 = __shfl_sync(0xffffffffu, v, r1 - clo), k2 = __shfl_sync(0xffffffffu, v, r2 - clo);
+            if (lane == 0) a.raw[b] = median_of_keys(k1, k2);
+        }
+    }
+}
+
+// The cells whose neighbourhood had no value (NaN in the mesh) take the median of
+// the non-NaN box values by radix select over global memory (one CTA), 0 if there
+// are none.  Leaves at once where there is no such cell, as in nearly every frame
+// (the selection takes 90 us on 15,000 boxes).
 __global__ void __launch_bounds__(FILL_THREADS) mesh_fill_kernel(BgArgs a) {
     __shared__ int hist[256];
     __shared__ int red[32];
     __shared__ int sh[2];
     __shared__ unsigned long long umin[32];
+    if (*a.missing == 0) return;
     const int ncell = a.nx * a.ny;
+    const auto fill_in = [&](double v) {
+        for (int i = threadIdx.x; i < ncell; i += FILL_THREADS)
+            if (isnan(a.mesh[i])) {
+                a.mesh[i] = v;
+                a.meshf[i] = (float)v;
+            }
+    };
     int nv = 0;
     for (int i = threadIdx.x; i < ncell; i += FILL_THREADS) nv += isnan(a.raw[i]) ? 0 : 1;
     const int n = block_sum(nv, red);
     if (n == 0) {
-        if (threadIdx.x == 0) *a.fill = 0.0;
+        fill_in(0.0);
         return;
     }
     int k = (n - 1) / 2;
@@ -295,7 +430,7 @@ __global__ void __launch_bounds__(FILL_THREADS) mesh_fill_kernel(BgArgs a) {
         for (int i = 0; i < FILL_THREADS / 32; i++) mm = umin[i] < mm ? umin[i] : mm;
         k2 = nle >= n / 2 + 1 ? k1 : mm;
     }
-    if (threadIdx.x == 0) *a.fill = 0.5 * (unkey64(k1) + unkey64(k2));
+    fill_in(0.5 * (unkey64(k1) + unkey64(k2)));
 }
 
 // The filtered value of box (cx, cy): the median of the values that exist in its
@@ -324,7 +459,10 @@ __global__ void __launch_bounds__(256) mesh_filter_kernel(BgArgs a) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= a.nx * a.ny) return;
     const int cy = c / a.nx, cx = c - cy * a.nx;
-    a.mesh[c] = filter_cell(a.raw, a.nx, a.ny, cx, cy, a.filt, *a.fill);
+    const double v = filter_cell(a.raw, a.nx, a.ny, cx, cy, a.filt, __longlong_as_double(0x7ff8000000000000ll));
+    a.mesh[c] = v;
+    a.meshf[c] = (float)v;
+    if (isnan(v)) atomicAdd(a.missing, 1);
 }
 
 // Interpolation coordinate along one axis: lower box index i (upper i + 1) and
@@ -347,8 +485,8 @@ __host__ __device__ __forceinline__ void axis_weight(int p, int n, int box, int 
 }
 
 // Bilinear value from the mesh row r0 (lower box ix, next box ix + jx, next row
-// + jy) in FP32.
-__host__ __device__ __forceinline__ float bilinear(const double* r0, int ix, int jx, int jy, float tx, float ty) {
+// + jy) in FP32 (what the CPU checks run; interp_kernel does the same per row).
+[[maybe_unused]] __host__ __device__ __forceinline__ float bilinear(const double* r0, int ix, int jx, int jy, float tx, float ty) {
     const float m00 = (float)r0[ix], m01 = (float)r0[ix + jx];
     const float m10 = (float)r0[jy + ix], m11 = (float)r0[jy + ix + jx];
     const float top = m00 + (m01 - m00) * tx;
@@ -356,25 +494,49 @@ __host__ __device__ __forceinline__ float bilinear(const double* r0, int ix, int
     return top + (bot - top) * ty;
 }
 
+// The two mesh rows' interpolated values stay in registers while the rows of a
+// thread lie between the same centres, so a pixel costs a subtraction, a fused
+// multiply-add and its store; converting four FP64 mesh values per pixel took 422 us
+// on a 9576 x 6388 map (the FP64 pipe does two conversions per clock and SM), this 53 us.
+constexpr int INTERP_ROWS = 16;
+
 __global__ void __launch_bounds__(256) interp_kernel(BgArgs a) {
     const int x0 = (blockIdx.x * 256 + threadIdx.x) * 4;
     if (x0 >= a.pitch) return;
     int ix[4];
-    float tx[4];
+    float tx[4], top[4], dif[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) axis_weight(min(x0 + k, a.w - 1), a.w, a.box, a.nx, ix[k], tx[k]);
-    const int jx = a.nx > 1 ? 1 : 0;
-    for (int y = blockIdx.y; y < a.h; y += gridDim.y) {
+    for (int k = 0; k < 4; k++) {
+        axis_weight(min(x0 + k, a.w - 1), a.w, a.box, a.nx, ix[k], tx[k]);
+        top[k] = dif[k] = 0.0f;
+    }
+    const int jx = a.nx > 1 ? 1 : 0, jy = a.ny > 1 ? a.nx : 0;
+    int last = -1;
+    for (int yb = blockIdx.y; yb * INTERP_ROWS < a.h; yb += gridDim.y)
+    for (int y = yb * INTERP_ROWS, y1 = min(y + INTERP_ROWS, a.h); y < y1; y++) {
         int iy;
         float ty;
         axis_weight(y, a.h, a.box, a.ny, iy, ty);
-        const int jy = a.ny > 1 ? a.nx : 0;
-        const double* r0 = a.mesh + (long)iy * a.nx;
+        if (iy != last) {
+            last = iy;
+            const float* r0 = a.meshf + (long)iy * a.nx;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const float m00 = r0[ix[k]], m01 = r0[ix[k] + jx], m10 = r0[jy + ix[k]], m11 = r0[jy + ix[k] + jx];
+                top[k] = m00 + (m01 - m00) * tx[k];
+                dif[k] = m10 + (m11 - m10) * tx[k] - top[k];
+            }
+        }
         float o[4];
 #pragma unroll
-        for (int k = 0; k < 4; k++) o[k] = x0 + k < a.w ? bilinear(r0, ix[k], jx, jy, tx[k], ty) : 0.0f;
+        for (int k = 0; k < 4; k++) o[k] = x0 + k < a.w ? top[k] + dif[k] * ty : 0.0f;
         *reinterpret_cast<float4*>(a.map + (long)y * a.pitch + x0) = make_float4(o[0], o[1], o[2], o[3]);
     }
+}
+
+template <int NPL>
+void launch_box_medians(const BgArgs& a, cudaStream_t s) {
+    box_median_kernel<NPL><<<a.nx * a.ny, BOX_THREADS, 0, s>>>(a);
 }
 
 }  // namespace
@@ -396,17 +558,22 @@ extern "C" int argus_background(argus_ctx* ctx, const float* img, const uint8_t*
     BgArgs a;
     a.img = img; a.flags = flags; a.mesh = mesh; a.map = map; a.pitch = shape.pitch;
     a.w = shape.w; a.h = shape.h; a.box = box; a.filt = filt; a.nx = nx; a.ny = ny; a.min_frac = min_frac;
-    // scratch: the raw mesh and the fill value in the detection label buffer
-    // (max_pixels ints >= 2 doubles per box + 1, as box >= 8)
+    // scratch in the detection label buffer: the raw mesh, its FP32 copy and the count of
+    // cells to fill, 12 bytes per box and 4 (max_pixels ints are 256 bytes per 8 x 8 box)
     a.raw = reinterpret_cast<double*>(ctx->label);
-    a.fill = a.raw + (long)nx * ny;
-    box_median_kernel<<<dim3(nx, ny), BM_THREADS, 0, s>>>(a); argus_count_launch(1);
-    mesh_fill_kernel<<<1, FILL_THREADS, 0, s>>>(a); argus_count_launch(1);
-    mesh_filter_kernel<<<(nx * ny + 255) / 256, 256, 0, s>>>(a); argus_count_launch(1);
+    a.meshf = reinterpret_cast<float*>(a.raw + (long)nx * ny);
+    a.missing = reinterpret_cast<int*>(a.meshf + (long)nx * ny);
+    if (cudaMemsetAsync(a.missing, 0, sizeof(int), s) != cudaSuccess) return ARGUS_ERR_CUDA;
+    const int npl = (box * box + BOX_THREADS - 1) / BOX_THREADS;   // keys per thread: the smallest compiled bound
+    if (npl <= 2) launch_box_medians<2>(a, s);
+    else if (npl <= 8) launch_box_medians<8>(a, s);
+    else if (npl <= 18) launch_box_medians<18>(a, s);
+    else launch_box_medians<32>(a, s);
+    mesh_filter_kernel<<<(nx * ny + 255) / 256, 256, 0, s>>>(a);
+    mesh_fill_kernel<<<1, FILL_THREADS, 0, s>>>(a); argus_count_launch(3);
     if (map) {
         const int gx = (int)((shape.pitch / 4 + 255) / 256);
-        int gy = ctx->num_sms * 16 / gx;
-        gy = gy < 1 ? 1 : (gy > shape.h ? shape.h : gy);
+        const int gy = min((shape.h + INTERP_ROWS - 1) / INTERP_ROWS, 65535);
         interp_kernel<<<dim3(gx, gy), 256, 0, s>>>(a); argus_count_launch(1);
     }
     return argus_launch_status();

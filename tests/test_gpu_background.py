@@ -86,3 +86,27 @@ def test_background_full_frame():
     w, h = 9576, 6388
     img, fl = _field(w, h, seed=11)
     _check(img, fl, 64, 3)
+
+
+@pytest.mark.parametrize("w,h,box,kind", [(200, 130, 64, "equal"), (200, 130, 64, "two"), (300, 70, 48, "whole"),
+                                          (129, 65, 33, "spread"), (90, 50, 16, "signs"), (65, 130, 64, "pair")])
+def test_background_selection(ora, w, h, box, kind):
+    """Boxes whose keys are hard to bracket: all equal, two values in equal numbers, repeated whole
+    numbers, magnitudes over the whole range of FP32, both signs and zeros, and boxes of one or two
+    valid pixels."""
+    rng = np.random.default_rng(w + box)
+    if kind == "equal":
+        img = np.full((h, w), 7.25, np.float32)
+    elif kind == "two":
+        img = np.where((np.arange(h * w) % 2).reshape(h, w), 1e5, -3.0).astype(np.float32)
+    elif kind == "whole":
+        img = rng.integers(0, 5, (h, w)).astype(np.float32)
+    elif kind == "spread":
+        img = (np.sign(rng.normal(size=(h, w))) * 10.0 ** rng.uniform(-44, 38, (h, w))).astype(np.float32)
+    elif kind == "signs":
+        img = rng.choice(np.array([-1.5, -0.0, 0.0, 2.0, 1e30], np.float32), (h, w))
+    else:
+        img = np.full((h, w), np.nan, np.float32)
+        img[3::64, 5::64] = 4.0
+        img[4::64, 7::64] = -9.5
+    _check(img, None, box, 3, min_frac=0.0)
