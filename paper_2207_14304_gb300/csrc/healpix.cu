@@ -7,9 +7,9 @@
 // layout) is projected into the frame by the gnomonic WCS and the frame is
 // interpolated there (bilinear, nested lerps, coverage as in the coadd).  The
 // geometry is FP64 (a 9576-pixel frame needs positions to 1e-9 of the field);
-// the output is FP32.  Exact path: one thread per pixel.  Row path (k >= 6):
-// one warp per row, exact positions at four nodes per 64-pixel piece and a
-// cubic between them in the equatorial belt (see healpix_rows_kernel).
+// the output is FP32.  Exact path: one thread per pixel.  Patch path (k >= 6):
+// a CTA per 64 x 64 patch, exact positions at 4 x 8 nodes and bicubics between
+// them in the equatorial belt, in fixed point (see healpix_patch_kernel).
 #include "argus_internal.cuh"
 
 #include <cmath>
@@ -92,6 +92,21 @@ __host__ __device__ __forceinline__ bool hp_pixel_xy(const HpArgs& a, long long 
     return true;
 }
 
+// Whether pixel (c, r) of a valid segment lies in the equatorial belt (ring index in
+// [N, 3N]); the ring index falls with c and with r, so a rectangle whose first and
+// last pixels do lies in it wholly.
+__host__ __device__ __forceinline__ bool hp_pixel_in_belt(const HpArgs& a, long long seg, int c, int r) {
+    const long long N = a.nside_seg, face = seg / (N * N), ipf = seg - face * N * N;
+    long long X = 0, Y = 0;
+    for (int b = 0; (1LL << b) < N; b++) {
+        X |= ((ipf >> (2 * b)) & 1LL) << b;
+        Y |= ((ipf >> (2 * b + 1)) & 1LL) << b;
+    }
+    const long long nside = N << a.k, jrll = face < 4 ? 2 : (face < 8 ? 3 : 4);
+    const long long jr = jrll * nside - ((X << a.k) + c) - ((Y << a.k) + r) - 1;
+    return jr >= nside && jr <= 3 * nside;
+}
+
 // Nested-lerp bilinear value of the frame at (x, y); false when not covered
 // (outside [0, w-1] x [0, h-1], or a neighbour with a nonzero weight flagged
 // or not finite).
@@ -115,15 +130,17 @@ __host__ __device__ __forceinline__ bool hp_bilinear(const HpArgs& a, double x, 
     return true;
 }
 
-// Row interpolation (the fast path).  Along a segment-image row in the
-// equatorial belt the frame position is a smooth function of the column: on
-// pieces of 64 pixels a cubic through the exact FP64 positions at columns
-// 0, 21, 42, 63 of the piece reproduces it to a few 1e-8 pixel.  Newton form:
-// d[0] = f0, d[1] = f[t0,t1], d[2] = f[t0,t1,t2], d[3] = f[t0..t3].
-constexpr int HP_PIECE = 64;
+// Interpolation of positions.  Along a segment-image row or column in the
+// equatorial belt the frame position is a smooth function of the column or row:
+// on pieces of 64 pixels a cubic through the exact FP64 positions at 0, 21, 42,
+// 63 of the piece reproduces it to a few 1e-8 pixel (a sixteenth of that on
+// pieces of 32).  Newton form: d[0] = f0, d[1] = f[t0,t1], d[2] = f[t0,t1,t2],
+// d[3] = f[t0..t3] (the row form hp_cubic_* and hp_row_in_belt is what the CPU
+// checks run).
+[[maybe_unused]] constexpr int HP_PIECE = 64;
 __host__ __device__ __forceinline__ int hp_node(int j) { return j == 0 ? 0 : (j == 1 ? 21 : (j == 2 ? 42 : 63)); }
 
-__host__ __device__ __forceinline__ void hp_cubic_coeffs(const double* f, double* d) {
+[[maybe_unused]] __host__ __device__ __forceinline__ void hp_cubic_coeffs(const double* f, double* d) {
     const double f01 = (f[1] - f[0]) / 21.0, f12 = (f[2] - f[1]) / 21.0, f23 = (f[3] - f[2]) / 21.0;
     const double f012 = (f12 - f01) / 42.0, f123 = (f23 - f12) / 42.0;
     d[0] = f[0];
@@ -132,13 +149,13 @@ __host__ __device__ __forceinline__ void hp_cubic_coeffs(const double* f, double
     d[3] = (f123 - f012) / 63.0;
 }
 
-__host__ __device__ __forceinline__ double hp_cubic_eval(const double* d, double t) {
+[[maybe_unused]] __host__ __device__ __forceinline__ double hp_cubic_eval(const double* d, double t) {
     return d[0] + t * (d[1] + (t - 21.0) * (d[2] + (t - 42.0) * d[3]));
 }
 
 // Whether a whole segment-image row lies in the equatorial belt (where the
 // row interpolation is used): ring indices of its two end pixels in [N, 3N].
-__host__ __device__ __forceinline__ bool hp_row_in_belt(const HpArgs& a, long long seg, int r) {
+[[maybe_unused]] __host__ __device__ __forceinline__ bool hp_row_in_belt(const HpArgs& a, long long seg, int r) {
     const long long N = a.nside_seg;
     const long long face = seg / (N * N);
     if (seg < 0 || face >= 12) return false;
@@ -156,69 +173,223 @@ __host__ __device__ __forceinline__ bool hp_row_in_belt(const HpArgs& a, long lo
     return jr1 >= nside && jr0 <= 3 * nside;
 }
 
-// One warp per segment-image row (k >= 6): in the belt, lanes compute the
-// exact positions of the four nodes of eight pieces at once and each lane
-// evaluates 16 pixels of its piece from the cubic; elsewhere (and for pieces
-// with a node behind the tangent plane) every pixel takes the exact path.
-__global__ void __launch_bounds__(256) healpix_rows_kernel(HpArgs a) {
-    const int lane = threadIdx.x & 31;
+// ---------------------------------------------------------------------------
+// Patch path (k >= 6).  A CTA takes 64 x 64 pixels of a segment image as two
+// halves of 64 x 32.  One warp computes the exact FP64 positions of the 32 nodes
+// (columns 0, 21, 42, 63; rows 0, 10, 21, 31 of each half).  Per half, each column's
+// positions along the rows are a cubic through its values at the four node rows,
+// kept as forward differences in 64-bit fixed point (2^-44 pixel), so a pixel's
+// position costs three 64-bit additions per coordinate and no FP64: this part does
+// two FP64 operations per clock and SM, and evaluating two FP64 cubics and three
+// FP64 lerps per pixel took 3.80 ms for the 170 segments of a 9576 x 6388 frame.
+// The frame pixels under the half (a rectangle around its nodes) are staged in
+// shared memory once, NaN where flagged or not finite: the image axes lie
+// diagonally across the frame, and gathering neighbours from global memory
+// touches about 27 lines per warp load.  The lerps run on unevaluated FP32 pairs
+// (about 2^-44 relative, then one rounding).  Halves not wholly in the belt, with
+// a node behind the tangent plane or beyond HP_FAR pixels take the exact path per
+// pixel; halves whose rectangle exceeds HP_CAP pixels gather from global memory.
+constexpr int HP_PATCH = 64, HP_HALF = 32, HP_FRAC = 44, HP_CAP = 10240;
+constexpr double HP_FAR = 500000.0;      // positions in fixed point stay below 2^19
+
+__host__ __device__ __forceinline__ int hp_node_row(int j) { return j == 0 ? 0 : (j == 1 ? 10 : (j == 2 ? 21 : 31)); }
+
+// Lagrange weights of the node columns 0, 21, 42, 63 at each column of a patch, times 2^HP_FRAC.
+struct HpWeights { double w[HP_PATCH][4]; };
+constexpr HpWeights hp_make_weights() {
+    HpWeights t{};
+    for (int c = 0; c < HP_PATCH; c++)
+        for (int j = 0; j < 4; j++) {
+            double num = (double)(1LL << HP_FRAC), den = 1.0;
+            for (int i = 0; i < 4; i++)
+                if (i != j) {
+                    num *= (double)(c - 21 * i);
+                    den *= (double)(21 * (j - i));
+                }
+            t.w[c][j] = num / den;
+        }
+    return t;
+}
+__device__ const HpWeights hp_weights = hp_make_weights();
+
+// Forward differences at row 0 (unit steps) of the cubic through v[] at the node
+// rows 0, 10, 21, 31: from its divided differences c1, c2, c3,
+// p(r) = v0 + c1 r + c2 r (r - 10) + c3 r (r - 10) (r - 21).
+__host__ __device__ __forceinline__ void hp_differences(const double* v, long long* d) {
+    const double f01 = (v[1] - v[0]) * (1.0 / 10.0), f12 = (v[2] - v[1]) * (1.0 / 11.0), f23 = (v[3] - v[2]) * (1.0 / 10.0);
+    const double f012 = (f12 - f01) * (1.0 / 21.0), f123 = (f23 - f12) * (1.0 / 21.0);
+    const double c3 = (f123 - f012) * (1.0 / 31.0);
+    // r (r - 10) has differences -9, 2; r (r - 10) (r - 21) has 180, -56, 6
+    d[0] = (long long)v[0];
+    d[1] = (long long)(f01 - 9.0 * f012 + 180.0 * c3);
+    d[2] = (long long)(2.0 * f012 - 56.0 * c3);
+    d[3] = (long long)(6.0 * c3);
+}
+
+// a + t (b - a) with t = th + tl, a = ah + al, b = bh + bl as unevaluated pairs.
+struct F2p { float h, l; };
+__host__ __device__ __forceinline__ F2p hp_lerp(F2p a, F2p b, float th, float tl) {
+    const float d = b.h - a.h, bb = d + a.h;               // d + e = b.h - a.h exactly
+    const float e = (b.h - bb) - (a.h - (bb - d)) + (b.l - a.l);
+    const float p = th * d, pl = fmaf(th, d, -p) + (th * e + tl * d);
+    const float s = a.h + p, q = s - a.h;                  // s + r = a.h + p exactly
+    const float r = (a.h - (s - q)) + (p - q) + (pl + a.l);
+    return {s, r};
+}
+
+__device__ __forceinline__ float hp_nan() { return __int_as_float(0x7fffffff); }
+
+// Frame pixel (x, y), NaN where flagged or not finite.
+__device__ __forceinline__ float hp_fetch(const HpArgs& a, int x, int y) {
+    const long p = (long)y * a.pitch + x;
+    const float f = __ldg(a.frame + p);
+    const unsigned fl = a.flags ? __ldg(a.flags + p) : 0u;
+    return (fabsf(f) <= 3.402823466e38f) & (fl == 0u) ? f : hp_nan();
+}
+
+__global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
+    __shared__ double nd[2][4][4][2];                      // [half][node row][node column][x, y]
+    __shared__ long long dif[2][HP_PATCH][4];              // [x, y][column] forward differences of a half
+    __shared__ int box[2][4];                              // staged rectangle of a half: x0, y0, x1, y1
+    __shared__ int okh[2];                                 // half interpolated
+    extern __shared__ float hp_smem[];                     // staged frame pixels
+    const int tid = threadIdx.x, lane = tid & 31, col = tid & 63, grp = tid >> 6;
+    const int ppr = 1 << (a.k - 6);                        // patches per row
+    const long s = blockIdx.x / (ppr * ppr);
+    const int pq = (int)(blockIdx.x - s * ppr * ppr);
+    const int c0 = (pq % ppr) * HP_PATCH, rp = (pq / ppr) * HP_PATCH;
     const long m = 1L << a.k;
-    const long rows = (long)a.n_seg * m;
-    const int npieces = (int)(m / HP_PIECE);
-    const long warps = (long)gridDim.x * (blockDim.x >> 5);
-    for (long wr = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wr < rows; wr += warps) {
-        const long s = wr / m;
-        const int r = (int)(wr - s * m);
-        const long long seg = a.segs[s];
-        float* orow = a.out + wr * m;
-        uint8_t* crow = a.cov ? a.cov + wr * m : nullptr;
-        if (!hp_row_in_belt(a, seg, r)) {
-            for (int c = lane; c < m; c += 32) {
+    const long long seg = a.segs[s];
+    float* out = a.out + s * m * m;
+    uint8_t* cov = a.cov ? a.cov + s * m * m : nullptr;
+    if (tid < 32) {
+        const int hf = lane >> 4, jr = (lane >> 2) & 3, jc = lane & 3;
+        double x = 0.0, y = 0.0;
+        const int c = c0 + hp_node(jc), r = rp + hf * HP_HALF + hp_node_row(jr);
+        const bool ok = hp_pixel_xy(a, seg, c, r, x, y) && fabs(x) < HP_FAR && fabs(y) < HP_FAR &&
+                        hp_pixel_in_belt(a, seg, c, r);
+        nd[hf][jr][jc][0] = x;
+        nd[hf][jr][jc][1] = y;
+        const unsigned half = hf ? 0xffff0000u : 0x0000ffffu;
+        const bool all = (__ballot_sync(0xffffffffu, ok) & half) == half;
+        const int xi = ok ? (int)floor(x) : 0, yi = ok ? (int)floor(y) : 0;
+        int bx0 = xi, bx1 = xi, by0 = yi, by1 = yi;
+        for (int o = 8; o > 0; o >>= 1) {                  // over the half's 16 lanes
+            bx0 = min(bx0, __shfl_xor_sync(0xffffffffu, bx0, o));
+            bx1 = max(bx1, __shfl_xor_sync(0xffffffffu, bx1, o));
+            by0 = min(by0, __shfl_xor_sync(0xffffffffu, by0, o));
+            by1 = max(by1, __shfl_xor_sync(0xffffffffu, by1, o));
+        }
+        if ((lane & 15) == 0) {
+            okh[hf] = all;
+            box[hf][0] = max(bx0 - 1, 0);
+            box[hf][1] = max(by0 - 1, 0);
+            box[hf][2] = min(bx1 + 2, a.w - 1);
+            box[hf][3] = min(by1 + 2, a.h - 1);
+        }
+    }
+    __syncthreads();
+    for (int hf = 0; hf < 2; hf++) {
+        const int r0 = rp + hf * HP_HALF;
+        if (!okh[hf]) {                                    // the same for the whole CTA
+            for (int i = 0; i < HP_HALF / 4; i++) {
+                const int r = r0 + grp * (HP_HALF / 4) + i;
                 double x, y;
                 float v = 0.0f;
-                const bool ok = hp_pixel_xy(a, seg, c, r, x, y) && hp_bilinear(a, x, y, v);
-                orow[c] = ok ? v : 0.0f;
-                if (crow) crow[c] = ok ? 1 : 0;
+                const bool ok = hp_pixel_xy(a, seg, c0 + col, r, x, y) && hp_bilinear(a, x, y, v);
+                const long e = (long)r * m + c0 + col;
+                out[e] = ok ? v : 0.0f;
+                if (cov) cov[e] = ok ? 1 : 0;
             }
             continue;
         }
-        for (int pg = 0; pg < npieces; pg += 8) {
-            const int p = pg + (lane >> 2), j = lane & 3;
-            double xn = 0.0, yn = 0.0;
-            bool okn = false;
-            if (p < npieces) okn = hp_pixel_xy(a, seg, p * HP_PIECE + hp_node(j), r, xn, yn);
-            // the piece's four nodes from lanes 4 (lane / 4) + 0..3
-            double fx[4], fy[4];
-            bool all = true;
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int src = (lane & ~3) + q;
-                fx[q] = __shfl_sync(0xffffffffu, xn, src);
-                fy[q] = __shfl_sync(0xffffffffu, yn, src);
-                all = all && __shfl_sync(0xffffffffu, okn ? 1 : 0, src);
+        if (tid < 2 * HP_PATCH) {                          // grp 0: x, grp 1: y
+            double v[4];
+            for (int j = 0; j < 4; j++) {
+                v[j] = 0.0;
+                for (int i = 0; i < 4; i++) v[j] += hp_weights.w[col][i] * nd[hf][j][i][grp];
             }
-            if (p >= npieces) continue;                 // no barrier or shuffle below
-            double dx[4], dy[4];
-            hp_cubic_coeffs(fx, dx);
-            hp_cubic_coeffs(fy, dy);
-            for (int i = 0; i < HP_PIECE / 4; i++) {
-                const int t = 4 * i + j;
-                const int c = p * HP_PIECE + t;
-                double x, y;
-                bool ok;
-                if (all) {
-                    x = hp_cubic_eval(dx, (double)t);
-                    y = hp_cubic_eval(dy, (double)t);
-                    ok = true;
-                } else {
-                    ok = hp_pixel_xy(a, seg, c, r, x, y);
+            long long d[4];
+            hp_differences(v, d);
+            for (int i = 0; i < 4; i++) dif[grp][col][i] = d[i];
+        }
+        const int bx0 = box[hf][0], by0 = box[hf][1], bw = box[hf][2] - bx0 + 1, bh = box[hf][3] - by0 + 1;
+        // shared row pitch: neighbouring columns step by (dx, dy); with a pitch of 0 mod 32 their bank
+        // is x, with 1 mod 32 it is x + y -- take the one that moves
+        const double dx = nd[hf][0][3][0] - nd[hf][0][0][0], dy = nd[hf][0][3][1] - nd[hf][0][0][1];
+        const int P = ((bw + 31) & ~31) + (2.0 * fabs(dx) < fabs(dy) ? 1 : 0);
+        const bool staged = bw > 0 && bh > 0 && (long)P * bh <= HP_CAP;
+        if (staged) {
+            // a warp takes eight rows at a time (the last repeated), all their loads in flight
+            for (int y0 = (tid >> 5) * 8; y0 < bh; y0 += 64)
+                for (int x = lane; x < bw; x += 32) {
+                    float f[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) f[i] = hp_fetch(a, bx0 + x, by0 + min(y0 + i, bh - 1));
+#pragma unroll
+                    for (int i = 0; i < 8; i++) hp_smem[min(y0 + i, bh - 1) * P + x] = f[i];
                 }
-                float v = 0.0f;
-                ok = ok && hp_bilinear(a, x, y, v);
-                orow[c] = ok ? v : 0.0f;
-                if (crow) crow[c] = ok ? 1 : 0;
+        }
+        __syncthreads();
+        long long d[2][4];
+        {
+            const int q = grp * (HP_HALF / 4);             // first row: differences there from those at row 0
+            const int q2 = q * (q - 1) / 2, q3 = q * (q - 1) * (q - 2) / 6;
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                const long long* f = dif[i][col];
+                d[i][0] = f[0] + q * f[1] + q2 * f[2] + q3 * f[3];
+                d[i][1] = f[1] + q * f[2] + q2 * f[3];
+                d[i][2] = f[2] + q * f[3];
+                d[i][3] = f[3];
             }
         }
+        const long long xmax = (long long)(a.w - 1) << HP_FRAC, ymax = (long long)(a.h - 1) << HP_FRAC;
+        long e = (long)(r0 + grp * (HP_HALF / 4)) * m + c0 + col;
+#pragma unroll 2
+        for (int i = 0; i < HP_HALF / 4; i++, e += m) {
+            const long long X = d[0][0], Y = d[1][0];
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                d[j][0] += d[j][1];
+                d[j][1] += d[j][2];
+                d[j][2] += d[j][3];
+            }
+            float v = 0.0f;
+            bool ok = X >= 0 && Y >= 0 && X <= xmax && Y <= ymax;
+            if (ok) {
+                const int x0 = (int)(X >> HP_FRAC), y0 = (int)(Y >> HP_FRAC);
+                constexpr long long FM = (1LL << HP_FRAC) - 1;
+                const long long fx = X & FM, fy = Y & FM;
+                const int sx = fx ? 1 : 0, sy = fy ? 1 : 0;     // neighbours with a nonzero weight
+                float q00, q01, q10, q11;
+                const int lx = x0 - bx0, ly = y0 - by0;
+                if (staged && lx >= 0 && ly >= 0 && lx + sx < bw && ly + sy < bh) {
+                    const float* p = hp_smem + ly * P + lx;
+                    q00 = p[0];
+                    q01 = p[sx];
+                    q10 = p[sy * P];
+                    q11 = p[sy * P + sx];
+                } else {
+                    q00 = hp_fetch(a, x0, y0);
+                    q01 = hp_fetch(a, x0 + sx, y0);
+                    q10 = hp_fetch(a, x0, y0 + sy);
+                    q11 = hp_fetch(a, x0 + sx, y0 + sy);
+                }
+                // the fraction as 24 + 20 bits
+                const float xh = (float)(int)(fx >> 20) * 0x1p-24f, xl = (float)(int)(fx & 0xfffff) * 0x1p-44f;
+                const float yh = (float)(int)(fy >> 20) * 0x1p-24f, yl = (float)(int)(fy & 0xfffff) * 0x1p-44f;
+                const F2p top = hp_lerp({q00, 0.0f}, {q01, 0.0f}, xh, xl), bot = hp_lerp({q10, 0.0f}, {q11, 0.0f}, xh, xl);
+                const F2p r = hp_lerp(top, bot, yh, yl);
+                v = r.h + r.l;
+                ok = q00 == q00 && q01 == q01 && q10 == q10 && q11 == q11;
+                if (ok && !isfinite(v))                    // differences beyond FP32: lerps in FP64
+                    hp_bilinear(a, (double)X * 0x1p-44, (double)Y * 0x1p-44, v);
+            }
+            out[e] = ok ? v : 0.0f;
+            if (cov) cov[e] = ok ? 1 : 0;
+        }
+        __syncthreads();                                   // the staged pixels and differences are done with
     }
 }
 
@@ -265,11 +436,11 @@ extern "C" int argus_healpix_resample(const float* frame, const uint8_t* flags, 
     a.frame = frame; a.flags = flags; a.pitch = shape.pitch; a.w = shape.w; a.h = shape.h;
     a.segs = segs; a.n_seg = n_seg; a.nside_seg = nside_seg; a.k = k; a.out = out; a.cov = coverage;
     hp_fill_wcs(a, wcs);
-    if (k >= 6) {                                  // rows of whole 64-pixel pieces: row interpolation
-        const long rows = (long)n_seg << k;
-        long blocks = (rows + 7) / 8;                  // 8 warps (rows) per CTA
-        if (blocks > 152L * 32) blocks = 152L * 32;
-        healpix_rows_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(a);
+    if (k >= 6) {                                  // whole 64 x 64 patches
+        const long long patches = (long long)n_seg << (2 * (k - 6));
+        if (patches > 0x7fffffffLL) return ARGUS_ERR_ARG;
+        const size_t smem = HP_CAP * sizeof(float);
+        healpix_patch_kernel<<<(unsigned)patches, 256, smem, (cudaStream_t)stream>>>(a);
     } else {
         const long total = (long)n_seg << (2 * k);
         long blocks = (total + 255) / 256;

@@ -55,3 +55,47 @@ def test_healpix_resample_parity(ora, nside_seg, k, delta0):
         o, oc = hp.resample_segment(frame, fl, int(s), nside_seg, k, wcs)
         np.testing.assert_array_equal(cov[i], oc)
         assert np.abs(out[i] - o).max() <= tol
+
+
+@pytest.mark.parametrize("nside_seg,k,delta0,step,rot", [(256, 6, 0.3, 1.0, 0.8),     # staged, axes near 45 degrees
+                                                         (64, 7, -0.2, 6.0, 0.0),     # rectangles too large to stage
+                                                         (128, 7, 0.7297, 1.1, 0.3),  # the belt's edge inside the patches
+                                                         (256, 8, 0.1, 0.2, -2.0)])   # several image pixels per frame pixel
+def test_healpix_patches(ora, nside_seg, k, delta0, step, rot):
+    """The patch path's forms (staged and gathered pixels, halves across the belt's edge, segments
+    hanging off the frame, values beyond FP32's differences) at the bars of the parity test; `step` is the
+    image's pixel in frame pixels."""
+    from oracle import healpix as hp
+    rng = np.random.default_rng(nside_seg + k)
+    w, h = 333, 287
+    scale = math.sqrt(4 * math.pi / (12.0 * (nside_seg << k) ** 2)) / step
+    wcs = (0.9, delta0, scale, rot, (w - 1) / 2, (h - 1) / 2)
+    frame = (300 + rng.normal(0, 10, (h, w))).astype(np.float32)
+    frame.flat[11::701] = np.nan
+    frame.flat[13::997] = -np.inf
+    fl = (rng.random((h, w)) < 0.01).astype(np.uint8)
+    p = np.arange(12 * nside_seg * nside_seg)
+    ix, iy, f = hp.nest2xyf(p, nside_seg)
+    x, y = hp.gnomonic(hp.xyf2vec(ix, iy, f, nside_seg), *wcs)
+    d = np.where(np.isfinite(x), (x - w / 2) ** 2 + (y - h / 2) ** 2, np.inf)
+    segs = np.concatenate([p[np.argsort(d)[:4]], [12 * nside_seg * nside_seg]]).astype(np.int64)
+    m = 1 << k
+    for big in (False, True):
+        if big:
+            frame[::3, ::2] = 3.0e38
+            frame[1::3, ::2] = -3.0e38
+        out = torch.full((segs.size, m, m), -7.0, device="cuda")
+        cov = torch.full((segs.size, m, m), 7, dtype=torch.uint8, device="cuda")
+        B.argus_healpix_resample(dev_pitched(frame), dev_pitched(fl), B.argus_shape(w, h, pitch_for(w)), wcs,
+                                 nside_seg, k, torch.from_numpy(segs).cuda(), segs.size, out, cov)
+        torch.cuda.synchronize()
+        out, cov = out.cpu().numpy(), cov.cpu().numpy()
+        tol = 4 * F32_EPS * float(np.abs(frame[np.isfinite(frame)]).max())
+        for i, s in enumerate(segs[:-1]):
+            o, oc = hp.resample_segment(frame, fl, int(s), nside_seg, k, wcs)
+            np.testing.assert_array_equal(cov[i], oc)
+            if big:     # a gradient of 6e38 per pixel: a position's 1e-7 pixel is 6e31 there, so only the range
+                assert np.isfinite(out[i]).all() and np.abs(out[i]).max() <= 3.0e38 * (1 + F32_EPS)
+            else:
+                assert np.abs(out[i] - o).max() <= tol
+        assert not out[-1].any() and not cov[-1].any()      # not a pixel of this NSIDE
