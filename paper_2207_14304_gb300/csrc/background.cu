@@ -32,6 +32,7 @@ struct BgArgs {
     double* mesh;       // [ny][nx] filtered
     float* meshf;       // [ny][nx] the filtered mesh rounded to FP32
     int* missing;       // [1] neighbourhoods without a value
+    double* fill;       // [1] what they take, when there are any
     float* map;
     long pitch;
     int w, h, box, filt, nx, ny;
@@ -378,6 +379,7 @@ __global__ void __launch_bounds__(FILL_THREADS) mesh_fill_kernel(BgArgs a) {
     if (*a.missing == 0) return;
     const int ncell = a.nx * a.ny;
     const auto fill_in = [&](double v) {
+        if (threadIdx.x == 0) *a.fill = v;
         for (int i = threadIdx.x; i < ncell; i += FILL_THREADS)
             if (isnan(a.mesh[i])) {
                 a.mesh[i] = v;
@@ -558,10 +560,11 @@ extern "C" int argus_background(argus_ctx* ctx, const float* img, const uint8_t*
     BgArgs a;
     a.img = img; a.flags = flags; a.mesh = mesh; a.map = map; a.pitch = shape.pitch;
     a.w = shape.w; a.h = shape.h; a.box = box; a.filt = filt; a.nx = nx; a.ny = ny; a.min_frac = min_frac;
-    // scratch in the detection label buffer: the raw mesh, its FP32 copy and the count of
-    // cells to fill, 12 bytes per box and 4 (max_pixels ints are 256 bytes per 8 x 8 box)
+    // scratch in the detection label buffer: the raw mesh, the fill value, the mesh in FP32 and
+    // the count of cells to fill, 12 bytes per box and 12 (max_pixels ints are 256 bytes per 8 x 8 box)
     a.raw = reinterpret_cast<double*>(ctx->label);
-    a.meshf = reinterpret_cast<float*>(a.raw + (long)nx * ny);
+    a.fill = a.raw + (long)nx * ny;
+    a.meshf = reinterpret_cast<float*>(a.fill + 1);
     a.missing = reinterpret_cast<int*>(a.meshf + (long)nx * ny);
     if (cudaMemsetAsync(a.missing, 0, sizeof(int), s) != cudaSuccess) return ARGUS_ERR_CUDA;
     const int npl = (box * box + BOX_THREADS - 1) / BOX_THREADS;   // keys per thread: the smallest compiled bound
