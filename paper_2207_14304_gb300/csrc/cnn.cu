@@ -20,6 +20,7 @@
 #include <stdlib.h>
 
 #include "argus_internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace {
 
@@ -267,66 +268,135 @@ __global__ void __launch_bounds__(256) cnn_conv7_dgrad_kernel(const float* dh_ou
     }
 }
 
-// weight gradient of a conv7 layer for one kernel row ky (blockIdx.y):
-// dW[ky][kx][i][o] = sum_{img,y,x} in[y+ky-3][x+kx-3][i] dz[y][x][o], db[o] = sum dz[o].
-// 448 threads: (kx, 4 input channels, 4 output channels) each; images in chunks per CTA.
-// Each CTA (chunk bx of images, kernel row ky) writes its sums to its own partial slot
-// part[bx][ky * KS * C * C .. + KS * C * C) (and the bias partial at [bx][49 C C ..] for
-// ky = 0); the slots are reduced in a fixed order afterwards.
+// Weight gradient of a conv7 layer for one kernel row ky (blockIdx.y):
+// dW[ky][kx][i][o] = sum_{img,y,x} in[y+ky-3][x+kx-3][i] dz[y][x][o], db[o] = sum dz[o],
+// dz = dh_out * (h_out > 0).  FP32 on the CUDA cores, whose multiply-adds bound it
+// (45 G a step of 512 stamps: 1.2 ms at 128 per clock and SM).
+//
+// A thread holds 2 input x 4 output channels for all 7 kx: along a row it keeps the
+// last 7 inputs in registers (a window that rotates by name, the row of 21 being
+// three turns of 7), so a pixel costs one 8-byte and one 16-byte shared load for 56
+// multiply-adds, on packed FP32 pairs (two output channels).  128 threads cover
+// the 32 x 32 channels; a CTA stages half an image (11 or 10 rows and the input rows
+// they read, 68 KB), so that three CTAs an SM hide one another's staging.  The version
+// with 4 x 4 channels of one kx per thread loaded 8 words for 16 multiply-adds from
+// rows of odd pitch.  The sums of one half image (231 terms) are added to the CTA's
+// totals, so no FP32 sum runs over thousands of terms.
+//
+// CTA (bx, ky) takes half images bx, bx + gridDim.x, ... and writes its sums to its own
+// partial slot part[bx][ky * KS * C * C .. + KS * C * C) (and the bias partial at
+// [bx][49 C C ..] for ky = 0); the slots are reduced in a fixed order afterwards.
 constexpr long WPART = 49L * 1024 + 32;   // one layer's weights and biases
-__global__ void __launch_bounds__(448) cnn_conv7_wgrad_kernel(const float* hin, const float* dh_out,
-                                                              const float* h_out, float* part, int n,
-                                                              int per_cta) {
+constexpr int WG_T = 128, WG_ROWS = 11;
+constexpr size_t WG_SMEM = sizeof(float) * (WG_ROWS * SP * C + WG_ROWS * S * C);
+
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void add2(unsigned long long& d, unsigned long long a) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a));
+}
+__device__ __forceinline__ unsigned long long both(float v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+
+__global__ void __launch_bounds__(WG_T, 3) cnn_conv7_wgrad_kernel(const float* hin, const float* dh_out,
+                                                                  const float* h_out, float* part, int n) {
     extern __shared__ __align__(16) float sm[];
-    float* pad = sm;                                 // input, zero padded
-    float* dz = pad + PADSZ;                  // [441][CS]
-    const int ky = blockIdx.y;
-    const int t = threadIdx.x;
-    const int kx = t / 64, r = t - kx * 64, i4 = r & 7, o4 = r >> 3;
-    float acc[4][4];
+    float* hs = sm;                           // [WG_ROWS][27][32] input rows, zero padded
+    float* ds = sm + WG_ROWS * SP * C;        // [WG_ROWS][21][32] dz
+    const int ky = blockIdx.y, t = threadIdx.x, ip = t & 15, oq = t >> 4;
+    for (int e = t; e < WG_ROWS * 6 * C; e += WG_T) {             // the padding columns, once
+        const int r = e / (6 * C), q = e - r * 6 * C, x = q / C;
+        hs[(r * SP + (x < 3 ? x : x + S)) * C + q % C] = 0.0f;
+    }
+    unsigned long long tot[KS][2][2];
 #pragma unroll
-    for (int a = 0; a < 4; a++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[a][c] = 0.0f;
-    float accb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    const int i0 = blockIdx.x * per_cta, i1 = min(n, i0 + per_cta);
-    for (int img = i0; img < i1; img++) {
-        __syncthreads();
-        stage_padded(hin + (long)img * NPX * C, pad, nullptr);
-        for (int e = threadIdx.x; e < NPX * C; e += blockDim.x) {
-            const int p = e / C, c = e - p * C;
-            const float hv = h_out[(long)img * NPX * C + e];
-            dz[p * CS + c] = hv > 0.0f ? dh_out[(long)img * NPX * C + e] : 0.0f;
+    for (int k = 0; k < KS; k++) tot[k][0][0] = tot[k][0][1] = tot[k][1][0] = tot[k][1][1] = 0ull;
+    float totb = 0.0f;
+    for (int item = blockIdx.x; item < 2 * n; item += gridDim.x) {
+        const int yb = (item & 1) * WG_ROWS, nr = min(WG_ROWS, S - yb), nch = nr * S * (C / 4);
+        const long base = (long)(item >> 1) * NPX * C;
+        __syncthreads();                      // the previous item is consumed
+        for (int e = t; e < nch; e += WG_T) {
+            const int r = e / (S * C / 4), q = e - r * (S * C / 4), gy = yb + r + ky - 3;
+            const bool in = gy >= 0 && gy < S;
+            tc::cp_async16(hs + (r * SP + 3) * C + q * 4, hin + base + (in ? (long)gy * S * C + q * 4 : 0L), in ? 16 : 0);
         }
+        tc::cp_async_commit();
+        const float4* g4 = reinterpret_cast<const float4*>(dh_out + base + yb * S * C);
+        const float4* m4 = reinterpret_cast<const float4*>(h_out + base + yb * S * C);
+#pragma unroll 4
+        for (int e = t; e < nch; e += WG_T) {
+            float4 g = __ldg(g4 + e);
+            const float4 m = __ldg(m4 + e);
+            g.x = m.x > 0.0f ? g.x : 0.0f;
+            g.y = m.y > 0.0f ? g.y : 0.0f;
+            g.z = m.z > 0.0f ? g.z : 0.0f;
+            g.w = m.w > 0.0f ? g.w : 0.0f;
+            reinterpret_cast<float4*>(ds)[e] = g;
+        }
+        tc::cp_async_wait<0>();
         __syncthreads();
-        if (kx < KS) {
-            for (int p = 0; p < NPX; p++) {
-                const int y = p / S, x = p - y * S;
-                const float* hi = pad + ((y + ky) * SP + (x + kx)) * CS + i4 * 4;
-                const float* dd = dz + p * CS + o4 * 4;
-                float hv[4], dv[4];
+        unsigned long long acc[KS][2][2];
 #pragma unroll
-                for (int a = 0; a < 4; a++) { hv[a] = hi[a]; dv[a] = dd[a]; }
+        for (int k = 0; k < KS; k++) acc[k][0][0] = acc[k][0][1] = acc[k][1][0] = acc[k][1][1] = 0ull;
+#pragma unroll 1
+        for (int r = 0; r < nr; r++) {
+            const float* hr = hs + r * SP * C + 2 * ip;
+            const float* dr = ds + r * S * C + 4 * oq;
+            unsigned long long w[KS][2];      // input columns x .. x + 6 at index (x + k) mod 7, each value twice
 #pragma unroll
-                for (int a = 0; a < 4; a++)
+            for (int k = 0; k < KS - 1; k++) {
+                const float2 h = *reinterpret_cast<const float2*>(hr + k * C);
+                w[k][0] = both(h.x);
+                w[k][1] = both(h.y);
+            }
+#pragma unroll 1
+            for (int x = 0; x < S; x += KS) {
 #pragma unroll
-                    for (int c = 0; c < 4; c++) acc[a][c] = fmaf(hv[a], dv[c], acc[a][c]);
-                if (ky == 0 && kx == 0 && i4 == 0)
+                for (int j = 0; j < KS; j++) {
+                    const float2 h = *reinterpret_cast<const float2*>(hr + (x + j + KS - 1) * C);
+                    const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(dr + (x + j) * C);
+                    w[(j + KS - 1) % KS][0] = both(h.x);
+                    w[(j + KS - 1) % KS][1] = both(h.y);
 #pragma unroll
-                    for (int c = 0; c < 4; c++) accb[c] += dv[c];
+                    for (int k = 0; k < KS; k++)
+#pragma unroll
+                        for (int a = 0; a < 2; a++) {
+                            fma2(acc[k][a][0], d.x, w[(j + k) % KS][a]);
+                            fma2(acc[k][a][1], d.y, w[(j + k) % KS][a]);
+                        }
+                }
             }
         }
+#pragma unroll
+        for (int k = 0; k < KS; k++)
+#pragma unroll
+            for (int a = 0; a < 2; a++) {
+                add2(tot[k][a][0], acc[k][a][0]);
+                add2(tot[k][a][1], acc[k][a][1]);
+            }
+        if (ky == 0) {                        // bias: channel t % 32, every fourth pixel
+            float b = 0.0f;
+            for (int p = t / C; p < nr * S; p += WG_T / C) b += ds[p * C + t % C];
+            totb += b;
+        }
     }
-    if (kx < KS) {
-        float* gW = part + (long)blockIdx.x * WPART;
+    float* gW = part + (long)blockIdx.x * WPART;
 #pragma unroll
-        for (int a = 0; a < 4; a++)
+    for (int k = 0; k < KS; k++)
 #pragma unroll
-            for (int c = 0; c < 4; c++)
-                gW[((long)(ky * KS + kx) * C + i4 * 4 + a) * C + o4 * 4 + c] = acc[a][c];
-        if (ky == 0 && kx == 0 && i4 == 0)
-#pragma unroll
-            for (int c = 0; c < 4; c++) gW[49L * 1024 + o4 * 4 + c] = accb[c];
+        for (int a = 0; a < 2; a++)
+            *reinterpret_cast<ulonglong2*>(gW + ((long)(ky * KS + k) * C + 2 * ip + a) * C + 4 * oq) =
+                make_ulonglong2(tot[k][a][0], tot[k][a][1]);
+    if (ky == 0) {
+        __syncthreads();
+        sm[t] = totb;
+        __syncthreads();
+        if (t < C) gW[49L * 1024 + t] = (sm[t] + sm[C + t]) + (sm[2 * C + t] + sm[3 * C + t]);
     }
 }
 
@@ -738,7 +808,6 @@ struct argus_cnn {
 };
 
 static size_t fwd_smem() { return sizeof(float) * ((size_t)PADSZ + (size_t)KS * C * C); }
-static size_t wgrad_smem() { return sizeof(float) * ((size_t)PADSZ + (size_t)NPX * CS); }
 
 extern "C" int argus_cnn_create(argus_cnn** out, int device, int max_batch, unsigned long long seed) {
     if (!out || max_batch < 1) return ARGUS_ERR_ARG;
@@ -782,7 +851,8 @@ extern "C" int argus_cnn_create(argus_cnn** out, int device, int max_batch, unsi
     cudaFuncSetAttribute(cnn_conv7_dgrad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem());
     cudaFuncSetAttribute(cnn_conv7_dgrad_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)fwd_smem());
-    cudaFuncSetAttribute(cnn_conv7_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem());
+    cudaFuncSetAttribute(cnn_conv7_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
+    cudaFuncSetAttribute(cnn_conv7_wgrad_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         argus_cnn_destroy(n);
         return ARGUS_ERR_CUDA;
@@ -877,10 +947,9 @@ static int backward_impl(argus_cnn* nn, const WT* w, const float* x, const float
     for (int l = 3; l >= 0; l--) {
         const float* hin = nn->acts + l * L;
         const float* hout = nn->acts + (l + 1) * L;
-        int per = (n + nn->num_sms - 1) / nn->num_sms;
-        if (per < 1) per = 1;
-        const int nbx = (n + per - 1) / per;
-        cnn_conv7_wgrad_kernel<<<dim3(nbx, KS), 448, wgrad_smem(), st>>>(hin, dh, hout, nn->part, n, per); argus_count_launch(1);
+        // three CTAs per SM in all, one chunk of half images per kernel row each (nbx <= num_sms slots)
+        const int nbx = max(1, min(2 * n, 3 * nn->num_sms / KS));
+        cnn_conv7_wgrad_kernel<<<dim3(nbx, KS), WG_T, WG_SMEM, st>>>(hin, dh, hout, nn->part, n); argus_count_launch(1);
         cnn_reduce_kernel<<<rg, 256, 0, st>>>(nn->part, nbx, WPART, nn->grad + off_w(l)); argus_count_launch(1);
         if (tc_dgrad) {
             const int rc = argus_cnn_dgrad_tc(dh, hout, nn->wbf, nn->wpack, l, n, dn, nn->num_sms, nn->d_status, st);
