@@ -3,16 +3,18 @@
 // a 15-minute coadd; the clipped mean stands in for the matched filter there),
 // with calibration fused in.
 //
-// One thread per output pixel of a 32 x 8 tile.  Per frame, the raw window
-// the tile needs is loaded once, coalesced, and calibrated into shared memory.
-// The frame loop is unrolled to the compile-time stack bound NMAX so every
-// per-frame sample lives in a register at a static index: invalid or absent
-// frames hold +inf and sort to the end.  A bitonic network sorts the samples;
-// because rejection |v - c| > kappa*s keeps a value-closed set, the survivors
-// stay one contiguous range [lo, hi) of the sorted array, so each clipping
-// pass touches only that range of the sorted column in shared memory.
-// Traffic: 2 bytes per frame plus 9 bytes of calibration per pixel in, 9 out.
+// One thread per output pixel of a 31 x 8 tile.  Per frame, the raw window the
+// tile needs is loaded once, coalesced, calibrated and interpolated along x into
+// shared memory.  The frame loop is unrolled to the compile-time stack bound NMAX
+// so every per-frame sample lives in a register at a static index: invalid or
+// absent frames hold +inf and sort to the end.  A merge-exchange network sorts the
+// samples; because rejection |v - c| > kappa*s keeps a value-closed set, the
+// survivors stay one contiguous range [lo, hi) of the sorted array.
+// Traffic: 2 bytes per frame plus 9 bytes of calibration per pixel in, 9 out;
+// the instructions per sample bound it (clipping passes, sort, staging).
 #include "argus_internal.cuh"
+
+#include <utility>
 
 namespace {
 
@@ -30,25 +32,42 @@ struct CoaddArgs {
     float gain, rn2, kappa;
 };
 
+// Batcher's merge exchange (odd-even merge sort) of N values: 191 compare-exchanges
+// for N = 32 (a bitonic network has 240), the pairs listed at compile time so
+// that every index is static.
+template <int N> struct SortNet {
+    unsigned char a[N * 16], b[N * 16];
+    int n;
+};
+template <int N> constexpr SortNet<N> make_sort_net() {
+    SortNet<N> t{};
+    for (int p = 1; p < N; p *= 2)
+        for (int k = p; k >= 1; k /= 2)
+            for (int j = k % p; j + k < N; j += 2 * k)
+                for (int i = 0; i < k && i + j + k < N; i++)
+                    if ((i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+                        t.a[t.n] = (unsigned char)(i + j);
+                        t.b[t.n++] = (unsigned char)(i + j + k);
+                    }
+    return t;
+}
+template <int N> struct SortPairs { static constexpr SortNet<N> net = make_sort_net<N>(); };
+template <int I, int J, int N>
+__device__ __forceinline__ void exchange(float (&s)[N]) {
+    const float a = s[I], b = s[J];
+    s[I] = fminf(a, b);
+    s[J] = fmaxf(a, b);
+}
+template <int N, int... E>
+__device__ __forceinline__ void sort_list(float (&s)[N], std::integer_sequence<int, E...>) {
+    (exchange<SortPairs<N>::net.a[E], SortPairs<N>::net.b[E], N>(s), ...);
+}
 template <int N>
-__device__ __forceinline__ void bitonic_sort(float (&s)[N]) {
-#pragma unroll
-    for (int k = 2; k <= N; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1)
-#pragma unroll
-            for (int i = 0; i < N; i++) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const float a = s[i], b = s[l];
-                    const bool up = (i & k) == 0;
-                    s[i] = up ? fminf(a, b) : fmaxf(a, b);
-                    s[l] = up ? fmaxf(a, b) : fminf(a, b);
-                }
-            }
+__device__ __forceinline__ void sort_values(float (&s)[N]) {
+    sort_list(s, std::make_integer_sequence<int, SortPairs<N>::net.n>());
 }
 
-// One CTA per 32 x 8 output tile.  Per tile:
+// One CTA per 31 x 8 output tile.  Per tile:
 //
 // Phase 0: the calibration constants (the reciprocal of the flat, or NaN where
 // the pixel is unusable -- outside the frame, flagged bad, flat not positive
@@ -58,26 +77,32 @@ __device__ __forceinline__ void bitonic_sort(float (&s)[N]) {
 // UCAP pixels (shifts spread by more than 4 px) each frame's window reads its
 // constants from global memory instead.
 //
-// Phase 1: every frame's (33 x 9) window of raw pixels -- at the frame's
-// integer offset -- calibrated into shared memory as (value, variance) pairs:
-// value NaN where unusable.  The nf x 297 window pixels are spread evenly over
-// the threads; per pixel one raw load and table lookups.  The flat enters
-// through its correctly rounded reciprocal (within 1 ulp of the quotient).
+// Phase 1: a warp per frame: the frame's 32 x 9 window of raw pixels -- at the
+// frame's integer offset -- row by row, one pixel per lane, calibrated (the flat
+// enters through its correctly rounded reciprocal, within 1 ulp of the quotient)
+// and interpolated along x with the next lane's pixel: the row lerp of the value
+// (NaN where a needed pixel is unusable) and the same for the variance by the
+// squared weights.  A row lerp serves the output rows above and below it, and
+// everything about the frame is the same for the whole warp.  Tiles are 31 wide
+// so that the 32 lanes hold every neighbour.
 //
-// Phase 2: each thread interpolates its samples from four shared pairs per
-// frame (the value by nested lerps, the variance by the squared weights) and
-// sums the variances of the valid samples as it goes; it sorts the values in
-// registers with a bitonic network and writes the sorted column to shared
-// memory.  The survivors of a clipping pass stay one contiguous range [lo, hi)
-// of the sorted samples, so each pass reads only that range: the median from
-// two slots, the mean and the spread in two loops over the range, and the
-// rejected samples by scanning inward from both ends (the rejected set is a
-// prefix below the median and a suffix above it, because the rounded distance
-// to the median is monotone in the sample).  The variance of the mean is the
-// valid samples' sum minus the rejected samples' variances, summed with
-// error-free transformations.
-constexpr int CTX = 32, CTY = 8, CWX = CTX + 1, CWY = CTY + 1, CWN = CWX * CWY;
-constexpr int CT = CTX * CTY;                  // threads (one per output pixel of the tile)
+// Phase 2: each thread interpolates its samples along y from two shared values
+// per frame, sorts them in registers and writes the sorted column to shared
+// memory.  A clipping pass takes the median from two slots of it, the sums of
+// v - c and (v - c)^2 over the range from the registers, in ascending order
+// (values outside the range are skipped), and the rejected samples by scanning
+// inward from both ends (the rejected set is a prefix below the median and a
+// suffix above it, because the rounded distance to the median is monotone in the
+// sample).  The variance of the mean then sums the variances of the samples
+// inside the surviving range, compensated.
+//
+// 30 frames of 9576 x 6388: 11.5 ms (4,340 thread instructions per pixel of a
+// 32-frame stack: staging and samples 55 a frame, sort and set-up 820, clipping 920;
+// issue slots 58 % busy with the 16 warps that 105 KB a CTA leave room for), against
+// 18.7 ms with the window staged pixel by pixel over all threads, four-neighbour
+// samples, a bitonic sort and clipping sums from shared memory.
+constexpr int CTX = 31, CTY = 8, CWX = 32, CWY = CTY + 1, CWN = CWX * CWY;
+constexpr int CT = 32 * CTY;                   // threads (one per output pixel of the tile; lane 31 has none)
 constexpr int UCAP = 512;                      // union window capacity (pixels): shift spreads up to 4 px
 constexpr float FMAXF = 3.402823466e38f;
 
@@ -105,177 +130,153 @@ __device__ __forceinline__ float2 calib_const(const CoaddArgs& a, int gx, int gy
     return c;
 }
 
-// Calibrated (value, variance) of one raw pixel given its constants.
+// Calibrated (value, variance) of one raw pixel given its constants, without a
+// branch: the value is NaN where unusable (the variance then means nothing).
 __device__ __forceinline__ float2 calib_pair(const CoaddArgs& a, int raw, float2 c) {
-    float2 r = make_float2(qnan(), 0.0f);
-    if (c.x == c.x && raw < a.sat) {
-        const float ng = (float)(raw - a.bias) * a.gain;
-        const float cv = (ng - c.y) * c.x;
-        if (fabsf(cv) <= FMAXF) {   // non-finite: unusable
-            r.x = cv;
-            r.y = (fmaxf(ng, 0.0f) + a.rn2) * (c.x * c.x);
-        }
+    const float ng = (float)(raw - a.bias) * a.gain;
+    const float cv = (ng - c.y) * c.x;
+    const bool ok = (raw < a.sat) & (fabsf(cv) <= FMAXF);   // false for NaN constants
+    return make_float2(ok ? cv : qnan(), (fmaxf(ng, 0.0f) + a.rn2) * (c.x * c.x));
+}
+
+// The raw pixels of column gx, rows gy .. gy + 8 of frame f (clamped to the frame).
+__device__ __forceinline__ void load_window(const CoaddArgs& a, int f, int gx, int gy, int (&raw)[CWY]) {
+    const uint16_t* src = a.raw + (long)f * a.frame_stride + min(max(gx, 0), a.w - 1);
+    if (gy >= 0 && gy + CWY <= a.h) {      // the same for the whole warp
+        src += (long)gy * a.pitch;
+#pragma unroll
+        for (int r = 0; r < CWY; r++, src += a.pitch) raw[r] = __ldg(src);
+        return;
     }
-    return r;
-}
-
-// s + e = a + b exactly (Knuth's two-sum; no reassociation: the library is not
-// built with fast-math).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// Bilinear sample of one frame from its calibrated window: the value by nested
-// lerps with explicit fused multiply-adds (non-finite when a needed pixel is
-// unusable), the variance as the sum of squared weights (q) times the four
-// pixels' variances.
-__device__ __forceinline__ float sample(const float2* w, int o, float fx, float fy, float4 q, float& var) {
-    const bool n1 = fx > 0.0f, n2 = fy > 0.0f;
-    const float2 p00 = w[o];
-    const float2 p10 = n1 ? w[o + 1] : p00;
-    const float2 p01 = n2 ? w[o + CWX] : p00;
-    const float2 p11 = (n1 && n2) ? w[o + CWX + 1] : (n1 ? p10 : p01);
-    var = q.x * p00.y + (n1 ? q.y * p10.y : 0.0f) + (n2 ? q.z * p01.y : 0.0f) + (n1 && n2 ? q.w * p11.y : 0.0f);
-    const float top = __fmaf_rn(fx, __fsub_rn(p10.x, p00.x), p00.x);
-    const float bot = __fmaf_rn(fx, __fsub_rn(p11.x, p01.x), p01.x);
-    return __fmaf_rn(fy, __fsub_rn(bot, top), top);
+#pragma unroll
+    for (int r = 0; r < CWY; r++) raw[r] = __ldg(src + (long)min(max(gy + r, 0), a.h - 1) * a.pitch);
 }
 
 template <int NMAX>
 __global__ void __launch_bounds__(CT, NMAX <= 32 ? 2 : 1) coadd_kernel(CoaddArgs a) {
     extern __shared__ float4 coadd_smem[];
-    float2* wvr = reinterpret_cast<float2*>(coadd_smem);         // [nf][CWN] (value, variance)
-    float* ss = reinterpret_cast<float*>(wvr + a.nf * CWN);      // [NMAX][CT] sorted samples, a column per thread
+    float* wv = reinterpret_cast<float*>(coadd_smem);            // [nf][CWN] row-interpolated values
+    float* wq = wv + a.nf * CWN;                                 // [nf][CWN] and variances
+    float* ss = wq + a.nf * CWN;                                 // [NMAX][CT] sorted samples, a column per thread
     float2* ucal = reinterpret_cast<float2*>(ss + NMAX * CT);    // [UCAP] union calibration window
-    __shared__ int2 s_j[CWN];              // window pixel j: (union offset jy * UW + jx, raw offset jy * pitch + jx)
-    __shared__ short2 s_jxy[CWN];          // (jx, jy)
-    __shared__ int s_ix[NMAX], s_iy[NMAX], s_fofs[NMAX];
-    __shared__ long long s_rb[NMAX];       // per tile: raw element offset of frame f's window origin
-    __shared__ float2 s_fxy[NMAX];
-    __shared__ float4 s_q[NMAX];
+    __shared__ int s_ix[NMAX], s_iy[NMAX];
+    __shared__ float s_fx[NMAX];
+    __shared__ float4 s_y[NMAX];           // fy, (1 - fy)^2, fy^2, offset of the next row (0 when it has no weight)
     __shared__ int s_umin[2], s_uwh[2];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) { s_umin[0] = s_umin[1] = 1 << 30; s_uwh[0] = s_uwh[1] = -(1 << 30); }
     __syncthreads();
-    for (int f = tid; f < NMAX; f += blockDim.x) {
-        float fxf = 0.0f, fyf = 0.0f;
-        int ix = 0, iy = 0;
-        if (f < a.nf) {
-            const double dx = a.shifts[2 * f], dy = a.shifts[2 * f + 1];
-            const double fx = floor(dx), fy = floor(dy);
-            ix = (int)fx;
-            iy = (int)fy;
-            fxf = (float)(dx - fx);
-            fyf = (float)(dy - fy);
-            atomicMin(&s_umin[0], ix); atomicMin(&s_umin[1], iy);
-            atomicMax(&s_uwh[0], ix); atomicMax(&s_uwh[1], iy);
-        }
+    for (int f = tid; f < a.nf; f += blockDim.x) {
+        const double dx = a.shifts[2 * f], dy = a.shifts[2 * f + 1];
+        const double fx = floor(dx), fy = floor(dy);
+        const int ix = (int)fx, iy = (int)fy;
+        const float fxf = (float)(dx - fx), fyf = (float)(dy - fy);
+        atomicMin(&s_umin[0], ix); atomicMin(&s_umin[1], iy);
+        atomicMax(&s_uwh[0], ix); atomicMax(&s_uwh[1], iy);
         s_ix[f] = ix;
         s_iy[f] = iy;
-        s_fxy[f] = make_float2(fxf, fyf);
-        const float w0 = (1.0f - fxf) * (1.0f - fyf), w1 = fxf * (1.0f - fyf);
-        const float w2 = (1.0f - fxf) * fyf, w3 = fxf * fyf;
-        s_q[f] = make_float4(w0 * w0, w1 * w1, w2 * w2, w3 * w3);
+        s_fx[f] = fxf;
+        s_y[f] = make_float4(fyf, (1.0f - fyf) * (1.0f - fyf), fyf * fyf, __int_as_float(fyf > 0.0f ? CWX : 0));
     }
     __syncthreads();
     const int ixmin = s_umin[0], iymin = s_umin[1];
     const int UW = CWX + (s_uwh[0] - ixmin), UH = CWY + (s_uwh[1] - iymin);
     const bool uni = UW * UH <= UCAP;      // the same for every CTA
-    for (int j = tid; j < CWN; j += blockDim.x) {
-        const int jy = j / CWX, jx = j - jy * CWX;
-        s_j[j] = make_int2(jy * UW + jx, (int)(jy * a.pitch) + jx);
-        s_jxy[j] = make_short2((short)jx, (short)jy);
-    }
-    for (int f = tid; f < a.nf; f += blockDim.x) s_fofs[f] = (s_iy[f] - iymin) * UW + (s_ix[f] - ixmin);
     const int ntx = (a.w + CTX - 1) / CTX, nty = (a.h + CTY - 1) / CTY;
-    const int lx = tid % CTX, ly = tid / CTX;
-    const int o = ly * CWX + lx;
-    const int tot = a.nf * CWN;
+    const int o = warp * CWX + lane;       // output row `warp`, column `lane`
     float* col = ss + tid;
     for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
         const int tx0 = (tile % ntx) * CTX, ty0 = (tile / ntx) * CTY;
-        const int x = tx0 + lx, y = ty0 + ly;
-        __syncthreads();   // tables staged; previous tile's windows consumed
-        for (int f = tid; f < a.nf; f += blockDim.x)
-            s_rb[f] = (long long)f * a.frame_stride + (long long)(ty0 + s_iy[f]) * a.pitch + (tx0 + s_ix[f]);
-        if (uni)
+        const int x = tx0 + lane, y = ty0 + warp;
+        // a warp's next frame is loaded while it works on this one; pixels off the frame read the
+        // nearest one and are unusable through their constants
+        int raw[CWY];
+        if (warp < a.nf) load_window(a, warp, tx0 + s_ix[warp] + lane, ty0 + s_iy[warp], raw);
+        __syncthreads();   // the previous tile's windows are consumed
+        if (uni) {
             for (int e = tid; e < UW * UH; e += blockDim.x) {
                 const int uy = e / UW, ux = e - uy * UW;
                 ucal[e] = calib_const(a, tx0 + ixmin + ux, ty0 + iymin + uy);
             }
-        __syncthreads();
-        // window pixel e = f * CWN + j, e = tid + k * CT: j advances by CT < CWN, wrapping at most once
-        int f = 0, j = tid;
-        constexpr int U = 4;
-        for (int e0 = tid; e0 < tot; e0 += U * CT) {
-            int fu[U], ju[U], raw[U];
-            float2 cu[U];
+            __syncthreads();
+        }
+        for (int f = warp; f < a.nf; f += CTY) {
+            const int gx = tx0 + s_ix[f] + lane, gy = ty0 + s_iy[f];
+            float2 c[CWY];
+            if (uni) {
+                const float2* uc = ucal + (s_iy[f] - iymin) * UW + (s_ix[f] - ixmin) + lane;
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                fu[u] = f;
-                ju[u] = j;
-                j += CT;
-                if (j >= CWN) { j -= CWN; f++; }
+                for (int r = 0; r < CWY; r++) c[r] = uc[r * UW];
+            } else {
+#pragma unroll
+                for (int r = 0; r < CWY; r++) c[r] = calib_const(a, gx, gy + r);
             }
+            float2 p[CWY];
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                const bool live = e0 + u * CT < tot;
-                const int fc = live ? fu[u] : 0;
-                if (uni) {
-                    cu[u] = ucal[s_fofs[fc] + s_j[ju[u]].x];
-                } else {
-                    const short2 jj = s_jxy[ju[u]];
-                    cu[u] = calib_const(a, tx0 + s_ix[fc] + jj.x, ty0 + s_iy[fc] + jj.y);
+            for (int r = 0; r < CWY; r++) p[r] = calib_pair(a, raw[r], c[r]);
+            const int fn = f + CTY;
+            if (fn < a.nf) load_window(a, fn, tx0 + s_ix[fn] + lane, ty0 + s_iy[fn], raw);
+            const float fx = s_fx[f], w0 = (1.0f - fx) * (1.0f - fx), w1 = fx * fx;
+            float* dv = wv + f * CWN + lane;
+            float* dq = wq + f * CWN + lane;
+            if (fx > 0.0f) {
+#pragma unroll
+                for (int r = 0; r < CWY; r++) {
+                    const float nv = __shfl_down_sync(0xffffffffu, p[r].x, 1), nq = __shfl_down_sync(0xffffffffu, p[r].y, 1);
+                    dv[r * CWX] = __fmaf_rn(fx, __fsub_rn(nv, p[r].x), p[r].x);
+                    dq[r * CWX] = w0 * p[r].y + w1 * nq;
                 }
-                raw[u] = (live && cu[u].x == cu[u].x) ? (int)__ldg(a.raw + s_rb[fc] + s_j[ju[u]].y) : 0;
-            }
+            } else {
 #pragma unroll
-            for (int u = 0; u < U; u++)
-                if (e0 + u * CT < tot) wvr[fu[u] * CWN + ju[u]] = calib_pair(a, raw[u], cu[u]);
+                for (int r = 0; r < CWY; r++) {
+                    dv[r * CWX] = p[r].x;
+                    dq[r * CWX] = p[r].y;
+                }
+            }
         }
         __syncthreads();
-        if (x >= a.w || y >= a.h) continue;
-        float u[NMAX], s[NMAX];
+        if (lane >= CTX || x >= a.w || y >= a.h) continue;
+        float s[NMAX];
         int n = 0;
-        float svh = 0.0f, svl = 0.0f;   // compensated sum of the valid samples' variances
+        const float* pv = wv + o;
 #pragma unroll
         for (int fi = 0; fi < NMAX; fi++) {
-            float sv = __int_as_float(0x7f800000);   // +inf: absent or invalid
-            u[fi] = sv;
+            s[fi] = __int_as_float(0x7f800000);      // +inf: absent or invalid
             if (fi < a.nf) {
-                const float2 fxy = s_fxy[fi];
-                float vr;
-                const float v = sample(wvr + fi * CWN, o, fxy.x, fxy.y, s_q[fi], vr);
+                const float4 fy = s_y[fi];
+                const float top = pv[fi * CWN], bot = pv[fi * CWN + __float_as_int(fy.w)];
+                const float v = __fmaf_rn(fy.x, __fsub_rn(bot, top), top);
                 const bool ok = fabsf(v) <= FMAXF;
-                u[fi] = v;
-                sv = ok ? v : sv;
+                s[fi] = ok ? v : s[fi];
                 n += ok ? 1 : 0;
-                float e;
-                two_sum(svh, ok ? vr : 0.0f, svh, e);
-                svl += e;
             }
-            s[fi] = sv;
         }
-        bitonic_sort(s);
+        sort_values(s);
 #pragma unroll
         for (int i = 0; i < NMAX; i++) col[i * CT] = s[i];
         int lo = 0, hi = n;
         float last_s1 = 0.0f;   // sum of v - median over [lo, hi) when the last pass kept every sample
         bool have_s1 = false;
+        // the sums over [lo, hi) about c, in ascending order
+        const auto sums = [&](float c, float& s1, float& s2) {
+            const unsigned long long in = (hi < 64 ? (1ull << hi) - 1ull : ~0ull) & ~((1ull << lo) - 1ull);
+            s1 = s2 = 0.0f;
+#pragma unroll
+            for (int i = 0; i < NMAX; i++)
+                if ((in >> i) & 1ull) {
+                    const float d = s[i] - c;
+                    s1 += d;
+                    s2 = fmaf(d, d, s2);
+                }
+        };
         for (int it = 0; it < a.max_iter && hi > lo; it++) {
             const int cnt = hi - lo;
             const float c = median_col(col, lo, hi);
             // mean and spread in one pass over the range, about the median (the sums of
             // v - c and (v - c)^2; the median lies inside the samples, so the difference
             // of the second sum and the squared first one does not cancel)
-            float s1 = 0.0f, s2 = 0.0f;
-            for (int i = lo; i < hi; i++) {
-                const float d = col[i * CT] - c;
-                s1 += d;
-                s2 = fmaf(d, d, s2);
-            }
+            float s1, s2;
+            sums(c, s1, s2);
             const float d1 = s1 / (float)cnt;
             const float ks = a.kappa * sqrtf(fmaxf(s2 / (float)cnt - d1 * d1, 0.0f));
             int nlo = 0, nhi = 0;
@@ -309,30 +310,28 @@ __global__ void __launch_bounds__(CT, NMAX <= 32 ? 2 : 1) coadd_kernel(CoaddArgs
         const float c = median_col(col, lo, hi);
         const float vlo = col[lo * CT], vhi = col[(hi - 1) * CT];
         float sd = last_s1;   // the converged pass's sum over the same range about the same median
-        if (!have_s1)
-            for (int i = lo; i < hi; i++) sd += col[i * CT] - c;
-        if (cnt < n) {   // the rejected samples' variances out (compensated: a rejected cosmic
-                         // ray's variance can exceed the survivors' sum many times); the
-                         // rejected frames as a bit mask first, then one sample per set bit,
-                         // so a warp runs as many samples as its lane with the most rejections
-            unsigned long long rej = 0ull;
-#pragma unroll
-            for (int fi = 0; fi < NMAX; fi++)
-                if (fi < a.nf && fabsf(u[fi]) <= FMAXF && (u[fi] < vlo || u[fi] > vhi)) rej |= 1ull << fi;
-            while (rej) {
-                const int fi = __ffsll((long long)rej) - 1;
-                rej &= rej - 1ull;
-                const float2 fxy = s_fxy[fi];
-                float vr;
-                sample(wvr + fi * CWN, o, fxy.x, fxy.y, s_q[fi], vr);
-                float e;
-                two_sum(svh, -vr, svh, e);
-                svl += e;
+        if (!have_s1) {
+            float s2;
+            sums(c, sd, s2);
+        }
+        // the survivors' variances (Kahan's compensated sum; the library is not built with fast-math)
+        float sv = 0.0f, se = 0.0f;
+        const float* pq = wq + o;
+#pragma unroll 6
+        for (int fi = 0; fi < a.nf; fi++) {
+            const float4 fy = s_y[fi];
+            const int dn = __float_as_int(fy.w);
+            const float top = pv[fi * CWN], bot = pv[fi * CWN + dn];
+            const float v = __fmaf_rn(fy.x, __fsub_rn(bot, top), top);
+            const float q = fy.y * pq[fi * CWN] + fy.z * pq[fi * CWN + dn];
+            if (v >= vlo && v <= vhi) {                // NaN and infinite samples lie outside
+                const float t = q - se, u = sv + t;
+                se = (u - sv) - t;
+                sv = u;
             }
         }
-        const float svar = svh + svl;
         a.coadd[p] = c + sd / (float)cnt;
-        a.var[p] = svar / ((float)cnt * (float)cnt);
+        a.var[p] = sv / ((float)cnt * (float)cnt);
         a.n_used[p] = (uint8_t)cnt;
     }
 }

@@ -528,3 +528,41 @@ def test_coadd_parity(ora, nf, w, h, amp):
         assert_rel(vg[safe], va[safe], np.maximum(va[safe], 1e-6), 2e-6, "var")
     finally:
         B.argus_destroy(ctx)
+
+
+@pytest.mark.parametrize("nf,w,h,shifts", [
+    (3, 31, 8, [(0.0, 0.0), (1.0, 0.0), (0.0, -1.0)]),                    # whole-pixel shifts: one row or column of weight
+    (9, 33, 17, [(0.0, 0.25), (0.5, 0.0), (-2.0, 3.0), (0.0, 0.0)]),      # a stack larger than 8, tiles of one column
+    (17, 5, 3, [(0.3, -0.4), (0.0, 0.0), (-1.0, 0.5)]),                   # a frame smaller than a tile
+    (33, 62, 40, [(0.1, 0.2), (9.5, -7.25), (0.0, 12.0), (-11.0, 0.0)]),  # windows too far apart to share constants
+])
+def test_coadd_shift_forms(ora, nf, w, h, shifts):
+    """Shifts with no weight on a neighbour, tiles cut by the frame, and every sort size, at the
+    bars of test_coadd_parity."""
+    cal = synth.make_calib(w, h, seed=nf, bad_frac=0.02)
+    sh = np.array([shifts[f % len(shifts)] for f in range(nf)], np.float32)
+    rng = np.random.default_rng(nf)
+    raw = rng.normal(420, 20, (nf, h, w))
+    raw[rng.random(raw.shape) < 0.03] += 5e3
+    raw = raw.round().clip(0, 65535).astype(np.uint16)
+    co, va, nu, mg = ora.coadd(raw, sh, bias=cal.bias, dark=cal.dark.numpy(), flat=cal.flat.numpy(),
+                               bpm=cal.bpm.numpy(), gain=cal.gain, read_noise=cal.read_noise, sat=60000)
+    pitch = pitch_for(w)
+    ctx = ctx_for(w, h)
+    try:
+        stack = torch.zeros((nf, h, pitch), dtype=torch.uint16)
+        stack[:, :, :w] = torch.from_numpy(raw)
+        calg = B.make_calib(cal.bias, dev_pitched(cal.dark.numpy()), dev_pitched(cal.flat.numpy()),
+                            dev_pitched(cal.bpm.numpy()), cal.gain, cal.read_noise, 60000)
+        dco, dva = torch.full((h, pitch), -7.0, device="cuda"), torch.full((h, pitch), -7.0, device="cuda")
+        dnu = torch.full((h, pitch), 7, dtype=torch.uint8, device="cuda")
+        B.argus_coadd(ctx, stack.cuda(), nf, B.argus_shape(w, h, pitch), torch.from_numpy(sh).cuda(), calg, 3.0, 5,
+                      dco, dva, dnu)
+        torch.cuda.synchronize()
+        cg, vg, ng = host(dco, w), host(dva, w), host(dnu, w)
+        safe = mg > 1e-4
+        np.testing.assert_array_equal(ng[safe], nu[safe])
+        assert_rel(cg[safe], co[safe], np.maximum(np.abs(co[safe]), 1.0), 2e-6, "coadd")
+        assert_rel(vg[safe], va[safe], np.maximum(va[safe], 1e-6), 2e-6, "var")
+    finally:
+        B.argus_destroy(ctx)
