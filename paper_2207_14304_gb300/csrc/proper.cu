@@ -103,20 +103,27 @@ __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) row_fwd_k
     const fft::TwReg<T> tw(a.tw, lane);
     float2* b0 = sm + seq * Rg::PT;
     float2* b1 = sm + (Rg::CB + seq) * Rg::PT;
-#pragma unroll 1
-    for (int i = 0; i < ROW_ITER; i++) {
-        const int y = y0 + i * Rg::CB + seq;
+    float2 v[8], nx[8];
+    // row y of the pair (the next group's row is loaded while this one is transformed)
+    const auto load = [&](int y, float2 (&d)[8]) {
         const int gy = oy + y;
         const bool row = gy >= 0 && gy < a.h;
-        float2 v[8];
 #pragma unroll
         for (int m = 0; m < 8; m++) {
             const int gx = ox + lane + m * Rg::LANES;
             const bool in = row && gx >= 0 && gx < a.w;
             const long q = (long)gy * a.pitch + gx;
-            v[m].x = in ? __ldg(s0 + q) : 0.0f;
-            v[m].y = in && s1 ? __ldg(s1 + q) : 0.0f;
+            d[m].x = in ? __ldg(s0 + q) : 0.0f;
+            d[m].y = in && s1 ? __ldg(s1 + q) : 0.0f;
         }
+    };
+    load(y0 + seq, nx);
+#pragma unroll 1
+    for (int i = 0; i < ROW_ITER; i++) {
+        const int y = y0 + i * Rg::CB + seq;
+#pragma unroll
+        for (int m = 0; m < 8; m++) v[m] = nx[m];
+        if (i + 1 < ROW_ITER) load(y + Rg::CB, nx);
         fft::fft_reg<T, -1, 1>(v, tw, b0, b1, lane);
 #pragma unroll
         for (int m = 0; m < 8; m++) z[blocked<T>(y, lane + m * Rg::LANES)] = v[m];
@@ -501,7 +508,7 @@ int run(argus_proper_plan* p, ZArgs& a, const RowArgs& rows, const PsfArgs* psf,
 // IDFT[den / F_R], F_R = sqrt(sum_j F_j^2 / s_j^2).
 // The column kernel keeps U of its columns in registers while it walks the frame
 // pairs, so a pair costs one write and one read of its row transforms: 30 frames
-// of 216 512^2 tiles take 6.95 ms, against 63.8 ms with separate column, separation
+// of 216 512^2 tiles take 5.96 ms, against 63.8 ms with separate column, separation
 // and accumulation passes and FP64 sums for every tile.  The filters and den^2 are made once per
 // PSF, not per tile.  Tiles are taken in chunks whose pairs fit the plan's pool;
 // where not even one tile's do, the pairs are taken in groups and U is carried.
@@ -667,18 +674,24 @@ __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) coadd_col
     const fft::TwReg<T> tw(a.tw, lane);
     float2* b0 = sm + c;
     float2* b1 = sm + CB * Rg::PT + c;
-    float2 u[8], v[8];
+    float2 u[8], v[8], nx[8];
+#pragma unroll
+    for (int m = 0; m < 8; m++) nx[m] = __ldcs(z + m * L * CB);
 #pragma unroll
     for (int m = 0; m < 8; m++) u[m] = a.first ? make_float2(0.0f, 0.0f) : a.zs[blk + m * L * CB];
 #pragma unroll 1
     for (int p = 0; p < a.n_pairs; p++) {
 #pragma unroll
-        for (int m = 0; m < 8; m++) v[m] = __ldcs(z + m * L * CB);
+        for (int m = 0; m < 8; m++) v[m] = nx[m];
         float2 g[8];
 #pragma unroll
         for (int m = 0; m < 8; m++) g[m] = __ldg(f + m * L);
         z += (long)a.n_tiles * T * T;
         f += T * T;
+        if (p + 1 < a.n_pairs) {                           // the next pair's rows arrive during this one's transform
+#pragma unroll
+            for (int m = 0; m < 8; m++) nx[m] = __ldcs(z + m * L * CB);
+        }
         fft::fft_reg<T, -1, CB>(v, tw, b0, b1, lane);
 #pragma unroll
         for (int m = 0; m < 8; m++) {
