@@ -986,7 +986,10 @@ extern "C" int argus_cnn_train_step(argus_cnn* nn, const float* x, const float* 
     if (!nn || !x || !target || n < 1 || n > nn->max_batch || !(lr > 0.0f)) return ARGUS_ERR_ARG;
     if (cudaSetDevice(nn->device) != cudaSuccess) return ARGUS_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = argus_cnn_forward(nn, x, n, nn->y, stream);
+    int rc = nn->precision == ARGUS_PREC_BF16_SPLIT
+                 ? argus_cnn_forward_train_tc(x, nn->wbf, nn->wpack, n, nn->y, nn->acts, (long)nn->max_batch * NPX * C,
+                                              nn->num_sms, nn->d_status, st)
+                 : argus_cnn_forward(nn, x, n, nn->y, stream);
     if (rc) return rc;
     double* loss = loss_out ? loss_out : nn->loss;
     cnn_mse_kernel<<<nn->num_sms * 2, 256, 0, st>>>(nn->y, target, (long)n * NPX, nn->dy, nn->lpart); argus_count_launch(1);

@@ -49,6 +49,21 @@ __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_
         : "memory");
 }
 
+// An MMA issued by the lanes with `elected` set (one), for code that the whole warp runs:
+// where every lane computes the descriptors the compiler keeps them in uniform registers,
+// and an issue costs a few instructions; in a branch that one lane takes, each operand goes
+// through a lane-to-uniform move first, and beside 16 busy warps an issue took 150 to 230
+// clocks (the learned kernel: 61 us an image, 46 us in this form).  Kernels whose issuers
+// wait per few MMAs gained nothing from it (subtraction, segment fit, stamp convolution).
+__device__ __forceinline__ void mma_bf16_warp(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accum, uint32_t elected) {
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum), "r"(elected)
+        : "memory");
+}
+
 __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accum) {
     asm volatile(
@@ -62,6 +77,19 @@ __device__ __forceinline__ void commit(uint64_t* mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                      smem_u32(mbar))
                  : "memory");
+}
+
+// A wait that every lane of an issuing warp makes has one outcome, so that the warp stays
+// together (a lane that gave up alone would leave the others at the next warp barrier).
+__device__ __forceinline__ bool all_lanes(bool ok) { return __all_sync(0xffffffffu, ok); }
+
+// Arrive on an mbarrier when the MMAs issued so far by the lanes with `elected` set have completed.
+__device__ __forceinline__ void commit_warp(uint64_t* mbar, uint32_t elected) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(mbar)),
+        "r"(elected)
+        : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -151,6 +179,17 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[16], uint32_t (&b)[16
                    "+r"(c[8]), "+r"(c[9]), "+r"(c[10]), "+r"(c[11]), "+r"(c[12]), "+r"(c[13]), "+r"(c[14]), "+r"(c[15])
                  :
                  : "memory");
+}
+
+// 32 lanes x 8 consecutive 32-bit columns; the caller waits (tmem_wait_ld, then tmem_use8
+// on each array, so that no use of the registers is scheduled before the wait).
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_use8(uint32_t (&r)[8]) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns; the caller waits (tmem_wait_ld)
