@@ -906,6 +906,7 @@ __global__ void gram_reduce_kernel(const float* part, int nslots, int NP, double
         const int i = (int)(e / NP), j = (int)(e - (long)i * NP);
         if (i > j) continue;
         double s = 0.0;
+#pragma unroll 8
         for (int sl = 0; sl < nslots; sl++) s += (double)part[(long)sl * tot + e];
         M[(long)i * NP + j] = s;
         M[(long)j * NP + i] = s;
@@ -920,7 +921,7 @@ __global__ void gram_reduce_kernel(const float* part, int nslots, int NP, double
 // rate on this part, so the kernels keep FP64 dependency chains short and
 // spread the FP64 work over many SMs: four warps factor the diagonal block
 // (columns interleaved over the warps, reciprocal square roots from an FP32
-// estimate and two FP64 Newton steps); the panel below, L_ip = A_ip L_pp^-T,
+// estimate and one third-order FP64 step); the panel below, L_ip = A_ip L_pp^-T,
 // is one row-parallel triangular solve per warp over the whole GPU, and the
 // same launch solves 32 identity rows, which gives the inverse of the
 // diagonal block; the trailing lower triangle is updated in 16x16 tiles
@@ -938,70 +939,96 @@ __global__ void chol_init_kernel(const double* M, int ld, int n, double* L, doub
     if (blockIdx.x == 0 && threadIdx.x == 0) flag[0] = 0.0;
 }
 
-// 1/sqrt(d) for d > 0: FP32 estimate, then two Newton-Raphson steps
-// r <- r (3 - d r^2) / 2 in FP64 (each squares the relative error, 2^-22 ->
-// 2^-44 -> FP64 rounding).  Outside the FP32 range the FP64 library path.
-__device__ __forceinline__ double rsqrt_newton(double d) {
-    if (!(d > 1e-30 && d < 1e30)) return 1.0 / sqrt(d);
-    double r = (double)rsqrtf((float)d);
-    const double hd = 0.5 * d;
-    r = r * fma(-hd, r * r, 1.5);
-    r = r * fma(-hd, r * r, 1.5);
-    return r;
+// 1/sqrt(d) for d > 0: FP32 estimate y (relative error 2^-22), then one third-order step
+// r = y (1 + e/2 + 3 e^2 / 8), e = 1 - d y^2, in FP64 (the next term, 5 e^3 / 16, is below
+// 2^-64; y^2 is exact).  Four dependent FP64 operations, where two Newton steps are
+// seven; the range is tested on the exponent bits, not with FP64 comparisons.  Outside
+// the FP32 range the FP64 library path.
+__device__ __forceinline__ double rsqrt_refined(double d) {
+    const int ex = __double2hiint(d) >> 20;                // sign and biased exponent
+    if (ex < 1023 - 99 || ex > 1023 + 99) return 1.0 / sqrt(d);
+    const double y = (double)rsqrtf((float)d);
+    const double e = fma(-d, y * y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// Whether a pivot is positive (and not NaN), on its bits.
+__device__ __forceinline__ bool pivot_ok(double d) {
+    const long long b = __double_as_longlong(d);
+    return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
 // Factor the pb x pb diagonal block at (p, p) in place; rdiag[j] = 1 / L_jj.
-// Four warps; warp w holds columns k = 4 q + w of row `lane`.
+// An SM partition starts one FP64 warp instruction per 64 clocks, so what counts is the
+// FP64 instructions of one warp between two pivots.  Warp 0 does nothing but pivots: it
+// takes column j + 1, up to date through column j - 1, from shared memory, applies
+// column j, takes the reciprocal root and writes the finished column: seven FP64
+// instructions.  Meanwhile warps 1-3 (columns k = 3 q + warp - 1 of row `lane`) apply
+// column j to the columns from j + 2 on, and the owner of column j + 2 puts it into
+// shared memory: five or six at the most.  One barrier a column; two buffers of each.
+// 24 us a block, against 35 us with the pivots taken by the warp that owns the column.
 __global__ void __launch_bounds__(128) chol_diag_kernel(double* L, int ld, int p, int pb, double* rdiag, double* flag,
                                                         int* status) {
-    __shared__ double col[CB];
+    __shared__ double col[2][CB], nxt[2][CB];              // finished column j; column j + 1 through column j - 1
     __shared__ int bad;
     if (flag[0] != 0.0) return;
+    constexpr int NQ = (CB + 2) / 3;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double a[CB / 4];
+    double* Lr = L + (long)(p + lane) * ld + p;            // row `lane` of the block
+    const auto load = [&](int k) { return lane < pb && k <= lane ? Lr[k] : 0.0; };
+    double a[NQ];
+    if (warp) {
 #pragma unroll
-    for (int q = 0; q < CB / 4; q++) {
-        const int k = 4 * q + warp;
-        a[q] = (lane < pb && k <= lane) ? L[(long)(p + lane) * ld + p + k] : 0.0;
+        for (int q = 0; q < NQ; q++) {
+            const int k = 3 * q + warp - 1;
+            a[q] = k < CB ? load(k) : 0.0;
+        }
     }
     if (threadIdx.x == 0) bad = 0;
+    // column j from its value `v` in the lanes: finished, stored, and put into col[j & 1]
+    const auto pivot = [&](int j, double v) {
+        const double d = __shfl_sync(0xffffffffu, v, j);
+        const bool ok = pivot_ok(d);
+        const double r = rsqrt_refined(ok ? d : 1.0);
+        const double lij = lane >= j ? v * r : 0.0;        // v is d itself on lane j
+        col[j & 1][lane] = lij;
+        if (lane >= j && lane < pb) Lr[j] = lij;
+        if (lane == 0) {
+            rdiag[p + j] = r;
+            if (!ok) bad = 1;
+        }
+    };
+    __syncthreads();
+    if (warp == 0) {
+        const double v = load(0);
+        pivot(0, v);
+    } else if (warp == 2) {
+        nxt[1][lane] = a[0];                               // column 1, as it came
+    }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < CB; j++) {
-        if (j < pb) {
-            if (warp == (j & 3)) {
-                const double d = __shfl_sync(0xffffffffu, a[j >> 2], j);
-                const bool ok = d > 0.0;
-                const double r = rsqrt_newton(ok ? d : 1.0);
-                const double lij = lane == j ? d * r : (lane > j ? a[j >> 2] * r : 0.0);
-                a[j >> 2] = lij;
-                col[lane] = lij;
-                if (lane == 0) {
-                    rdiag[p + j] = r;
-                    if (!ok) bad = 1;
+    for (int j = 0; j < CB - 1; j++) {
+        if (j < pb - 1) {
+            const double* cj = col[j & 1];
+            const double lij = cj[lane];
+            if (warp == 0) {
+                pivot(j + 1, fma(-lij, cj[j + 1], nxt[(j + 1) & 1][lane]));
+            } else {
+#pragma unroll
+                for (int q = 0; q < NQ; q++) {
+                    const int k = 3 * q + warp - 1;
+                    if (k > j + 1 && k < CB) {
+                        a[q] = fma(-lij, cj[k], a[q]);     // (above the diagonal: never read)
+                        if (k == j + 2) nxt[j & 1][lane] = a[q];
+                    }
                 }
             }
             __syncthreads();
-            const double lij = col[lane];
-#pragma unroll
-            for (int q = 0; q < CB / 4; q++) {
-                const int k = 4 * q + warp;
-                if (k > j && k <= lane) a[q] -= lij * col[k];
-            }
-            __syncthreads();
         }
     }
-    if (bad) {
-        if (threadIdx.x == 0) {
-            flag[0] = 1.0;
-            argus_latch(status, ARGUS_ERR_SINGULAR);
-        }
-        return;
-    }
-#pragma unroll
-    for (int q = 0; q < CB / 4; q++) {
-        const int k = 4 * q + warp;
-        if (lane < pb && k <= lane) L[(long)(p + lane) * ld + p + k] = a[q];
+    if (bad && threadIdx.x == 0) {
+        flag[0] = 1.0;
+        argus_latch(status, ARGUS_ERR_SINGULAR);
     }
 }
 
@@ -1074,59 +1101,79 @@ __global__ void __launch_bounds__(256) chol_update_kernel(double* L, int ld, int
     }
 }
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// x = (L L^T)^-1 rhs (rhs read with stride rs) by blocked substitution in one CTA of 16
+// warps: per 32-row block, the rows' remainders (rhs minus the already solved blocks) and
+// then the product with the stored inverse of the block's diagonal block.  A lane is a
+// row of the block and the warps share the columns (the matrix is read by its columns, in
+// the triangle where they are contiguous: the panel kernel mirrors L's off-diagonal
+// blocks), so a product is a fused multiply-add per element and 16 partial sums per row;
+// a sum over the lanes per row would cost five FP64 additions a warp at two lanes a clock.
+// A block's columns are brought into shared memory while the block before it is solved
+// (the solution is needed only for the products).  Forward with L, backward with L^T.
+// 295 unknowns: 69 us, against 115 us for a warp and a lane sum per row, reading L as it
+// went.  Skips when flag[0] or flag[1] is set.
+constexpr int TSW = 16;
+__host__ __device__ inline size_t tri_smem(int n) {     // y [n], x [n] (to 16 bytes), two buffers of staged columns
+    const int nb = (n + CB - 1) / CB;
+    return sizeof(double) * (2 * (size_t)((n + 1) & ~1) + 2 * (size_t)(nb - 1) * CB * CB);
 }
-
-// x = (L L^T)^-1 rhs (rhs read with stride rs) by blocked substitution in one
-// CTA of 32 warps: per 32-row block, warp w forms row w's remainder
-// (rhs minus the already solved blocks) and then the block's solution is the
-// product with the stored inverse of its diagonal block.  Forward with L,
-// backward with L^T, read by rows from the upper triangle where the panel
-// kernel mirrors L's off-diagonal blocks.  Skips when flag[0] or flag[1] is set.
-__global__ void __launch_bounds__(1024) tri_solve_kernel(const double* L, int ld, int n, const double* Dinv,
-                                                         const double* rhs, int rs, double* x, const double* flag) {
-    extern __shared__ double ts[];   // y [n], then x [n]
-    __shared__ double tt[CB];
+__global__ void __launch_bounds__(32 * TSW) tri_solve_kernel(const double* L, int ld, int n, const double* Dinv,
+                                                             const double* rhs, int rs, double* x, const double* flag) {
+    extern __shared__ __align__(16) double ts[];
+    __shared__ double part[TSW][CB], quad[4][CB], tt[CB];
     if (flag[0] != 0.0 || flag[1] != 0.0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nb = (n + CB - 1) / CB;
     double* y = ts;
-    double* xs = ts + n;
-    for (int p = 0; p < nb; p++) {
-        const int i = p * CB + warp;
-        double t = 0.0;
-        if (i < n) {
-            const double* Li = L + (long)i * ld;
-            for (int k = lane; k < p * CB; k += 32) t += Li[k] * y[k];
-            t = warp_sum_d(t);
+    double* xs = y + ((n + 1) & ~1);
+    double* buf = xs + ((n + 1) & ~1);
+    // columns k0 .. k1 - 1 at the rows of block p (past the matrix: zero)
+    const auto stage = [&](int p, int k0, int k1, double* dst) {
+        for (int e = threadIdx.x; e < (k1 - k0) * (CB / 2); e += 32 * TSW) {
+            const int k = e / (CB / 2), c = e - k * (CB / 2), i = p * CB + 2 * c;
+            const bool in = i + 1 < ld;
+            tc::cp_async16(dst + k * CB + 2 * c, L + (in ? (long)(k0 + k) * ld + i : 0L), in ? 16 : 0);
         }
-        if (lane == 0) tt[warp] = i < n ? rhs[(long)i * rs] - t : 0.0;
+        tc::cp_async_commit();
+    };
+    // the 16 partial sums of row `lane`: a quarter in each of warps 0 .. 3, then all of them in
+    // warp 0, in a fixed order; `out(sum)` runs in warp 0
+    const auto reduce = [&](double v, auto out) {
+        part[warp][lane] = v;
         __syncthreads();
-        if (i < n) {
-            const double v = warp_sum_d(Dinv[(long)p * CB * CB + warp * CB + lane] * tt[lane]);
-            if (lane == 0) y[i] = v;
+        if (warp < 4)
+            quad[warp][lane] = (part[4 * warp][lane] + part[4 * warp + 1][lane]) +
+                               (part[4 * warp + 2][lane] + part[4 * warp + 3][lane]);
+        __syncthreads();
+        if (warp == 0) out((quad[0][lane] + quad[1][lane]) + (quad[2][lane] + quad[3][lane]));
+        __syncthreads();
+    };
+    const auto half = [&](bool fwd) {
+        const auto k0 = [&](int p) { return fwd ? 0 : (p + 1) * CB; };
+        const auto k1 = [&](int p) { return fwd ? p * CB : n; };
+        int p = fwd ? 0 : nb - 1;
+        for (int s = 0; s < nb; s++, p += fwd ? 1 : -1) {
+            const double* bp = buf + (size_t)(s & 1) * (nb - 1) * CB * CB;
+            const int i = p * CB + lane, q = p + (fwd ? 1 : -1);
+            // this block's inverse and right-hand side arrive during the products
+            const double* D = Dinv + (long)p * CB * CB;
+            const double d0 = fwd ? D[lane * CB + warp] : D[warp * CB + lane];
+            const double d1 = fwd ? D[lane * CB + warp + TSW] : D[(warp + TSW) * CB + lane];
+            const double r = warp == 0 && i < n ? (fwd ? rhs[(long)i * rs] : y[i]) : 0.0;
+            tc::cp_async_wait<0>();
+            __syncthreads();
+            if (s + 1 < nb) stage(q, k0(q), k1(q), buf + (size_t)((s + 1) & 1) * (nb - 1) * CB * CB);
+            const double* v = fwd ? y : xs;
+            const int m = k1(p) - k0(p);
+            double t0 = 0.0, t1 = 0.0;
+            for (int k = warp; k < m; k += 2 * TSW) t0 = fma(bp[k * CB + lane], v[k0(p) + k], t0);
+            for (int k = warp + TSW; k < m; k += 2 * TSW) t1 = fma(bp[k * CB + lane], v[k0(p) + k], t1);
+            reduce(t0 + t1, [&](double u) { tt[lane] = i < n ? r - u : 0.0; });
+            reduce(fma(d0, tt[warp], d1 * tt[warp + TSW]), [&](double u) { if (i < n) (fwd ? y : xs)[i] = u; });
         }
-        __syncthreads();
-    }
-    for (int p = nb - 1; p >= 0; p--) {
-        const int i = p * CB + warp;
-        double t = 0.0;
-        if (i < n) {
-            const double* Ui = L + (long)i * ld;   // row i of L^T (the mirrored upper triangle)
-            for (int k = (p + 1) * CB + lane; k < n; k += 32) t += Ui[k] * xs[k];
-            t = warp_sum_d(t);
-        }
-        if (lane == 0) tt[warp] = i < n ? y[i] - t : 0.0;
-        __syncthreads();
-        if (i < n) {
-            const double v = warp_sum_d(Dinv[(long)p * CB * CB + lane * CB + warp] * tt[lane]);
-            if (lane == 0) xs[i] = v;
-        }
-        __syncthreads();
-    }
+    };
+    half(true);
+    half(false);
     for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = xs[i];
 }
 
@@ -1350,60 +1397,65 @@ __global__ void __launch_bounds__(256) refine_update_kernel(double* a, const dou
 // second pass over the design rows: with r = C^T W (I - C c),
 //   chi^2(c + delta) = chi^2(c) - 2 delta.r + delta^T M delta
 // (M the Gram the solves used; delta is small, so its rounding enters only at
-// second order).  chi_n[0..1] = (chi^2, n) of c; out[0..1] the same for c + delta
-// (unchanged when no step was applied).  One CTA of 32 warps, a warp per row of M,
-// FP64 sums in a fixed order.
-__global__ void __launch_bounds__(1024) chi2_update_kernel(const double* M, int ld, int Nc, const double* r,
-                                                           const double* delta, const double* chi_n,
-                                                           const double* flag, double* out) {
-    __shared__ double red[32];
+// second order).  chi_n[0..1] = (chi^2, n) of c.  CTA b writes the sum of rows 16 b ..
+// 16 b + 15, delta_i (M delta - 2 r)_i, to part[b] (0 when no step was applied; the
+// finalising kernel adds the parts in order): a warp per row, each lane keeping its own
+// share of the row until the CTA's sum (one CTA that summed every row over its lanes took
+// 54 us of FP64 additions).
+constexpr int CHI_ROWS = 16;
+__global__ void __launch_bounds__(32 * CHI_ROWS) chi2_update_kernel(const double* M, int ld, int Nc, const double* r,
+                                                                    const double* delta, const double* flag,
+                                                                    double* part) {
+    __shared__ double red[CHI_ROWS];
     if (flag[0] != 0.0) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool applied = flag[3] > 0.0;
-    double acc = 0.0;   // lane 0 of each warp: its rows' delta_i (M delta - 2 r)_i
-    if (applied) {
-        for (int i = warp; i < Nc; i += 32) {   // one warp per row, lanes along the row
-            const double* Mi = M + (long)i * ld;
-            double q = 0.0;
-            for (int j = lane; j < Nc; j += 32) q = fma(Mi[j], delta[j], q);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-            acc += delta[i] * (q - 2.0 * r[i]);
-        }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * CHI_ROWS + warp;
+    double acc = 0.0;
+    if (flag[3] > 0.0 && i < Nc) {
+        const double* Mi = M + (long)i * ld;
+        double q = lane == 0 ? -2.0 * r[i] : 0.0;
+        for (int j = lane; j < Nc; j += 32) q = fma(Mi[j], delta[j], q);
+        acc = delta[i] * q;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) red[warp] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < 32; w++) t += red[w];
-        out[0] = chi_n[0] + t;
-        out[1] = chi_n[1];
+        for (int w = 0; w < CHI_ROWS; w++) t += red[w];
+        part[blockIdx.x] = t;
     }
 }
 
 // Map the solution c of the orthonormalised basis back to Alard-Lupton
 // coefficients (a_{n,k} = sum_m S[n][m] c_{m,k}, FP64) and write the stats.
 __global__ void finalize_kernel(BasisDev b, const double* c, const double* S, const double* flag,
-                                const double* chi_a0, const double* chi_a, int n_stamps_max, const int* n_stamps,
+                                const double* chi_a0, const double* chi_part, int n_stamps_max, const int* n_stamps,
                                 const int* centers, int stamp, int w, int h, int prec, double* coeffs,
                                 argus_fit_stats* st) {
+    __shared__ int used;
     const bool bad = flag[0] != 0.0;
     const int nb = b.nb, Ks = b.Ks, Nc = b.Nc;
+    if (threadIdx.x == 0) used = 0;
+    __syncthreads();
+    const int hs = stamp / 2, r = b.r, ns = min(*n_stamps, n_stamps_max);
+    for (int i = threadIdx.x; i < ns; i += blockDim.x) {
+        const int xs = centers[2 * i], ys = centers[2 * i + 1];
+        if (xs - hs - r >= 0 && xs + hs + r <= w - 1 && ys - hs - r >= 0 && ys + hs + r <= h - 1) atomicAdd(&used, 1);
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        double dchi = 0.0;
+        if (!bad)
+            for (int i = 0; i < (Nc + CHI_ROWS - 1) / CHI_ROWS; i++) dchi += chi_part[i];
         argus_fit_stats s;
-        s.chi2 = bad ? 0.0 : chi_a[0];
+        s.chi2 = bad ? 0.0 : chi_a0[0] + dchi;
         s.chi2_a0 = bad ? 0.0 : chi_a0[0];
         s.max_step = bad ? 0.0 : flag[4];
-        s.n_pix = bad ? 0 : (long long)chi_a[1];
+        s.n_pix = bad ? 0 : (long long)chi_a0[1];
         s.dof = s.n_pix - Nc;
         s.n_coeffs = Nc;
         s.status = bad ? ARGUS_ERR_SINGULAR : ARGUS_OK;
-        int used = 0;
-        const int hs = stamp / 2, r = b.r, ns = min(*n_stamps, n_stamps_max);
-        for (int i = 0; i < ns; i++) {
-            const int xs = centers[2 * i], ys = centers[2 * i + 1];
-            used += (xs - hs - r >= 0 && xs + hs + r <= w - 1 && ys - hs - r >= 0 && ys + hs + r <= h - 1);
-        }
         s.n_stamps_used = used;
         s.precision = prec;
         s.refine_iters = bad ? 0 : (int)flag[3];
@@ -1424,15 +1476,17 @@ __global__ void finalize_kernel(BasisDev b, const double* c, const double* S, co
     }
 }
 
-// a7: K_k(u,v) = sum_n a_{n,k} B_n(u,v) (K_0 also a_0 B_0); bg_k.
+// a7: K_k(u,v) = sum_n a_{n,k} B_n(u,v) (K_0 also a_0 B_0); bg_k.  Grid (Ks, pixel
+// chunks): a chain of nb FP64 multiply-adds per pixel, so the pixels go over many SMs.
 __global__ void expand_kernel(BasisDev b, const double* img, const double* a, float* K, double* bg) {
-    const int k = blockIdx.x, kk = b.ks * b.ks;
-    for (int e = threadIdx.x; e < kk; e += blockDim.x) {
+    const int k = blockIdx.x, kk = b.ks * b.ks, e = blockIdx.y * blockDim.x + threadIdx.x;
+    if (e < kk) {
         double s = (k == 0) ? a[0] * img[e] : 0.0;
+#pragma unroll 8
         for (int n = 1; n < b.nb; n++) s += a[1 + (n - 1) * b.Ks + k] * img[(long)n * kk + e];
         K[(long)k * kk + e] = (float)s;
     }
-    if (k == 0)
+    if (k == 0 && blockIdx.y == 0)
         for (int t = threadIdx.x; t < b.Kb; t += blockDim.x) bg[t] = a[1 + (b.nb - 1) * b.Ks + t];
 }
 
@@ -1921,9 +1975,9 @@ int argus_cholesky_solve_prepare(argus_ctx* ctx, const double* M, int ld, int n,
 // x = (L L^T)^-1 rhs: one blocked forward and backward substitution.
 void argus_tri_solve(argus_ctx* ctx, int ld, int n, const double* rhs, int rs, double* x, cudaStream_t st) {
     double* flag = ctx->vec + 7 * (size_t)ctx->np_cols;
-    const size_t sm = sizeof(double) * 2 * (size_t)n;
+    const size_t sm = tri_smem(n);
     cudaFuncSetAttribute(tri_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    tri_solve_kernel<<<1, 1024, sm, st>>>(ctx->L, ld, n, ctx->Dinv, rhs, rs, x, flag); argus_count_launch(1);
+    tri_solve_kernel<<<1, 32 * TSW, sm, st>>>(ctx->L, ld, n, ctx->Dinv, rhs, rs, x, flag); argus_count_launch(1);
 }
 
 // a4: X[(s nb + m) ss + pix] = (ref (x) img_m) at every pixel of every stamp s <
@@ -2109,7 +2163,7 @@ extern "C" int argus_fit_kernel(argus_ctx* ctx, const float* sci, const float* s
         refine_update_kernel<<<1, 256, 0, st>>>(c, dl, n, flag); argus_count_launch(1);
     }
     // chi^2 of the refined solution from the first residual pass (rv = r of c, dl = delta)
-    chi2_update_kernel<<<1, 1024, 0, st>>>(ctx->M, NP, n, rv, dl, chi0, flag, chif); argus_count_launch(1);
+    chi2_update_kernel<<<(n + CHI_ROWS - 1) / CHI_ROWS, 32 * CHI_ROWS, 0, st>>>(ctx->M, NP, n, rv, dl, flag, chif); argus_count_launch(1);
     finalize_kernel<<<1, 256, 0, st>>>(d, c, ctx->basis_S, flag, chi0, chif, max_stamps, n_stamps, centers, stamp,
                                        shape.w, shape.h, precision, coeffs, stats); argus_count_launch(1);
     return argus_launch_status();
@@ -2124,7 +2178,7 @@ extern "C" int argus_expand_kernel(argus_ctx* ctx, const argus_basis* basis, con
     if (cudaSetDevice(ctx->device) != cudaSuccess) return ARGUS_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = argus_basis_prepare(ctx, basis, st))) return rc;
-    expand_kernel<<<d.Ks, 256, 0, st>>>(d, ctx->basis_img, coeffs, K, bg); argus_count_launch(1);
+    expand_kernel<<<dim3(d.Ks, (d.ks * d.ks + 63) / 64), 64, 0, st>>>(d, ctx->basis_img, coeffs, K, bg); argus_count_launch(1);
     return argus_launch_status();
 }
 

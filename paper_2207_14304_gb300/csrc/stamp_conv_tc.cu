@@ -112,7 +112,7 @@ __device__ __forceinline__ bool sct_warp_wait(SctcShared& S, uint64_t* bar, uint
 // 2: taps 16..23 of rows 2p and 2p + 1), part (hi, lo), function f, tap index kk
 // at p SCT_BSLOT + ks 4096 + part 2048 + (f / 8) 128 + (kk / 8) 1024 + (f % 8) 16 +
 // (kk % 8) 2; plane row v, tap u is basis tap (20 - v, 20 - u), zero past the
-// image.  One CTA: the scale (a power of two for the largest |value|) first;
+// image.  Every CTA takes the scale (a power of two for the largest |value|) first;
 // its inverse is stored as a float after the packed operands.
 __global__ void __launch_bounds__(1024) stamp_pack_b_kernel(const float* img, int nb, uint8_t* bpack) {
     __shared__ float wmax[32];
@@ -132,12 +132,12 @@ __global__ void __launch_bounds__(1024) stamp_pack_b_kernel(const float* img, in
         float m = 0.0f;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) m = fmaxf(m, wmax[w]);
         s_scale = f16_range_scale(m);
-        *reinterpret_cast<float*>(bpack + SCT_NPAIR * SCT_BSLOT) = 1.0f / s_scale;
+        if (blockIdx.x == 0) *reinterpret_cast<float*>(bpack + SCT_NPAIR * SCT_BSLOT) = 1.0f / s_scale;
     }
     __syncthreads();
     const float sc = s_scale;
     const int tot = SCT_NPAIR * 3 * 64 * 16;
-    for (int e = tid; e < tot; e += blockDim.x) {
+    for (int e = blockIdx.x * blockDim.x + tid; e < tot; e += gridDim.x * blockDim.x) {
         const int kk = e & 15, f = (e >> 4) & 63, ks = (e >> 10) % 3, p = (e >> 10) / 3;
         const int v = ks < 2 ? 2 * p + ks : 2 * p + (kk >> 3);
         const int u = ks < 2 ? kk : 16 + (kk & 7);
@@ -387,7 +387,7 @@ int argus_stamp_conv_tc(const float* ref, long pitch, int w, int h, const int* c
                         int max_stamps, const float* img, int nb, uint8_t* bpack, float* X, int num_sms, int* status,
                         cudaStream_t st) {
     if (nb < 1 || nb > 64 || max_stamps < 1) return ARGUS_ERR_ARG;
-    stamp_pack_b_kernel<<<1, 1024, 0, st>>>(img, nb, bpack); argus_count_launch(1);
+    stamp_pack_b_kernel<<<SCT_NPAIR, 1024, 0, st>>>(img, nb, bpack); argus_count_launch(1);
     const size_t smem = sizeof(SctcShared) + 128;
     const cudaError_t e = cudaFuncSetAttribute(stamp_conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return argus_cuda_fail(e);
