@@ -60,7 +60,7 @@
 // mbarrier rounds lengthened a critical path the epilogue only just keeps
 // (measured 1.02-1.11 against 0.85 ms per full frame, whatever the waits and
 // fences were).  Persistent CTAs walk the strips of 128 columns x a band of TCY
-// output rows (256 for the difference image, 128 for the variance), streaming
+// output rows (chosen per call, see band_rows), streaming
 // each band's TCY + 2r source rows in blocks of G (the difference image: G = 4,
 // one CTA of 320 threads per SM; the variance: G = 8, two CTAs per SM).
 // Warps 0-3: epilogue, one output column per thread and TMEM lane; warp w
@@ -83,10 +83,38 @@ namespace {
 using namespace argus_sub;
 
 constexpr int TCX = 128;                     // output columns per CTA (MMA M)
-// output rows per band: the variance's strip is one 128 x 128 variance tile; the
-// difference image takes 256-row bands (half the halo rows of 128-row bands)
+// Output rows per band, chosen per call.  A CTA is held for the longest share of bands
+// any SM gets, ceil(bands / CTAs) of them, and a band costs its rows, the 2r halo rows and
+// a start (BAND_COST rows' worth): small frames want bands enough for every SM, large ones
+// few halo rows and a full last round.  A band starts on a block boundary of the frame
+// (rows a multiple of G), so every output row's sums run over the same blocks of source
+// rows whatever the band.  The variance's bands divide a 128 x 128 variance tile.  With
+// bands of 256 and 128 rows a 9576 x 6388 difference image took 13 rounds of 276 rows
+// where 3,152 are each SM's share; 3001 x 2047 pixels were 192 bands on 152 SMs, 1024 x
+// 1024 were 32.  Measured against those bands: the difference kernel 860 -> 778 us at
+// 9576 x 6388, 67 -> 21 us at 1024 x 1024 (its variance 25 -> 16); difference and variance
+// of 3001 x 2047 together 208 -> 168 us.
+constexpr int BAND_MIN = 16, BAND_COST = 16;
 template <bool VAR>
-__host__ __device__ constexpr int tcy() { return VAR ? VAR_TILE : 256; }
+inline int band_rows(int w, int h, int r, int ctas) {
+    const int gx = (w + TCX - 1) / TCX;
+    int best = VAR ? VAR_TILE : 256;
+    long cost = -1;
+    const auto consider = [&](int rows) {
+        const long items = (long)gx * ((h + rows - 1) / rows), c = (items + ctas - 1) / ctas * (rows + 2 * r + BAND_COST);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = rows;
+        }
+    };
+    if (VAR) {
+        for (int rows = VAR_TILE; rows >= BAND_MIN; rows /= 2) consider(rows);
+    } else {
+        const int most = (h + BAND_MIN - 1) / BAND_MIN;
+        for (int n = most < 256 ? most : 256; n >= 1; n--) consider(((h + n - 1) / n + 3) / 4 * 4);
+    }
+    return best;
+}
 // source rows per block: the variance's narrow MMAs leave the tensor pipe idle, so its
 // blocks are larger (fewer barrier rounds per row); the difference image's MMA width
 // grows with G (N = (KS - 1 + G) NK), so it keeps four
@@ -218,7 +246,7 @@ __device__ __noinline__ void drain_copies(uint64_t* bars, int nsl, int q0, int b
 template <int KS, int NK, bool VAR>
 __global__ void __launch_bounds__(TC_THREADS, VAR ? 2 : 1)
     subtract_tc_kernel(SubArgs a, const __grid_constant__ CUtensorMap tm_src, const __grid_constant__ CUtensorMap tm_obs,
-                       const __grid_constant__ CUtensorMap tm_flg, int* status) {
+                       const __grid_constant__ CUtensorMap tm_flg, int TCY, int* status) {
     using Sh = TcShared<KS, NK, VAR>;
     constexpr int G = Sh::G;
     using C = TcCfg<KS, NK, G>;
@@ -228,8 +256,8 @@ __global__ void __launch_bounds__(TC_THREADS, VAR ? 2 : 1)
     static_assert(NSL > LA, "a slot is re-armed only after its last reads");
     constexpr int P = VAR ? 1 : 3;               // products per K slice: hi*hi (+ hi*lo + lo*hi)
     static_assert(!VAR || NK == 1, "the variance convolution has one term");
-    constexpr int TCY = tcy<VAR>();
-    static_assert(!VAR || (TCX == VAR_TILE && TCY == VAR_TILE), "one variance tile per strip");
+    static_assert(!VAR || TCX == VAR_TILE, "one variance tile per strip");
+    static_assert(BAND_MIN % G == 0 && VAR_TILE % BAND_MIN == 0, "bands start on block boundaries");
     float* outp = VAR ? a.diff_var : a.diff;
     constexpr int R = (KS - 1) / 2;
     constexpr int SOFF = (4 - R % 4) % 4;        // wsrc[.][SOFF + c] = R(x0 - R + c); x0 - R - SOFF is a multiple of 4
@@ -529,7 +557,7 @@ __global__ void __launch_bounds__(TC_THREADS, VAR ? 2 : 1)
                     issued = gb;
                 }
                 // this issuer's MMAs of the strip done: its Z set may be rewritten (both
-                // issuers have blocks in every strip: a strip has at least 3)
+                // issuers have blocks in every strip: a strip has at least 2)
                 if (VAR && run) tc::commit(&S.bfree[bs]);
             }
             // every issued MMA must land before TMEM is released (a commit
@@ -767,14 +795,15 @@ int launch_tc(const SubArgs& a, int* status, cudaStream_t st) {
         if (!rc) rc = argus_tmap_2d(&tflg, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.flags, a.w, a.h, a.pitch, 32, Sh::G);
         if (rc) return rc;
     }
-    const int nitems = ((a.w + TCX - 1) / TCX) * ((a.h + tcy<VAR>() - 1) / tcy<VAR>());
     // persistent: the CTAs walk the strips (the set-up once per CTA)
-    int grid = nitems, dev = 0, sms = 0;
+    int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return argus_cuda_fail(e);
-    if (grid > (VAR ? 2 : 1) * sms) grid = (VAR ? 2 : 1) * sms;
-    subtract_tc_kernel<KS, NK, VAR><<<grid, TC_THREADS, smem, st>>>(a, tsrc, tobs, tflg, status); argus_count_launch(1);
+    const int ctas = (VAR ? 2 : 1) * sms, rows = band_rows<VAR>(a.w, a.h, (KS - 1) / 2, ctas);
+    const int nitems = ((a.w + TCX - 1) / TCX) * ((a.h + rows - 1) / rows);
+    const int grid = nitems < ctas ? nitems : ctas;
+    subtract_tc_kernel<KS, NK, VAR><<<grid, TC_THREADS, smem, st>>>(a, tsrc, tobs, tflg, rows, status); argus_count_launch(1);
     return argus_launch_status();
 }
 

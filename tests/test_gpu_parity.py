@@ -566,3 +566,40 @@ def test_coadd_shift_forms(ora, nf, w, h, shifts):
         assert_rel(vg[safe], va[safe], np.maximum(va[safe], 1e-6), 2e-6, "var")
     finally:
         B.argus_destroy(ctx)
+
+
+@pytest.mark.parametrize("w,h,ks,deg", [(300, 700, 21, 2), (1100, 333, 11, 1), (129, 2200, 21, 0), (2600, 150, 11, 0)])
+def test_subtract_does_not_depend_on_bands(ora, w, h, ks, deg):
+    """The difference and its variance of a frame equal, bit for bit away from the cut, those of
+    the frame without its first 128 rows (other bands of output rows, the same frame coordinates),
+    and the difference agrees with the oracle at the unit bar."""
+    rng = np.random.default_rng(w + h)
+    nk, r, top = (deg + 1) * (deg + 2) // 2, ks // 2, 128
+    I, R = (rng.normal(300, 20, (h, w)).astype(np.float32) for _ in range(2))
+    V, Vr = (rng.uniform(200, 400, (h, w)).astype(np.float32) for _ in range(2))
+    fl = (rng.random((h, w)) < 0.01).astype(np.uint8)
+    K = (rng.normal(0, 1, (nk, ks, ks)) / ks ** 2).astype(np.float32)
+    bg = rng.normal(0, 2, nk)
+    pitch = pitch_for(w)
+    dI, dV, dR, dVr, dfl = (dev_pitched(a) for a in (I, V, R, Vr, fl))
+    dK, dbg = torch.from_numpy(K.reshape(-1)).cuda(), torch.from_numpy(bg).cuda()
+    ctx = ctx_for(w, h)
+    try:
+        out = []
+        for y0 in (0, top):
+            D, VD = (torch.zeros((h - y0, pitch), device="cuda") for _ in range(2))
+            B.argus_subtract(ctx, dI[y0:], dV[y0:], dR[y0:], dVr[y0:], dfl[y0:], B.argus_shape(w, h - y0, pitch), w, h, 0,
+                             y0, ks, deg, dK, deg, dbg, D, VD)
+            torch.cuda.synchronize()
+            assert B.argus_sync_status(ctx) == 0
+            out.append((D, VD))
+        for a, b in zip(*out):
+            if h - top > 2 * r:
+                assert torch.equal(a[top + r:], b[r:])
+        xy = np.stack([rng.integers(0, w, 400), rng.integers(0, h, 400)], 1).astype(np.int32)
+        Do, _ = ora.subtract_at(xy, I, V, R, Vr, fl, K.astype(np.float64), bg, sdeg=deg, bgdeg=deg)
+        Dg = host(out[0][0], w)[xy[:, 1], xy[:, 0]]
+        scale = np.maximum(np.abs(I[xy[:, 1], xy[:, 0]]), np.maximum(np.abs(I[xy[:, 1], xy[:, 0]] - Do), 1.0))
+        assert_rel(Dg, Do, scale, 1e-4, "D")
+    finally:
+        B.argus_destroy(ctx)
