@@ -323,48 +323,77 @@ __device__ __forceinline__ void col_code(const GramArgs& g, int j, int& n, int& 
 // column and all 21 rows of its four functions (84 accumulators).  Per tap
 // column the 41 window values of the thread's column are loaded once, then
 // KS taps x 21 rows x 4 functions of FMAs: ~93 % of the issued instructions.
-constexpr int SC_ST = 21, SC_NS = 3;
+// Where the stamps make fewer CTAs than SMs the work is split further (sc_split): the
+// two lane-halves over grid.y, the function groups over grid.z.  Neither changes an
+// output's sum.
+constexpr int SC_ST = 21, SC_NS = 3, SC_GROUPS = 13;
+
+struct ScSplit {
+    int halves, parts, groups;                     // grid.y, grid.z, function groups (warps) per CTA
+};
+
+// A CTA of all 13 groups keeps 3 or 4 warps on each scheduler of its SM, for both halves;
+// four groups leave one on each, below which a split adds only staging.  64 stamps of 49
+// functions: 79 -> 30 us.
+inline ScSplit sc_split(int nblk, int nb, int sms) {
+    const int groups = (nb + 3) / 4, most = (groups + 3) / 4;
+    ScSplit p{1, 1, SC_GROUPS};
+    if (nblk < sms) {
+        p.halves = 2;
+        p.parts = (sms + 2 * nblk - 1) / (2 * nblk);
+        if (p.parts > most) p.parts = most;
+        p.groups = (groups + p.parts - 1) / p.parts;
+    }
+    return p;
+}
 
 template <int KS>
-__global__ void __launch_bounds__(416, 1) stamp_conv_fast_kernel(BasisDev b, const float* ref, long pitch, int w,
+__global__ void __launch_bounds__(32 * SC_GROUPS, 1) stamp_conv_fast_kernel(BasisDev b, const float* ref, long pitch, int w,
                                                                  int h, const int* centers, const int* n_stamps,
                                                                  const float* imgf, float* X) {
     constexpr int R = KS / 2, WW = SC_ST + 2 * R, SS = SC_ST * SC_ST, KK = KS * KS;
     extern __shared__ __align__(16) float scs[];
     float* Rw = scs;                               // [SC_NS][WW][WW]
-    float* Bs = Rw + SC_NS * WW * WW;              // [nb][KK]
+    float* Bs = Rw + SC_NS * WW * WW;              // [functions of the CTA][KK]
     __shared__ int valid_s[SC_NS];
-    const int nb = b.nb;
+    __shared__ const float* win_s[SC_NS];
+    const int nb = b.nb, gpc = blockDim.x / 32, f0 = 4 * gpc * blockIdx.z;
+    const int nf = min(4 * gpc, nb - f0);          // functions f0 .. f0 + nf - 1
+    if (nf <= 0) return;
     const int ns = *n_stamps;
     const int s0 = blockIdx.x * SC_NS;
     if (s0 >= ns) return;
     if (threadIdx.x < SC_NS) {
         const int s = s0 + threadIdx.x, hs = SC_ST / 2;
         int v = 0;
+        const float* win = ref;
         if (s < ns) {
             const int xs = centers[2 * s], ys = centers[2 * s + 1];
             v = xs - hs - R >= 0 && xs + hs + R <= w - 1 && ys - hs - R >= 0 && ys + hs + R <= h - 1;
+            if (v) win = ref + (long)(ys - hs - R) * pitch + xs - hs - R;
         }
         valid_s[threadIdx.x] = v;
+        win_s[threadIdx.x] = win;
     }
     __syncthreads();
+    // a stamp that is not taken reads the frame's first pixel for every window value, so
+    // that the loads carry no branch and go out in batches
+#pragma unroll 8
     for (int e = threadIdx.x; e < SC_NS * WW * WW; e += blockDim.x) {
         const int t = e / (WW * WW), rem = e - t * WW * WW;
         const int wj = rem / WW, wi = rem - wj * WW;
-        float v = 0.0f;
-        if (valid_s[t]) {
-            const int s = s0 + t;
-            const int wx0 = centers[2 * s] - SC_ST / 2 - R, wy0 = centers[2 * s + 1] - SC_ST / 2 - R;
-            v = __ldg(ref + (long)(wy0 + wj) * pitch + wx0 + wi);
-        }
-        Rw[e] = v;
+        const int ok = valid_s[t];
+        const float v = __ldg(win_s[t] + (ok ? (long)wj * pitch + wi : 0));
+        Rw[e] = ok ? v : 0.0f;
     }
-    for (int e = threadIdx.x; e < nb * KK; e += blockDim.x) Bs[e] = __ldg(imgf + e);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < nf * KK; e += blockDim.x) Bs[e] = __ldg(imgf + f0 * KK + e);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = warp;                           // function group
-    if (4 * g >= nb) return;
-    for (int half = 0; half < 2; half++) {
+    const int g = warp;                           // function group of the CTA
+    if (4 * g >= nf) return;
+    const int half1 = gridDim.y == 2 ? blockIdx.y + 1 : 2;
+    for (int half = gridDim.y == 2 ? blockIdx.y : 0; half < half1; half++) {
         const int c = half * 32 + lane;           // column of the 63-wide strip
         const bool live = c < SC_NS * SC_ST;
         const int t = live ? c / SC_ST : 0, i = live ? c - t * SC_ST : 0;
@@ -376,7 +405,7 @@ __global__ void __launch_bounds__(416, 1) stamp_conv_fast_kernel(BasisDev b, con
             for (int q = 0; q < 4; q++) acc[j][q] = 0.0f;
         const float* bf[4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) bf[q] = Bs + min(4 * g + q, nb - 1) * KK;
+        for (int q = 0; q < 4; q++) bf[q] = Bs + min(4 * g + q, nf - 1) * KK;
         // tap (iu, iv): R(x - iu + R, y - iv + R) = Rw[j + 2R - iv][i + 2R - iu]
 #pragma unroll 1
         for (int iu = 0; iu < KS; iu++) {
@@ -395,11 +424,11 @@ __global__ void __launch_bounds__(416, 1) stamp_conv_fast_kernel(BasisDev b, con
             }
         }
         if (live && s0 + t < ns) {
-            float* Xs = X + (long)(s0 + t) * nb * SS;
+            float* Xs = X + ((long)(s0 + t) * nb + f0) * SS;
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const int m = 4 * g + q;
-                if (m < nb)
+                if (m < nf)
 #pragma unroll
                     for (int j = 0; j < SC_ST; j++) Xs[(long)m * SS + j * SC_ST + i] = valid_s[t] ? acc[j][q] : 0.0f;
             }
@@ -1997,12 +2026,12 @@ static int stamp_basis_conv(argus_ctx* ctx, const float* ref, const argus_shape&
     d.r = (ks - 1) / 2;
     d.nb = nb;
     const int WW = stamp + 2 * d.r, kk = ks * ks;
-    if (stamp == SC_ST && ks == 11 && nb <= 52) {
-        // 13 warps x 4 functions cover up to 52 basis functions
-        const size_t fsm = sizeof(float) * ((size_t)SC_NS * WW * WW + (size_t)nb * kk);
+    if (stamp == SC_ST && ks == 11 && nb <= 4 * SC_GROUPS) {
         const int nblk = (max_stamps + SC_NS - 1) / SC_NS;
+        const ScSplit sp = sc_split(nblk, nb, ctx->num_sms);
+        const size_t fsm = sizeof(float) * ((size_t)SC_NS * WW * WW + (size_t)(4 * sp.groups < nb ? 4 * sp.groups : nb) * kk);
         cudaFuncSetAttribute(stamp_conv_fast_kernel<11>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
-        stamp_conv_fast_kernel<11><<<nblk, 416, fsm, st>>>(d, ref, shape.pitch, shape.w, shape.h, centers,
+        stamp_conv_fast_kernel<11><<<dim3(nblk, sp.halves, sp.parts), 32 * sp.groups, fsm, st>>>(d, ref, shape.pitch, shape.w, shape.h, centers,
                                                            n_stamps, img, X); argus_count_launch(1);
         return argus_launch_status();
     }

@@ -92,3 +92,28 @@ def test_stamp_basis_parity(ora, case, w, h, stamp, ks, nb, n, max_stamps):
     i = np.unravel_index(int(np.argmax(err)), err.shape)
     print(f"\n[stamp basis: {case}] worst |X - X_oracle| / S = {err[i]:.2e} at {i}")
     assert err[i] <= XTOL, f"{case}: {err[i]:.3e} at {i}: gpu {Xg[i]!r} oracle {Xo[i]!r}"
+
+
+@pytest.mark.parametrize("nb,n", [(1, 1), (4, 3), (17, 7), (33, 100), (49, 64), (52, 301)])
+def test_stamp_basis_does_not_depend_on_the_split(nb, n):
+    """11 x 11 images: the same bits whether the stamps' launch is split over lane-halves and
+    function groups (few stamps) or not (room for far more stamps than SMs)."""
+    w, h, stamp, ks = 400, 300, 21, 11
+    R, cen = _field(w, h, seed=nb), _centres(n, w, h, stamp, ks, seed=n)
+    dimg = torch.from_numpy(np.random.default_rng(nb).standard_normal((nb, ks * ks)).astype(np.float32)).cuda()
+    dR, ns = dev_pitched(R), torch.tensor([n, 0, 0, 0], dtype=torch.int32, device="cuda")
+    out = []
+    for max_stamps in (n, 3000):
+        ctx = ctx_for(w, h, max_stamps=max_stamps)
+        try:
+            dcen = torch.zeros((max_stamps, 2), dtype=torch.int32, device="cuda")
+            dcen[:n] = torch.from_numpy(cen).cuda()
+            X = torch.full((max_stamps, nb, stamp * stamp), -7.0, dtype=torch.float32, device="cuda")
+            B.argus_stamp_basis(ctx, dR, B.argus_shape(w, h, pitch_for(w)), dcen, ns, max_stamps, stamp, dimg, nb, ks, X)
+            torch.cuda.synchronize()
+            assert B.argus_sync_status(ctx) == 0
+            out.append(X[:n].clone())
+            assert (X[n:] == -7.0).all()
+        finally:
+            B.argus_destroy(ctx)
+    assert torch.equal(out[0], out[1])
