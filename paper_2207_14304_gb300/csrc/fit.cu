@@ -1634,6 +1634,12 @@ __global__ void select_ring_kernel(const float* R, const uint8_t* flags, const u
 //  4. One warp per remaining candidate scans the rest of the isolation window
 //     in R, testing the local-maximum rule only where R exceeds iso_frac * c,
 //     then the flag window (32-bit loads), then the cell atomicMax.
+// Before all that (step 0), a tile whose cells all hold a star already lists only the
+// pixels no fainter than the least of those stars, and without one it is done after one
+// read of its own pixels: steps 2 and 3 were most of the time (barriers and shared memory),
+// and their maxima can't win there.  9576 x 6388 in 20 x 20 cells: 319 -> 170 us, of which
+// one read of R is 36; a frame whose tiles all run at once gains nothing (1024 x 1024:
+// 17 -> 19 us, the extra read).
 constexpr int SEL_TX = 128, SEL_TY = 64, SEL_QR = 3, SEL_MAX_ISO = 32, SEL_THREADS = 512;
 constexpr int SEL_LIST = SEL_TX * SEL_TY / 4;
 
@@ -1693,6 +1699,33 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {
     return d;
 }
 
+constexpr int SEL_FEW = 256;    // candidates a tile takes directly
+
+__host__ __device__ __forceinline__ int sel_cell(int x, int gx, int w) { return (int)(((long)(x + 1) * gx - 1) / w); }
+
+// Tiles are taken in an order that visits every cell early: every sx-th column of every
+// sy-th tile row, then the next residue, a cell being about sx x sy tiles.  Once a cell
+// holds a star, nearly every pixel of its other tiles is fainter.  The residues are padded
+// to equal counts, so an origin can lie outside the frame.
+struct SelOrder {
+    int sx, sy, nx, ny;
+};
+__host__ __device__ __forceinline__ SelOrder sel_order(int w, int h, int gx, int gy) {
+    const int ntx = (w + SEL_TX - 1) / SEL_TX, nty = (h + SEL_TY - 1) / SEL_TY;
+    SelOrder o;
+    o.sx = max(w / gx / SEL_TX, 1);
+    o.sy = max(h / gy / SEL_TY, 1);
+    o.nx = (ntx + o.sx - 1) / o.sx;
+    o.ny = (nty + o.sy - 1) / o.sy;
+    return o;
+}
+__device__ __forceinline__ void sel_tile(int b, int w, int h, int gx, int gy, int& x0, int& y0) {
+    const SelOrder o = sel_order(w, h, gx, gy);
+    const int q = b / (o.nx * o.ny), i = b - q * (o.nx * o.ny);
+    x0 = (i % o.nx * o.sx + q % o.sx) * SEL_TX;
+    y0 = (i / o.nx * o.sy + q / o.sx) * SEL_TY;
+}
+
 template <int QR>
 __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float* R, const uint8_t* flags, long pitch,
                                                                     int w, int h, int gx, int gy, int m,
@@ -1709,11 +1742,59 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float
     unsigned short* cand = reinterpret_cast<unsigned short*>(mvr + MWP * MH);
     unsigned short* surv = cand + SEL_LIST;
     __shared__ int n_cand, n_surv, n_fin;
-    const int ntx = (w + SEL_TX - 1) / SEL_TX;
-    const int x0 = (int)(blockIdx.x % ntx) * SEL_TX, y0 = (int)(blockIdx.x / ntx) * SEL_TY;
+    __shared__ float least;
+    int x0, y0;
+    sel_tile(blockIdx.x, w, h, gx, gy, x0, y0);
+    if (x0 >= w || y0 >= h) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = SEL_THREADS / 32;
     const int XS = x0 - iso - 1 - g.ox, YS = y0 - iso - 1;      // frame position of r[0][0]
+    const float NEG = __int_as_float(0xff800000), INF = __int_as_float(0x7f800000);
     if (tid == 0) { n_cand = 0; n_surv = 0; n_fin = 0; }
+    // 0. the least of the best values found so far in the cells under the tile: a fainter
+    //    pixel wins in none of them.  Where few pixels are as bright, they are taken as the
+    //    candidates themselves (their isolation is then tested from the first ring on), and
+    //    where none is the tile is done
+    float4 own[SEL_TX * SEL_TY / 4 / SEL_THREADS];
+    constexpr int NOWN = sizeof(own) / sizeof(own[0]);
+#pragma unroll
+    for (int k = 0; k < NOWN; k++) {
+        const int e = tid + k * SEL_THREADS, Y = min(y0 + e / (SEL_TX / 4), h - 1);
+        own[k] = __ldg(reinterpret_cast<const float4*>(R + (long)Y * pitch + min(x0 + 4 * (e % (SEL_TX / 4)), (w - 1) & ~3)));
+    }
+    if (wid == 0) {
+        const int cx0 = sel_cell(x0, gx, w), ncx = sel_cell(min(x0 + SEL_TX, w) - 1, gx, w) - cx0 + 1;
+        const int cy0 = sel_cell(y0, gy, h), ncy = sel_cell(min(y0 + SEL_TY, h) - 1, gy, h) - cy0 + 1;
+        float best = INF;
+        for (int i = lane; i < ncx * ncy; i += 32) {
+            const unsigned long long key = __ldcg(cell_key + (cy0 + i / ncx) * gx + cx0 + i % ncx);
+            const unsigned ord = (unsigned)(key >> 32);
+            best = fminf(best, key ? __uint_as_float((ord & 0x80000000u) ? ord ^ 0x80000000u : ~ord) : NEG);
+        }
+        for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        if (lane == 0) least = best;
+    }
+    __syncthreads();
+    const float lst = least;
+    const bool few = lst > NEG;                                  // every cell has a star
+    if (few) {
+#pragma unroll
+        for (int k = 0; k < NOWN; k++) {
+            if (!(fmaxf(fmaxf(own[k].x, own[k].y), fmaxf(own[k].z, own[k].w)) >= lst)) continue;
+            const int e = tid + k * SEL_THREADS, y = e / (SEL_TX / 4), x = 4 * (e % (SEL_TX / 4)), Y = y0 + y;
+            const float v[4] = {own[k].x, own[k].y, own[k].z, own[k].w};
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const int X = x0 + x + c;
+                if (v[c] >= lst && v[c] < max_peak && v[c] < INF && X - m >= 0 && X + m <= w - 1 && Y - m >= 0 && Y + m <= h - 1) {
+                    const int at = atomicAdd(&n_fin, 1);
+                    if (at < SEL_FEW) cand[at] = (unsigned short)(y * SEL_TX + x + c);
+                }
+            }
+        }
+        __syncthreads();
+        if (n_fin == 0) return;
+    }
+    const bool direct = few && n_fin <= SEL_FEW;                 // the same for the whole CTA
     // 1. stage R in 16-byte chunks; XS is a multiple of 4, so a chunk is inside or
     //    outside the frame but for the one that holds column w (partly zero-filled)
     {
@@ -1733,118 +1814,126 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float
         tc::cp_async_wait<0>();
     }
     __syncthreads();
-    // 2. masked strict local maxima over the tile + QR, four rows x four columns per item
-    //    (each row of the item is one aligned 16-byte load of r and its two neighbours),
-    //    and the candidate list
-    const float NEG = __int_as_float(0xff800000), INF = __int_as_float(0x7f800000);
-    {
-        const int cx = iso + 1 + g.ox - QR, cy = iso + 1 - QR;     // r position of mv[0][0]; cx % 4 == MOFF
-        constexpr int NSTRIP = (MH + 3) / 4, NCG = MWP / 4, N = NCG * NSTRIP;
-        for (int e = tid; e < N; e += SEL_THREADS) {
-            const int js = e / NCG, jg = e - js * NCG;
-            const int jy0 = 4 * js, jx0 = 4 * jg - MOFF;          // columns jx0 .. jx0 + 3 (cx + jx0: 16-byte aligned)
-            const float* q = r + (cy + jy0 - 1) * g.rw + (cx + jx0);
-            // v[t][k]: r at row jy0 - 1 + t, column jx0 - 1 + k
-            float v[6][6], h3[6][4];
+    if (!direct) {
+        if (tid == 0) n_fin = 0;
+        // 2. masked strict local maxima over the tile + QR, four rows x four columns per item
+        //    (each row of the item is one aligned 16-byte load of r and its two neighbours),
+        //    and the candidate list
+        {
+            const int cx = iso + 1 + g.ox - QR, cy = iso + 1 - QR;     // r position of mv[0][0]; cx % 4 == MOFF
+            constexpr int NSTRIP = (MH + 3) / 4, NCG = MWP / 4, N = NCG * NSTRIP;
+            for (int e = tid; e < N; e += SEL_THREADS) {
+                const int js = e / NCG, jg = e - js * NCG;
+                const int jy0 = 4 * js, jx0 = 4 * jg - MOFF;          // columns jx0 .. jx0 + 3 (cx + jx0: 16-byte aligned)
+                const float* q = r + (cy + jy0 - 1) * g.rw + (cx + jx0);
+                // v[t][k]: r at row jy0 - 1 + t, column jx0 - 1 + k
+                float v[6][6], h3[6][4];
 #pragma unroll
-            for (int t = 0; t < 6; t++) {
-                const float* qt = q + t * g.rw;
-                const float4 c4 = *reinterpret_cast<const float4*>(qt);
-                v[t][0] = cx + jx0 > 0 ? qt[-1] : NEG;   // r column -1 only feeds a column jx < 0 (discarded)
-                v[t][1] = c4.x; v[t][2] = c4.y; v[t][3] = c4.z; v[t][4] = c4.w;
-                v[t][5] = qt[4];
+                for (int t = 0; t < 6; t++) {
+                    const float* qt = q + t * g.rw;
+                    const float4 c4 = *reinterpret_cast<const float4*>(qt);
+                    v[t][0] = cx + jx0 > 0 ? qt[-1] : NEG;   // r column -1 only feeds a column jx < 0 (discarded)
+                    v[t][1] = c4.x; v[t][2] = c4.y; v[t][3] = c4.z; v[t][4] = c4.w;
+                    v[t][5] = qt[4];
 #pragma unroll
-                for (int c = 0; c < 4; c++) h3[t][c] = fmax_nan(fmax_nan(v[t][c], v[t][c + 1]), v[t][c + 2]);
-            }
-            int nc = 0, ev0 = 0, ev1 = 0, ev2 = 0, ev3 = 0;
-#pragma unroll
-            for (int t = 1; t <= 4; t++) {
-                const int jy = jy0 + t - 1, y = jy - QR;
-                const int Y = y0 + y;
-                float o[4];
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    const int jx = jx0 + c, x = jx - QR, X = x0 - QR + jx;
-                    const bool xin = X >= 1 && X <= w - 2;
-                    const bool xc = x >= 0 && x < SEL_TX && X - m >= 0 && X + m <= w - 1;
-                    const float cv = v[t][c + 1];
-                    const float nb = fmax_nan(fmax_nan(h3[t - 1][c], h3[t + 1][c]), fmax_nan(v[t][c], v[t][c + 2]));
-                    const bool l = jy < MH && jx >= 0 && jx < MW && xin && Y >= 1 && Y <= h - 2 && cv > nb && cv < INF;
-                    o[c] = l ? cv : NEG;
-                    // at most one strict maximum per 2 x 2 block: at most four per item
-                    if (l && xc && y >= 0 && y < SEL_TY && Y - m >= 0 && Y + m <= h - 1 && cv < max_peak) {
-                        const int ev = y * SEL_TX + x;
-                        ev3 = nc == 3 ? ev : ev3;
-                        ev2 = nc == 2 ? ev : ev2;
-                        ev1 = nc == 1 ? ev : ev1;
-                        ev0 = nc == 0 ? ev : ev0;
-                        nc++;
-                    }
+                    for (int c = 0; c < 4; c++) h3[t][c] = fmax_nan(fmax_nan(v[t][c], v[t][c + 1]), v[t][c + 2]);
                 }
-                if (jy < MH) *reinterpret_cast<float4*>(mv + jy * MWP + jx0) = make_float4(o[0], o[1], o[2], o[3]);
+                int nc = 0, ev0 = 0, ev1 = 0, ev2 = 0, ev3 = 0;
+#pragma unroll
+                for (int t = 1; t <= 4; t++) {
+                    const int jy = jy0 + t - 1, y = jy - QR;
+                    const int Y = y0 + y;
+                    float o[4];
+#pragma unroll
+                    for (int c = 0; c < 4; c++) {
+                        const int jx = jx0 + c, x = jx - QR, X = x0 - QR + jx;
+                        const bool xin = X >= 1 && X <= w - 2;
+                        const bool xc = x >= 0 && x < SEL_TX && X - m >= 0 && X + m <= w - 1;
+                        const float cv = v[t][c + 1];
+                        const float nb = fmax_nan(fmax_nan(h3[t - 1][c], h3[t + 1][c]), fmax_nan(v[t][c], v[t][c + 2]));
+                        const bool l = jy < MH && jx >= 0 && jx < MW && xin && Y >= 1 && Y <= h - 2 && cv > nb && cv < INF;
+                        o[c] = l ? cv : NEG;
+                        // at most one strict maximum per 2 x 2 block: at most four per item
+                        if (l && xc && y >= 0 && y < SEL_TY && Y - m >= 0 && Y + m <= h - 1 && cv < max_peak) {
+                            const int ev = y * SEL_TX + x;
+                            ev3 = nc == 3 ? ev : ev3;
+                            ev2 = nc == 2 ? ev : ev2;
+                            ev1 = nc == 1 ? ev : ev1;
+                            ev0 = nc == 0 ? ev : ev0;
+                            nc++;
+                        }
+                    }
+                    if (jy < MH) *reinterpret_cast<float4*>(mv + jy * MWP + jx0) = make_float4(o[0], o[1], o[2], o[3]);
+                }
+                if (nc) {
+                    const int base = atomicAdd(&n_cand, nc);
+                    cand[base] = (unsigned short)ev0;
+                    if (nc > 1) cand[base + 1] = (unsigned short)ev1;
+                    if (nc > 2) cand[base + 2] = (unsigned short)ev2;
+                    if (nc > 3) cand[base + 3] = (unsigned short)ev3;
+                }
             }
-            if (nc) {
-                const int base = atomicAdd(&n_cand, nc);
-                cand[base] = (unsigned short)ev0;
-                if (nc > 1) cand[base + 1] = (unsigned short)ev1;
-                if (nc > 2) cand[base + 2] = (unsigned short)ev2;
-                if (nc > 3) cand[base + 3] = (unsigned short)ev3;
+        }
+        __syncthreads();
+        // 3. the other maxima within QR: radius 1 holds none (the neighbours of a strict
+        //    maximum are below it, so none of them is one); radius 2 for every candidate,
+        //    radius 3 only for the survivors of radius 2 (most noise peaks meet another
+        //    maximum at radius 2), listed in between so that warps stay full
+        for (int i = tid; i < n_cand; i += SEL_THREADS) {
+            const int e = cand[i];
+            const int y = e / SEL_TX, x = e - y * SEL_TX;
+            const float* q = mv + y * MWP + x;                         // window corner (y - QR, x - QR)
+            const float c = q[QR * MWP + QR];
+            float other = NEG;
+            if (QR >= 2) {
+#pragma unroll
+                for (int dy = QR - 2; dy <= QR + 2; dy++)
+#pragma unroll
+                    for (int dx = QR - 2; dx <= QR + 2; dx++)
+                        if (dy == QR - 2 || dy == QR + 2 || dx == QR - 2 || dx == QR + 2) other = fmaxf(other, q[dy * MWP + dx]);
             }
+            if (!(other > iso_frac * c)) surv[atomicAdd(&n_surv, 1)] = (unsigned short)e;
         }
-    }
-    __syncthreads();
-    // 3. the other maxima within QR: radius 1 holds none (the neighbours of a strict
-    //    maximum are below it, so none of them is one); radius 2 for every candidate,
-    //    radius 3 only for the survivors of radius 2 (most noise peaks meet another
-    //    maximum at radius 2), listed in between so that warps stay full
-    for (int i = tid; i < n_cand; i += SEL_THREADS) {
-        const int e = cand[i];
-        const int y = e / SEL_TX, x = e - y * SEL_TX;
-        const float* q = mv + y * MWP + x;                         // window corner (y - QR, x - QR)
-        const float c = q[QR * MWP + QR];
-        float other = NEG;
-        if (QR >= 2) {
+        __syncthreads();
+        for (int i = tid; i < n_surv; i += SEL_THREADS) {
+            const int e = surv[i];
+            const int y = e / SEL_TX, x = e - y * SEL_TX;
+            const float* q = mv + y * MWP + x;
+            const float c = q[QR * MWP + QR];
+            float other = NEG;
+            if (QR >= 3) {
 #pragma unroll
-            for (int dy = QR - 2; dy <= QR + 2; dy++)
+                for (int dy = 0; dy <= 2 * QR; dy++)
 #pragma unroll
-                for (int dx = QR - 2; dx <= QR + 2; dx++)
-                    if (dy == QR - 2 || dy == QR + 2 || dx == QR - 2 || dx == QR + 2) other = fmaxf(other, q[dy * MWP + dx]);
+                    for (int dx = 0; dx <= 2 * QR; dx++)
+                        if (dy == 0 || dy == 2 * QR || dx == 0 || dx == 2 * QR) other = fmaxf(other, q[dy * MWP + dx]);
+            }
+            if (!(other > iso_frac * c)) cand[atomicAdd(&n_fin, 1)] = (unsigned short)e;
         }
-        if (!(other > iso_frac * c)) surv[atomicAdd(&n_surv, 1)] = (unsigned short)e;
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = tid; i < n_surv; i += SEL_THREADS) {
-        const int e = surv[i];
-        const int y = e / SEL_TX, x = e - y * SEL_TX;
-        const float* q = mv + y * MWP + x;
-        const float c = q[QR * MWP + QR];
-        float other = NEG;
-        if (QR >= 3) {
-#pragma unroll
-            for (int dy = 0; dy <= 2 * QR; dy++)
-#pragma unroll
-                for (int dx = 0; dx <= 2 * QR; dx++)
-                    if (dy == 0 || dy == 2 * QR || dx == 0 || dx == 2 * QR) other = fmaxf(other, q[dy * MWP + dx]);
-        }
-        if (!(other > iso_frac * c)) cand[atomicAdd(&n_fin, 1)] = (unsigned short)e;
-    }
-    __syncthreads();
     // 4. one warp per survivor: rest of the isolation window, flag window, cell key
     const int side = 2 * iso + 1, fside = 2 * m + 1;
     for (int i = wid; i < n_fin; i += nw) {
         const int e = cand[i];
         const int y = e / SEL_TX, x = e - y * SEL_TX;
         const int X = x0 + x, Y = y0 + y;
-        const float c = mv[(y + QR) * MWP + x + QR];
+        const float* qc = r + (y + iso + 1) * g.rw + (x + iso + 1 + g.ox);   // the candidate
+        const float c = *qc;
         const float thr = iso_frac * c;
         bool bad = false;
-        if (iso > QR) {
-            // rings QR + 1 .. iso, 32 taps per step, nearest first: a noise peak meets
+        if (direct) {                                      // not yet known to be a strict maximum
+            const int k = lane < 4 ? lane : lane + 1;
+            const bool nb = lane < 8 && !(c > qc[(k / 3 - 1) * g.rw + k % 3 - 1]);
+            bad = __any_sync(0xffffffffu, nb) || X < 1 || X > w - 2 || Y < 1 || Y > h - 2;
+        }
+        const int q0 = direct ? min(QR, 1) : QR;           // isolation tested up to this radius
+        if (!bad && iso > q0) {
+            // rings q0 + 1 .. iso, 32 taps per step, nearest first: a noise peak meets
             // a brighter maximum within a step or two
-            const float* qc = r + (y + iso + 1) * g.rw + (x + iso + 1 + g.ox);   // the candidate
             const char2* ring = reinterpret_cast<const char2*>(g_sel_ring.d);
             const int p1 = side * side - 1;
-            for (int pb = (2 * QR + 1) * (2 * QR + 1) - 1; pb < p1; pb += 32) {
+            for (int pb = (2 * q0 + 1) * (2 * q0 + 1) - 1; pb < p1; pb += 32) {
                 const int p = pb + lane;
                 bool b = false;
                 if (p < p1) {
@@ -1897,7 +1986,8 @@ int launch_select_tile(const float* ref, const uint8_t* flags, const argus_shape
     if (cudaFuncSetAttribute(select_tile_kernel<QR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return ARGUS_ERR_CUDA;
-    const long tiles = (long)((shape.w + SEL_TX - 1) / SEL_TX) * ((shape.h + SEL_TY - 1) / SEL_TY);
+    const SelOrder o = sel_order(shape.w, shape.h, grid_x, grid_y);
+    const long tiles = (long)o.sx * o.sy * o.nx * o.ny;
     select_tile_kernel<QR><<<(unsigned)tiles, SEL_THREADS, smem, st>>>(ref, flags, shape.pitch, shape.w, shape.h,
                                                                        grid_x, grid_y, m, max_peak, iso, iso_frac,
                                                                        keys);

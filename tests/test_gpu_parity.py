@@ -391,6 +391,37 @@ def test_select_stamps_ties_and_plateaus(ora):
         B.argus_destroy(ctx)
 
 
+@pytest.mark.parametrize("gx,gy,iso,iso_frac,max_peak", [(8, 6, 10, 0.1, 3e4), (8, 6, 0, 0.1, 3e4), (5, 7, 1, 0.3, 3e4),
+                                                         (3, 1, 2, 0.9, 2e4), (60, 60, 3, 0.1, 3e4), (1, 1, 32, 0.2, 1e5),
+                                                         (16, 11, 10, 0.1, -400.0)])
+def test_select_stamps_of_many_tiles(gx, gy, iso, iso_frac, max_peak):
+    """A frame of far more tiles than run at once, so that later tiles meet cells that hold a star:
+    the same stamps as the per-pixel kernel's, with ties, negative peaks, NaN and infinities."""
+    w, h = 4003, 2601
+    rng = np.random.default_rng(gx * gy + iso)
+    R = np.rint(rng.normal(-500, 20, (h, w))).astype(np.float32)
+    y, x = rng.integers(0, h, 4000), rng.integers(0, w, 4000)
+    R[y, x] = np.rint(rng.uniform(0, 4e4, 4000) / 500) * 500
+    for v in (np.nan, np.inf, -np.inf):
+        R[rng.random((h, w)) < 1e-5] = v
+    fl = (rng.random((h, w)) < 2e-4).astype(np.uint8)
+    dR, dfl, shape = dev_pitched(R), dev_pitched(fl), B.argus_shape(w, h, pitch_for(w))
+    ctx = ctx_for(w, h)
+    try:
+        out = []
+        for f in (lambda *a: B.argus_select_stamps(ctx, *a), B.argus_select_stamps_noalloc):
+            cen = torch.full((gx * gy, 2), -1, dtype=torch.int32, device="cuda")
+            ns = torch.zeros(4, dtype=torch.int32, device="cuda")
+            f(dR, dfl, shape, gx, gy, 21, 5, max_peak, iso, iso_frac, cen, ns)
+            torch.cuda.synchronize()
+            out.append((int(ns[0].item()), cen))
+        n = out[0][0]
+        assert n == out[1][0] and n > 0
+        assert torch.equal(out[0][1][:n], out[1][1][:n])
+    finally:
+        B.argus_destroy(ctx)
+
+
 # --------------------------------------------------------------------------- fit + expand
 def _fit_field(w, h, seed, sdeg):
     cat = synth.star_catalog(w * h // 80, w, h, seed=seed, flux_min=1e2, flux_max=1e6)
