@@ -44,7 +44,7 @@ struct argus_seg_plan {
     int fit_tc;            // the fit runs on the tensor cores (kernel sides <= 15)
     int4* d_fit_tc_items;  // (segment, x0, y0, -): tensor-core fit, 128 columns x band rows
     int n_fit_tc_items;
-    int* d_fit_tc_start;   // [fit_tc_ctas + 1] item range of each CTA, equal row pairs
+    int* d_fit_tc_start;   // [fit_tc_ctas + 1] item range of each CTA, equal shares of the work
     float* d_rscale;       // [n] per-segment scale of R for the FP16 operands
     int fit_tc_ctas;
     int2* d_sub_items;     // (segment, tile index)
@@ -493,14 +493,16 @@ extern "C" int argus_segments_plan(argus_ctx* ctx, const argus_segment* table, i
         const int nt = (side + 31) / 32;
         for (int t = 0; t < nt * nt; t++) sub_items.push_back(make_int2(i, t));
     }
-    // the tensor-core fit's CTA ranges: row pairs (its unit of work) split evenly over one CTA per SM
+    // the tensor-core fit's CTA ranges, equal shares over one CTA per SM: a row pair costs a
+    // constant (its design rows) and its fold groups of 16 columns
     int fit_tc_ctas = 0;
     if (fit_tc) {
         std::vector<long> cum(fit_tc_items.size() + 1, 0);
         for (size_t k = 0; k < fit_tc_items.size(); k++) {
             const int4 it = fit_tc_items[k];
             const int rows = std::min(band, table[it.x].side - bd.r - it.z);
-            cum[k + 1] = cum[k] + (rows + 1) / 2;
+            const int cols = std::min(128, table[it.x].side - bd.r - it.y);
+            cum[k + 1] = cum[k] + (long)((rows + 1) / 2) * (4 + (cols + 15) / 16);
         }
         fit_tc_ctas = std::max(1, std::min(ctx->num_sms, (int)fit_tc_items.size()));
         fit_tc_start.assign(fit_tc_ctas + 1, 0);

@@ -121,6 +121,13 @@ def test_segments_parity(ora, use_graph, case):
         batch.close()
 
 
+def test_segments_at_the_edges_of_strips_and_sums(ora):
+    """Interiors one pixel around the fit's strips of 128 columns, its sums of 16 columns and its
+    pairs of rows, at the bars of the batch."""
+    sides = [14 + n for n in (33, 47, 48, 49, 127, 128, 129, 130, 143, 144, 145, 159)]
+    test_segments_parity(ora, False, (640, 480, sides, 512))
+
+
 def test_segments_subtract_with_the_oracles_kernels(ora):
     """The batched subtraction alone, given the oracle's kernels and backgrounds, against
     the oracle's difference and variance at the unit-test bars (1e-4 of max(|I|,
