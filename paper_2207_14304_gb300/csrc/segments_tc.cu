@@ -41,11 +41,17 @@
 // segment's FP64 normal matrix by atomics.
 //
 // Roles (16 warps): warps 0-3 read the accumulators (thread = pixel, the TMEM
-// lane), weight them and write the design rows of the pair (256 pixels) to
-// shared memory; warps 4-6 stage the source rows (16-byte cp.async, zero past
+// lane), weight them and write the design rows of the pair, one image row (128
+// pixels) at a time, to shared memory; warps 4-6 stage the source rows (16-byte cp.async, zero past
 // the segment) and write the A operands; warp 7 issues the MMAs; warps 8-15
-// and, once the rows are written, warps 0-3 sum the Gram: two sets of 192
-// threads (the 182 blocks of a 51-column Gram), one per row of the pair.  Two
+// and warps 0-3 sum the Gram: two sets of 192 threads (the 182 blocks of a
+// 51-column Gram), one per row of the pair.  The Gram's packed FP32 arithmetic
+// bounds the kernel, so its warps must not wait for the readers: three row
+// buffers, and the readers write the next pair's first row before their own
+// share of the last pair (one buffer of two rows that all waited for: 39.6 ms
+// for the 4 x 512 segments of 64 to 512 px, 15 x 15 kernels; now 34.3).  Room
+// for the third buffer is the A ring's, which holds one pair's source rows: its
+// MMAs and the staging of the next two rows are a third of the Gram's time.  Two
 // TMEM accumulators let the MMAs of one pair run while the previous one is read.
 // Every wait is bounded; a timeout latches ARGUS_ERR_TIMEOUT and all roles stop.
 #include <cuda_fp16.h>
@@ -61,7 +67,8 @@ constexpr int FT_THREADS = FT_WARPS * 32;
 constexpr int FT_NPROD = 3;                       // producer warps (4..6)
 constexpr int FT_MMA_WARP = 7;
 constexpr int FT_GRAM_WARP = 8;                   // warps 8..15
-constexpr int FT_NA = 20;                         // A ring slots (source rows; a pair holds 16)
+constexpr int FT_NA = 16;                         // A ring slots (source rows): one pair's at KS = 15
+constexpr int FT_NZ = 3;                          // buffers of one row's design (128 pixels)
 constexpr int FT_NCM = 17;                        // distinct core matrices of a Hankel operand (M 128, K 16)
 constexpr uint32_t FT_A_BYTES = FT_NCM * 128;     // one part (hi or lo) of one source row
 constexpr int FT_WIN = FT_NCM * 8 + 8;            // staged values of a source row (x0 - r .. + 143)
@@ -73,7 +80,7 @@ constexpr long long FT_WAIT = 2000000000LL;       // ~1 s of SM clock
 static_assert(FT_WIN % 4 == 0 && FT_WIN / 4 <= 64, "two 16-byte chunks per lane at most");
 
 struct FtBar {
-    uint64_t afull[FT_NA], aempty[FT_NA], tfull[2], tempty[2], zfull, zempty;
+    uint64_t afull[FT_NA], aempty[FT_NA], tfull[2], tempty[2], zfull[FT_NZ], zempty[FT_NZ];
     uint32_t tmem;
     int abort;
     float bscale;   // power of two: max |B'| bscale = 2^14
@@ -91,7 +98,7 @@ __host__ __device__ inline FtLayout ft_layout(int ks, int zs) {
     L.a = o; o += FT_NA * 2 * FT_A_BYTES;
     L.win = o; o += FT_NPROD * FT_NWIN * FT_WIN * 4;
     L.rowb = o; o += FT_NPROD * 2 * (FT_NCM + 1) * 4 * 4;
-    L.z = o; o += 256 * (uint32_t)zs * 4;
+    L.z = o; o += FT_NZ * 128 * (uint32_t)zs * 4;
     o = (o + 15) & ~15u;
     L.bar = o; o += (uint32_t)sizeof(FtBar);
     L.total = o;
@@ -162,20 +169,19 @@ __device__ __forceinline__ FtItem ft_item(const SegFitTcArgs& a, int item) {
     return t;
 }
 
-// One thread's share of the Gram of a pair's 256 design rows, stored pixel-pair
-// interleaved (Z [128 pixel pairs][zs][2]): the 2 x 4 block bidx (rows 2 bi, 2 bi + 1,
-// columns 4 bj .. 4 bj + 3) of the upper triangle of the NPC x NPC matrix, over the
-// pixel pairs of one half of the pair (two sets of 192 threads).  Arithmetic on packed
+// One thread's share of the Gram of one image row's 128 design rows, stored pixel-pair
+// interleaved (Z [64 pixel pairs][zs][2]): the 2 x 4 block bidx (rows 2 bi, 2 bi + 1,
+// columns 4 bj .. 4 bj + 3) of the upper triangle of the NPC x NPC matrix.  Two sets of
+// 192 threads take the first and the second row of every pair.  Arithmetic on packed
 // FP32 pairs: the two lanes of every accumulator sum the even and the odd pixel of the
 // pixel pairs, 8 pixels each per fold group (8 pixel pairs), each group folded into
 // (hi, lo) by an error-free two-sum.
 struct GramShare {
-    int bi, bj, half;
+    int bi, bj;
     bool active;
     uint64_t hi[8], lo[8];
-    __device__ __forceinline__ void init(int bidx, int half_, int NPC) {
+    __device__ __forceinline__ void init(int bidx, int NPC) {
         const int nbi = (NPC + 1) / 2, nbj = (NPC + 3) / 4;
-        half = half_;
         active = false;
         bi = bj = 0;
         // column block c holds row blocks 0 .. min(nbi - 1, (4c + 3) / 2); taken in strips of
@@ -196,8 +202,8 @@ struct GramShare {
     // The fold groups past the strip's columns, and a row past the band's, hold zero rows
     // only: left out, as adding zeros to (hi, lo) changes neither.  (A NaN that reaches such
     // a row through the zero weight lies in the window of an interior pixel too.)
-    __device__ __forceinline__ void add(const float* Z, int zs, int cols, int rows) {
-        if (!active || half >= rows) return;
+    __device__ __forceinline__ void add(const float* Z, int zs, int cols) {
+        if (!active) return;
         const int groups = (cols + 15) / 16;
         for (int g = 0; g < groups; g++) {
             uint64_t acc[8];
@@ -205,7 +211,7 @@ struct GramShare {
             for (int q = 0; q < 8; q++) acc[q] = 0ull;
 #pragma unroll
             for (int k = 0; k < 8; k++) {
-                const float* zp = Z + (size_t)(half * 64 + g * 8 + k) * zs * 2;
+                const float* zp = Z + (size_t)(g * 8 + k) * zs * 2;
                 const ulonglong2 i01 = *reinterpret_cast<const ulonglong2*>(zp + 4 * bi);
                 const ulonglong2 j01 = *reinterpret_cast<const ulonglong2*>(zp + 8 * bj);
                 const ulonglong2 j23 = *reinterpret_cast<const ulonglong2*>(zp + 8 * bj + 4);
@@ -252,7 +258,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
     uint8_t* aring = sm + L.a;                      // [FT_NA][2 parts][FT_A_BYTES]
     float* win = reinterpret_cast<float*>(sm + L.win);          // [FT_NPROD][FT_NWIN][FT_WIN]
     uint32_t* rowb = reinterpret_cast<uint32_t*>(sm + L.rowb);  // [FT_NPROD][2][(FT_NCM + 1) * 4]
-    float* Z = reinterpret_cast<float*>(sm + L.z);               // [128 pixel pairs][zs][2]
+    float* Z = reinterpret_cast<float*>(sm + L.z);               // [FT_NZ][64 pixel pairs][zs][2]
     FtBar& S = *reinterpret_cast<FtBar*>(sm + L.bar);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int* status = a.status;
@@ -300,8 +306,10 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
             tc::mbar_init(&S.tfull[b], 1);
             tc::mbar_init(&S.tempty[b], 4);   // the four accumulator-reading warps
         }
-        tc::mbar_init(&S.zfull, 4);
-        tc::mbar_init(&S.zempty, FT_WARPS - FT_GRAM_WARP + 4);   // the Gram warps and the readers
+        for (int b = 0; b < FT_NZ; b++) {
+            tc::mbar_init(&S.zfull[b], 4);    // the accumulator-reading warps
+            tc::mbar_init(&S.zempty[b], 6);   // one set's warps
+        }
         S.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -458,14 +466,24 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
         const int m = tid;
         const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
         GramShare gs;   // Gram threads 0 .. 127 of 384: set 0 (with Gram warps 8 and 9)
-        gs.init(tid, 0, NPC);
+        gs.init(tid, NPC);
         int tp = 0;
         bool run = true;
+        // the set's share of the last pair's first row, taken after the first row of the next
+        // pair is written: the other warps have rows to sum meanwhile
+        int gseg = -1, gcols = 0;
+        auto share = [&]() -> bool {
+            const int r = 2 * (tp - 1), b = r % FT_NZ;
+            if (!ft_warp_wait(S, &S.zfull[b], (uint32_t)(r / FT_NZ) & 1u, status, lane)) return false;
+            gs.add(Z + (size_t)b * 128 * zs, zs, gcols);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&S.zempty[b]);
+            return true;
+        };
         for (int item = ilo; item < ihi && run; item++) {
             const FtItem t = ft_item<KS>(a, item);
             int nvalid = 0;
-            // the pixel's variance, value and flag in the pair's two rows (read one pair ahead,
-            // before this set's Gram share, so that the loads overlap it)
+            // the pixel's variance, value and flag in the pair's two rows (read one pair ahead)
             float pv[2], pi[2];
             uint32_t pf[2];
             auto fetch = [&](int p) {
@@ -481,6 +499,9 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
                 }
             };
             fetch(0);
+            // the accumulators hold X rscale bscale (powers of two): scaled back exactly
+            // with the weight
+            const float unscale = 1.0f / (__ldg(a.rscale + t.s) * bscale);
             for (int p = 0; p < t.pairs; p++, tp++) {
                 float sqw[2], Iv[2];
 #pragma unroll
@@ -493,23 +514,19 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
                         nvalid++;
                     }
                 }
-                // the accumulators hold X rscale bscale (powers of two): scaled back exactly
-                // with the weight
-                const float unscale = 1.0f / (__ldg(a.rscale + t.s) * bscale);
-                const float wx[2] = {sqw[0] * unscale, sqw[1] * unscale};
+                if (p + 1 < t.pairs) fetch(p + 1);
                 const int acc = tp & 1;
-                bool ok = true;
-                if (lane == 0) ok = ft_wait(S, &S.tfull[acc], (uint32_t)(tp / 2) & 1u, status);
-                if (ok && lane == 0 && tp >= 1) ok = ft_wait(S, &S.zempty, (uint32_t)(tp - 1) & 1u, status);
-                if (!__shfl_sync(0xffffffffu, ok, 0)) { run = false; break; }
-                tc::fence_after();
-                // design rows, two pixels interleaved: value f of pixel px at
+                const bool odd = m & 1;
+                // row h: design rows, two pixels interleaved: value f of pixel px at
                 // Z[((px / 2) zs + f) 2 + px % 2]; lanes m, m + 1 (pixels 2k, 2k + 1) swap
                 // half of their values so that each writes whole 16-byte groups
-                const bool odd = m & 1;
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    float* zp = Z + (size_t)((h * 128 + m) >> 1) * zs * 2;
+                auto write = [&](int h) -> bool {
+                    const int r = 2 * tp + h, b = r % FT_NZ;
+                    bool ok = true;
+                    if (lane == 0 && r >= FT_NZ) ok = ft_wait(S, &S.zempty[b], (uint32_t)(r / FT_NZ - 1) & 1u, status);
+                    if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
+                    const float wx = sqw[h] * unscale;
+                    float* zp = Z + ((size_t)b * 128 + (m & ~1)) * zs;
                     // two 16-column chunks per TMEM wait
                     for (int c2 = 0; c2 < nb; c2 += 32) {
                         uint32_t rv[2][16];
@@ -526,10 +543,10 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
                             const int c = c2 + 16 * hc;
 #pragma unroll
                             for (int g = 0; g < 4; g++) {
-                                const float x0 = __uint_as_float(rv[hc][4 * g]) * wx[h];
-                                const float x1 = __uint_as_float(rv[hc][4 * g + 1]) * wx[h];
-                                const float x2 = __uint_as_float(rv[hc][4 * g + 2]) * wx[h];
-                                const float x3 = __uint_as_float(rv[hc][4 * g + 3]) * wx[h];
+                                const float x0 = __uint_as_float(rv[hc][4 * g]) * wx;
+                                const float x1 = __uint_as_float(rv[hc][4 * g + 1]) * wx;
+                                const float x2 = __uint_as_float(rv[hc][4 * g + 2]) * wx;
+                                const float x3 = __uint_as_float(rv[hc][4 * g + 3]) * wx;
                                 const float r0 = __shfl_xor_sync(0xffffffffu, odd ? x0 : x2, 1);
                                 const float r1 = __shfl_xor_sync(0xffffffffu, odd ? x1 : x3, 1);
                                 const int f = c + 4 * g + (odd ? 2 : 0);
@@ -539,49 +556,54 @@ __global__ void __launch_bounds__(FT_THREADS, 1) seg_fit_tc_kernel(SegFitTcArgs 
                             }
                         }
                     }
-                }
-                __syncwarp();   // the swapped groups are written before the last columns
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    float* zp = Z + (size_t)((h * 128 + m) >> 1) * zs * 2 + (odd ? 1 : 0);
+                    __syncwarp();   // the swapped groups are written before the last columns
+                    zp += odd ? 1 : 0;
                     zp[2 * nb] = sqw[h];
                     zp[2 * (nb + 1)] = sqw[h] * Iv[h];
                     for (int c = nb + 2; c < zs; c++) zp[2 * c] = 0.0f;
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (h == 1) tc::mbar_arrive(&S.tempty[acc]);
+                        tc::mbar_arrive(&S.zfull[b]);
+                    }
+                    return true;
+                };
+                bool ok = true;
+                if (lane == 0) ok = ft_wait(S, &S.tfull[acc], (uint32_t)(tp / 2) & 1u, status);
+                if (!__shfl_sync(0xffffffffu, ok, 0)) { run = false; break; }
+                tc::fence_after();
+                if (!write(0)) { run = false; break; }
+                if (gseg >= 0) {
+                    if (!share()) { run = false; break; }
+                    if (gseg != t.s) gs.flush(a.gram + (long)gseg * NPC * NPC, NPC);
                 }
-                tc::fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    tc::mbar_arrive(&S.tempty[acc]);
-                    tc::mbar_arrive(&S.zfull);
-                }
-                if (p + 1 < t.pairs) fetch(p + 1);
-                // this set's share of the pair's Gram, once all four readers have written
-                if (!ft_warp_wait(S, &S.zfull, (uint32_t)tp & 1u, status, lane)) { run = false; break; }
-                gs.add(Z, zs, t.cols, t.rows - 2 * p);
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&S.zempty);
+                gseg = t.s;
+                gcols = t.cols;
+                if (!write(1)) { run = false; break; }
             }
             if (!run) break;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) nvalid += __shfl_xor_sync(0xffffffffu, nvalid, o);
             if (lane == 0 && nvalid) atomicAdd(a.n_pix + t.s, nvalid);
-            if (item + 1 == ihi || a.items[item + 1].x != t.s) gs.flush(a.gram + (long)t.s * NPC * NPC, NPC);
         }
+        if (run && gseg >= 0 && share()) gs.flush(a.gram + (long)gseg * NPC * NPC, NPC);
     } else if (warp >= FT_GRAM_WARP) {
         // ---------------- Gram warps: Gram threads 128 .. 383 (the readers are 0 .. 127); set
-        // s = gt / 192 takes the pixel pairs of half s of the pair's rows
-        const int gt = 128 + tid - FT_GRAM_WARP * 32;
+        // h = gt / 192 takes row h of every pair
+        const int gt = 128 + tid - FT_GRAM_WARP * 32, h = gt / 192;
         GramShare gs;
-        gs.init(gt % 192, gt / 192, NPC);
+        gs.init(gt % 192, NPC);
         int tp = 0;
         bool run = true;
         for (int item = ilo; item < ihi && run; item++) {
             const FtItem t = ft_item<KS>(a, item);
             for (int p = 0; p < t.pairs; p++, tp++) {
-                if (!ft_warp_wait(S, &S.zfull, (uint32_t)tp & 1u, status, lane)) { run = false; break; }
-                gs.add(Z, zs, t.cols, t.rows - 2 * p);
+                const int r = 2 * tp + h, b = r % FT_NZ;
+                if (!ft_warp_wait(S, &S.zfull[b], (uint32_t)(r / FT_NZ) & 1u, status, lane)) { run = false; break; }
+                if (2 * p + h < t.rows) gs.add(Z + (size_t)b * 128 * zs, zs, t.cols);
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&S.zempty);
+                if (lane == 0) tc::mbar_arrive(&S.zempty[b]);
             }
             if (!run) break;
             // the segment's blocks are complete in this CTA when its next item is another segment's
