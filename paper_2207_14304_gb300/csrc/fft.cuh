@@ -60,6 +60,23 @@ template <int S, typename C> FFT_HD void dft8(C* v) {
     v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
 }
 
+// dft8 of values whose elements 2 .. 5 are zero, with the same roundings.
+template <int S, typename C> FFT_HD void dft8_few(C* v) {
+    using R = decltype(v[0].x);
+    const C a = v[0], b = v[1], c = v[6], d = v[7], ci = cmul_i<S>(c), di = cmul_i<S>(d);
+    const C e0 = cadd(a, c), e1 = csub(a, ci), e2 = csub(a, c), e3 = cadd(a, ci);
+    const C o0 = cadd(b, d);
+    C o1 = csub(b, di), o2 = csub(b, d), o3 = cadd(b, di);
+    const R r = (R)0.70710678118654752440;
+    o1 = cmul(o1, C{r, (R)S * r});
+    o2 = cmul_i<S>(o2);
+    o3 = cmul(o3, C{-r, (R)S * r});
+    v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
+    v[1] = cadd(e1, o1); v[5] = csub(e1, o1);
+    v[2] = cadd(e2, o2); v[6] = csub(e2, o2);
+    v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
+}
+
 // One Stockham pass of radix RAD over a sequence of length T held in a
 // (stride 1), writing b: butterfly j (0 <= j < T / RAD) reads a[j + r T/RAD],
 // multiplies by e^{S 2 pi i r k / (Ns RAD)} (k = j mod Ns) and writes the
@@ -145,8 +162,9 @@ template <int T> struct TwTab {
 };
 
 // Lane values of a pass of radix RAD with Ns points done, to the next pass's
-// lane values; ST the element stride of the sequence in shared memory.
-template <int T, int RAD, int Ns, int ST, typename C>
+// lane values; ST the element stride of the sequence in shared memory.  FEW: only
+// values 0, 1, 6 and 7 are used next.
+template <int T, int RAD, int Ns, int ST, bool FEW = false, typename C>
 __device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
     constexpr int L = T / 8, NB = 8 / RAD;
 #pragma unroll
@@ -162,6 +180,7 @@ __device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 8; m++) {
+        if (FEW && m >= 2 && m < 6) continue;
         const int p = lane + m * L;
         v[m] = s0[(p + (p >> 3)) * ST];
     }
@@ -185,13 +204,17 @@ __device__ __forceinline__ void radix4(C (&v)[8], const TW& tw, int i0) {
 }
 
 // Every pass after the first (whose butterflies the caller has done: the PSF
-// transforms skip its zeros).  Every thread of the CTA calls it.
-template <int T, int S, int ST, typename C, typename TW>
+// transforms skip its zeros).  Every thread of the CTA calls it.  FEW: only the
+// lanes below T/32 and from T/8 - T/32 on hold values after the first pass, which the
+// second pass meets as its elements 0, 1, 6 and 7.
+template <int T, int S, int ST, bool FEW = false, typename C, typename TW>
 __device__ __forceinline__ void fft_tail(C (&v)[8], const TW& tw, C*& s0, C*& s1, int lane) {
-    cross<T, 8, 1, ST>(v, s0, s1, lane);
+    cross<T, 8, 1, ST, FEW>(v, s0, s1, lane);
 #pragma unroll
-    for (int r = 1; r < 8; r++) v[r] = tmul<S>(v[r], tw.get(r - 1));
-    dft8<S>(v);
+    for (int r = 1; r < 8; r++)
+        if (!FEW || r < 2 || r > 5) v[r] = tmul<S>(v[r], tw.get(r - 1));
+    if (FEW) dft8_few<S>(v);
+    else dft8<S>(v);
     cross<T, 8, 8, ST>(v, s0, s1, lane);
     if constexpr (T == 512) {
 #pragma unroll

@@ -314,3 +314,37 @@ def test_proper_coadd_1024(ora):
                + np.linalg.norm(o["R"]))
     assert np.abs(R - o["R"]).max() <= 8 * eR
     assert np.abs(S - o["S"]).max() <= 8 * eS
+
+
+@pytest.mark.parametrize("T,ps", [(256, 15), (256, 3), (512, 31), (512, 29)])
+def test_zero_rim_of_a_stamp_changes_nothing(T, ps):
+    """PSF stamps up to the side whose transforms leave out zeros, and the same stamps inside a rim
+    of zeros that takes them past it: the same bits."""
+    rng = np.random.default_rng(T + ps)
+    rim = max((T // 16 - ps) // 2 + 1, 1)
+    small = rng.normal(0, 0.1, (2, ps, ps)).astype(np.float32)
+    small[:, ps // 2, ps // 2] = 1.0
+    large = np.pad(small, ((0, 0), (rim, rim), (rim, rim)))
+    assert ps // 2 < T // 32 <= large.shape[1] // 2
+    img = [torch.from_numpy(rng.normal(0, 5, (T, T)).astype(np.float32)).cuda() for _ in range(2)]
+    rec = np.zeros(1, B.ZOGY_TILE_DTYPE)
+    rec[0] = (0, 0, 1.05, 1.0, 5.0, 4.0)
+    d_rec, shape = torch.from_numpy(rec.view(np.uint8).copy()).cuda(), B.argus_shape(T, T, T)
+    org, F, sg = torch.zeros((1, 2), dtype=torch.int32, device="cuda"), torch.ones(2, device="cuda"), torch.full((2,), 5.0, device="cuda")
+    stack = torch.stack(img)
+    plan = B.proper_plan_create(0, T, 1)
+    try:
+        out = []
+        for p in (small, large):
+            D, S, PD, S2, R2, PR = (torch.full((1, T, T), -7.0, device="cuda") for _ in range(6))
+            sig = torch.zeros(1, dtype=torch.float64, device="cuda")
+            pn, pr = (torch.from_numpy(q[None].copy()).cuda() for q in p)
+            B.argus_zogy(plan, *img, shape, d_rec, 1, pn, pr, p.shape[1], 1e-8, D, S, PD, sig)
+            B.argus_proper_coadd(plan, stack, 2, shape, org, 1, F, sg, torch.from_numpy(p).cuda(), p.shape[1], 1e-8, S2,
+                                 R2, PR, psf_per_tile=False)
+            torch.cuda.synchronize()
+            out.append((D, S, PD, sig, S2, R2, PR))
+        for a, b in zip(*out):
+            assert torch.equal(a, b)
+    finally:
+        B.proper_plan_destroy(plan)
