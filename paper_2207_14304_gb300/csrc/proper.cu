@@ -406,6 +406,15 @@ __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) zogy_col_
     float2 v[8], xs[8], PD[8];
 #pragma unroll
     for (int m = 0; m < 8; m++) v[m] = a.z[blk + (long)(lane + m * L) * CB + c];
+    // the PSF transforms are wanted after this one: on their way to the L2 now (869 -> 830 us
+    // for 247 tiles of 512; registers leave no room to load them ahead)
+    if (lane % 8 == 0) {
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const int ky = lane + m * L;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.spec + sp + (mir ? (T - ky) & (T - 1) : ky)));
+        }
+    }
     fft::fft_reg<T, -1, CB>(v, tw, b0, b1, lane);
     float s = 0.0f, sl = 0.0f;                             // sum of |P_D|^2 as an unevaluated pair
 #pragma unroll
