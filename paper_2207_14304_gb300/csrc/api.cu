@@ -4,6 +4,7 @@
 // in argus_create, mirroring the paper's pre-allocation of reference and
 // calibration frames on the GPU at the start of each pointing (Sec. 4,
 // "Pipeline Implementation").  No entry point allocates afterwards.
+#include <algorithm>
 #include <stdlib.h>
 #include <string.h>
 
@@ -135,7 +136,9 @@ extern "C" int argus_create(argus_ctx** out, int device, size_t max_pixels, int 
     c->max_coeffs = max_coeffs;
     c->np_cols = argus_round_up(max_coeffs + 1, 16);
     c->det_cap = det_cap;
-    c->gram_parts = 64;
+    // partial normal matrices: more for narrow ones, where one matrix is little work (8 MB of
+    // them at 64 columns, 26 MB at 320)
+    c->gram_parts = std::max(64, (int)std::min(512L, 64L * 320 * 320 / ((long)c->np_cols * c->np_cols)));
     c->resid_parts = 512;
     c->max_cells = 4096;
     c->max_rows = (int)(max_pixels / 512 > 65536 ? (max_pixels / 512 > (1u << 26) ? (1u << 26) : max_pixels / 512) : 65536);

@@ -928,17 +928,31 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(GramArgs g, co
     if (warp == 0) tc::tmem_dealloc(tmem, 2 * GRAM_CW);
 }
 
-// M[i][j] = M[j][i] = sum over slots of part[slot][i][j] (i <= j), FP64, fixed order.
-__global__ void gram_reduce_kernel(const float* part, int nslots, int NP, double* M) {
+// M[i][j] = M[j][i] = sum over slots of part[slot][i][j] (i <= j), FP64, fixed order: 32 entries
+// per CTA, warp w sums slots w, w + 16, ... of them and the first warp the sixteen sums.  The
+// latency of the loads and FP64 adds bounds it; one thread per entry held the number of slots down.
+constexpr int GR_W = 16;
+__global__ void __launch_bounds__(32 * GR_W) gram_reduce_kernel(const float* part, int nslots, int NP, double* M) {
+    __shared__ double sum[GR_W][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long tot = (long)NP * NP;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < tot; e += (long)gridDim.x * blockDim.x) {
+    for (long e0 = blockIdx.x * 32L; e0 < tot; e0 += gridDim.x * 32L) {
+        const long e = e0 + lane;
         const int i = (int)(e / NP), j = (int)(e - (long)i * NP);
-        if (i > j) continue;
+        const bool use = e < tot && i <= j;
         double s = 0.0;
+        if (use) {
 #pragma unroll 8
-        for (int sl = 0; sl < nslots; sl++) s += (double)part[(long)sl * tot + e];
-        M[(long)i * NP + j] = s;
-        M[(long)j * NP + i] = s;
+            for (int sl = warp; sl < nslots; sl += GR_W) s += (double)part[(long)sl * tot + e];
+        }
+        sum[warp][lane] = s;
+        __syncthreads();
+        if (warp == 0 && use) {
+            for (int w = 1; w < GR_W; w++) s += sum[w][lane];
+            M[(long)i * NP + j] = s;
+            M[(long)j * NP + i] = s;
+        }
+        __syncthreads();
     }
 }
 
@@ -2203,11 +2217,13 @@ extern "C" int argus_fit_kernel(argus_ctx* ctx, const float* sci, const float* s
         design_kernel<<<ctx->num_sms * 4, 256, sizeof(int) * 2 * g.NP, st>>>(g, ctx->rowmeta, ctx->design); argus_count_launch(1);
         const int ntile = (g.NP + GT - 1) / GT;
         const int npair = ntile * (ntile + 1) / 2;
-        int nslots = ctx->num_sms * 3 / npair;   // three CTAs per SM
-        if (nslots < 1) nslots = 1;
+        // three CTAs per SM, as long as a slot has eight chunks of rows (64 stamps of 52 columns on
+        // 32 slots: 27 us and 14 in the reduction, now 12 and 9)
+        int nslots = ctx->num_sms * 3 / npair;
         if (nslots > ctx->gram_parts / 2) nslots = ctx->gram_parts / 2;
-        const long nch = (max_rows + GK - 1) / GK;
+        const long nch = (max_rows + 8 * GK - 1) / (8 * GK);
         if (nslots > nch) nslots = (int)nch;
+        if (nslots < 1) nslots = 1;
         g.nslots = nslots;
         part_slots = 2 * nslots;   // hi and lo halves of the double-float partials
         gram_cp_kernel<<<dim3(npair, nslots), 256, 0, st>>>(g, ctx->design, ntile); argus_count_launch(1);
@@ -2251,7 +2267,8 @@ extern "C" int argus_fit_kernel(argus_ctx* ctx, const float* sci, const float* s
     }
     if ((rc = argus_launch_status())) return rc;
     const int NP = g.NP;
-    gram_reduce_kernel<<<ctx->num_sms, 256, 0, st>>>(ctx->gram_part, part_slots, NP, ctx->M); argus_count_launch(1);
+    const long rblk = ((long)NP * NP + 31) / 32, rmax = 8L * ctx->num_sms;
+    gram_reduce_kernel<<<(unsigned)(rblk < rmax ? rblk : rmax), 32 * GR_W, 0, st>>>(ctx->gram_part, part_slots, NP, ctx->M); argus_count_launch(1);
 
     const size_t ld = (size_t)ctx->np_cols;
     double* c = ctx->vec + 1 * ld;      // current solution (orthonormal basis)
