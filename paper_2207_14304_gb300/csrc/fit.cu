@@ -1506,16 +1506,22 @@ __global__ void finalize_kernel(BasisDev b, const double* c, const double* S, co
         *st = s;
     }
     if (bad) return;
-    for (int j = threadIdx.x; j < Nc; j += blockDim.x) {
-        double v;
-        if (j == 0 || j >= 1 + (nb - 1) * Ks) {
-            v = c[j];
-        } else {
+    // eight lanes to a coefficient: the latency of the FP64 chain bounds the kernel (one lane: 16 us
+    // for 50 coefficients, now 7)
+    const int sub = threadIdx.x & 7;
+    for (int j0 = 0; j0 < Nc; j0 += blockDim.x / 8) {
+        const int j = j0 + threadIdx.x / 8;
+        const bool plain = j == 0 || j >= 1 + (nb - 1) * Ks;
+        double v = 0.0;
+        if (j < Nc && plain) {
+            if (sub == 0) v = c[j];
+        } else if (j < Nc) {
             const int n = 1 + (j - 1) / Ks, k = (j - 1) % Ks;
-            v = 0.0;
-            for (int m = n; m < nb; m++) v += S[n * nb + m] * c[1 + (m - 1) * Ks + k];
+#pragma unroll 4
+            for (int m = n + sub; m < nb; m += 8) v += S[n * nb + m] * c[1 + (m - 1) * Ks + k];
         }
-        coeffs[j] = v;
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (sub == 0 && j < Nc) coeffs[j] = v;
     }
 }
 
