@@ -157,7 +157,8 @@ int argus_calibrate(argus_ctx *ctx, const uint16_t *raw, argus_shape shape,
 /* Sigma-clipped mean coadd of n raw frames (paper Sec. 4.1.3, deep coaddition;
  * a clipped mean stands in for the matched filter there).  raw_stack: uint16
  * [n][h][pitch]; shifts_xy: float [n][2] (device), frame f is sampled at
- * (x + dx_f, y + dy_f) by bilinear interpolation of its calibrated pixels;
+ * (x + dx_f, y + dy_f) by bilinear interpolation of its calibrated pixels (a
+ * shift that leaves the frame or is not finite gives no valid sample);
  * clip: up to max_iter rounds of rejecting |v - median| > kappa * sigma
  * (population sigma about the mean); output coadd = c + sum(v - c)/n_used
  * about the final median c, var = sum V_f / n_used^2, n_used (uint8).

@@ -139,6 +139,21 @@ __device__ __forceinline__ float2 calib_pair(const CoaddArgs& a, int raw, float2
     return make_float2(ok ? cv : qnan(), (fmaxf(ng, 0.0f) + a.rn2) * (c.x * c.x));
 }
 
+// One axis of a frame's shift: its integer part and its fraction.  A window that starts
+// `size` pixels (the frame's extent along the axis) past a tile's own place, or the window's
+// own extent more than that before it, meets no pixel of the frame from any tile, so larger shifts are
+// held there; so is one that is not a number.  Window coordinates and the windows' union
+// then stay in range whatever the shifts are.
+struct ShiftPart { int whole; float frac; };
+__host__ __device__ __forceinline__ ShiftPart split_shift(float shift, int size) {
+    const double d = shift, fl = floor(d);
+    return {(int)fmin(fmax(fl, -(double)size - CWX), (double)size), (float)(d - fl)};
+}
+// Whether the union of windows whose integer shifts span dx and dy pixels fits the shared table.
+__host__ __device__ __forceinline__ bool union_fits(int dx, int dy) {
+    return ((long)CWX + dx) * ((long)CWY + dy) <= UCAP;
+}
+
 // The raw pixels of column gx, rows gy .. gy + 8 of frame f (clamped to the frame).
 __device__ __forceinline__ void load_window(const CoaddArgs& a, int f, int gx, int gy, int (&raw)[CWY]) {
     const uint16_t* src = a.raw + (long)f * a.frame_stride + min(max(gx, 0), a.w - 1);
@@ -167,10 +182,9 @@ __global__ void __launch_bounds__(CT, NMAX <= 32 ? 2 : 1) coadd_kernel(CoaddArgs
     if (tid == 0) { s_umin[0] = s_umin[1] = 1 << 30; s_uwh[0] = s_uwh[1] = -(1 << 30); }
     __syncthreads();
     for (int f = tid; f < a.nf; f += blockDim.x) {
-        const double dx = a.shifts[2 * f], dy = a.shifts[2 * f + 1];
-        const double fx = floor(dx), fy = floor(dy);
-        const int ix = (int)fx, iy = (int)fy;
-        const float fxf = (float)(dx - fx), fyf = (float)(dy - fy);
+        const ShiftPart sx = split_shift(a.shifts[2 * f], a.w), sy = split_shift(a.shifts[2 * f + 1], a.h);
+        const int ix = sx.whole, iy = sy.whole;
+        const float fxf = sx.frac, fyf = sy.frac;
         atomicMin(&s_umin[0], ix); atomicMin(&s_umin[1], iy);
         atomicMax(&s_uwh[0], ix); atomicMax(&s_uwh[1], iy);
         s_ix[f] = ix;
@@ -181,7 +195,7 @@ __global__ void __launch_bounds__(CT, NMAX <= 32 ? 2 : 1) coadd_kernel(CoaddArgs
     __syncthreads();
     const int ixmin = s_umin[0], iymin = s_umin[1];
     const int UW = CWX + (s_uwh[0] - ixmin), UH = CWY + (s_uwh[1] - iymin);
-    const bool uni = UW * UH <= UCAP;      // the same for every CTA
+    const bool uni = union_fits(s_uwh[0] - ixmin, s_uwh[1] - iymin);   // the same for every CTA
     const int ntx = (a.w + CTX - 1) / CTX, nty = (a.h + CTY - 1) / CTY;
     const int o = warp * CWX + lane;       // output row `warp`, column `lane`
     float* col = ss + tid;

@@ -599,6 +599,46 @@ def test_coadd_shift_forms(ora, nf, w, h, shifts):
         B.argus_destroy(ctx)
 
 
+@pytest.mark.parametrize("nf", [5, 13, 30])
+def test_coadd_shifts_off_the_frame(nf):
+    """Frames whose shift is not finite or leaves the frame count as frames without a usable pixel:
+    the same bits as with those frames saturated throughout."""
+    w, h = 77, 45
+    far = [(np.nan, 0.0), (0.0, np.nan), (np.inf, 0.5), (-0.5, -np.inf), (-3e9, 5e4), (5e4, -5e4), (0.0, 2147483520.0),
+           (np.nan, np.nan), (46341.0, 0.0), (0.25, -h - 9.0), (float(w), 0.0)]
+    rng = np.random.default_rng(nf)
+    raw = rng.normal(420, 20, (nf, h, w)).round().clip(0, 65535).astype(np.uint16)
+    sh = rng.uniform(-1.5, 1.5, (nf, 2)).astype(np.float32)
+    cal = synth.make_calib(w, h, seed=nf, bad_frac=0.02)
+    pitch = pitch_for(w)
+    calg = B.make_calib(cal.bias, dev_pitched(cal.dark.numpy()), dev_pitched(cal.flat.numpy()),
+                        dev_pitched(cal.bpm.numpy()), cal.gain, cal.read_noise, 60000)
+    ctx = ctx_for(w, h)
+    try:
+        for k in range(0, len(far), 2):
+            gone = {1: far[k], nf - 1: far[(k + 1) % len(far)]}
+            out = []
+            for lost in (True, False):
+                r, s = raw.copy(), sh.copy()
+                for f, v in gone.items():
+                    if lost:
+                        s[f] = v
+                    else:
+                        r[f], s[f] = 65535, 0.0
+                stack = torch.zeros((nf, h, pitch), dtype=torch.uint16)
+                stack[:, :, :w] = torch.from_numpy(r)
+                co, va = torch.full((h, pitch), -7.0, device="cuda"), torch.full((h, pitch), -7.0, device="cuda")
+                nu = torch.full((h, pitch), 7, dtype=torch.uint8, device="cuda")
+                B.argus_coadd(ctx, stack.cuda(), nf, B.argus_shape(w, h, pitch), torch.from_numpy(s).cuda(), calg, 3.0, 5,
+                              co, va, nu)
+                torch.cuda.synchronize()
+                out.append((co, va, nu))
+            for a, b in zip(*out):
+                assert torch.equal(a, b)
+    finally:
+        B.argus_destroy(ctx)
+
+
 @pytest.mark.parametrize("w,h,ks,deg", [(300, 700, 21, 2), (1100, 333, 11, 1), (129, 2200, 21, 0), (2600, 150, 11, 0)])
 def test_subtract_does_not_depend_on_bands(ora, w, h, ks, deg):
     """The difference and its variance of a frame equal, bit for bit away from the cut, those of

@@ -1,0 +1,61 @@
+"""The index and shift arithmetic of the kernels on the CPU: host-callable functions of
+the .cu files, compiled by nvcc as host code with a small driver each
+(tests/host_drivers).  Needs nvcc, no GPU."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2207_14304_gb300", "csrc")
+DRV = os.path.join(ROOT, "tests", "host_drivers")
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    """driver(name): the path of the compiled driver `name`; work files go beside it."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not found")
+    d = tmp_path_factory.mktemp("host_lanes")
+
+    def build(name):
+        if not (d / name).exists():
+            subprocess.check_call([nvcc, "-O2", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I", CSRC,
+                                   "-I", os.path.join(ROOT, "include"), "-I", DRV, "-o", str(d / name),
+                                   os.path.join(DRV, name + ".cu")])
+        return d / name
+    return build
+
+
+def _run(exe, *args):
+    subprocess.check_call([str(exe), *map(str, args)], cwd=exe.parent)
+
+
+# --------------------------------------------------------------------------- clipped coadd
+@pytest.mark.parametrize("size", [1, 31, 6388, 1 << 20])
+def test_coadd_shifts_stay_in_range(driver, size):
+    """Shifts inside the frame split exactly; any other, and any that is not finite, gives a
+    window that no tile of the frame finds a pixel in, with coordinates and a union in range."""
+    exe = driver("host_coadd_shift")
+    v = np.array([0, -0.25, 0.5, 1, -1, size - 1, -size, size, size + 0.5, -size - 40, 46341, -46341, 65536, 1e9, -1e9, 2147483520,
+                  -2147483648, 3e9, -3e9, 3e38, -3e38, np.inf, -np.inf, np.nan], np.float32)
+    v.tofile(exe.parent / "shifts.bin")
+    _run(exe, size, "shifts.bin", "shifts.out")
+    raw = (exe.parent / "shifts.out").read_bytes()
+    n = v.size
+    whole, frac = np.frombuffer(raw, np.int32, n), np.frombuffer(raw, np.float32, n, 4 * n)
+    fits = np.frombuffer(raw, np.uint8, n * n, 8 * n).reshape(n, n)
+    inside = np.abs(v) <= size
+    d = v[np.isfinite(v)].astype(np.float64)
+    np.testing.assert_array_equal(whole[inside], np.floor(v[inside]))
+    np.testing.assert_array_equal(frac[np.isfinite(v)], (d - np.floor(d)).astype(np.float32))
+    assert np.isnan(frac[~np.isfinite(v)]).all()
+    # a tile starts in [0, size); its window reaches 32 pixels on
+    first, last = whole.astype(np.int64), whole.astype(np.int64) + size - 1 + 31
+    assert ((first[~inside] >= size) | (last[~inside] < 0)).all()
+    assert (np.abs(first) <= size + 32).all()
+    span = np.abs(first[:, None] - first[None, :])
+    np.testing.assert_array_equal(fits, ((span + 32) * 9 <= 512) & ((span + 9) * 32 <= 512))
