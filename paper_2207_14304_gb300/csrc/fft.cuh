@@ -133,6 +133,9 @@ template <int T> struct Reg {
     static constexpr int NTW = T == 256 ? 13 : T == 512 ? 14 : 16;   // twiddles a lane uses
 };
 
+// Where position p of a sequence lies in its padded shared row.
+FFT_HD int pad(int p) { return p + (p >> 3); }
+
 // Index into the twiddle table of slot i of a lane: pass 2 (radix 8, Ns = 8) in
 // slots 0..6, then pass 3 (and 4), per butterfly.
 template <int T> FFT_HD int tw_index(int i, int lane) {
@@ -174,7 +177,7 @@ __device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
 #pragma unroll
         for (int r = 0; r < RAD; r++) {
             const int p = d + r * Ns;
-            s0[(p + (p >> 3)) * ST] = v[b + NB * r];
+            s0[pad(p) * ST] = v[b + NB * r];
         }
     }
     __syncthreads();
@@ -182,7 +185,7 @@ __device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
     for (int m = 0; m < 8; m++) {
         if (FEW && m >= 2 && m < 6) continue;
         const int p = lane + m * L;
-        v[m] = s0[(p + (p >> 3)) * ST];
+        v[m] = s0[pad(p) * ST];
     }
     C* t = s0;
     s0 = s1;

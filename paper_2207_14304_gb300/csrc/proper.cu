@@ -1,18 +1,8 @@
 // Proper-image statistics on square tiles: ZOGY subtraction (below) and the
 // proper coadd (after it) share one plan and the register FFTs of fft.cuh.
 //
-// Both are sums of real images filtered by kernels with real images: D =
-// IDFT[A N^ + B R^] in ZOGY (A = Fr Pr^ / den, B = -Fn Pn^ / den), S = sum_j
-// IDFT[c_j M_j^] in the coadd.  Two real images ride one complex transform, and
-// nothing separates them again: with Z = DFT[N + i R],
-//   Re IDFT[(A - i B) Z] = IDFT[A N^ + B R^]
-// (A, B are transforms of real images, so the other two products are imaginary).
-// So a filter is one complex product per frequency, a frequency needs nothing of
-// its mirror -k, and a whole column goes forward transform, product, inverse
-// transform in registers.  The real parts are taken where they cost least: row
-// kx and row -kx of the half-inverted image lie in the same row, and the row pass
-// folds two images into W = X + i Y with X, Y conjugate symmetric, so one row
-// transform returns both.
+// Both are sums of real images filtered by kernels with real images, and two real images
+// ride one complex row transform, Z = DFT[N + i R].
 //
 // ZOGY proper image subtraction (paper Sec. 4.2: ZOGY at base cadence and in
 // deep coadds; the statistic of Zackay, Ofek & Gal-Yam 2016), per T x T tile:
@@ -20,7 +10,8 @@
 //      with their centre at (0, 0) (wrapping around), each real PSF on the half
 //      plane kx <= T/2; (Pn, Pr) kept in FP32, max(|Pn|^2, |Pr|^2) also in FP64;
 //   2. row_fwd: rows of N + i R;
-//   3. zogy_col: columns; per frequency
+//   3. zogy_col: a column and its mirror per thread: both forward, the images
+//      separated (N^ = (Z(k) + conj Z(-k)) / 2), and per frequency of the half plane
 //        den = sqrt(sn^2 Fr^2 |Pr|^2 + sr^2 Fn^2 |Pn|^2)
 //        D   = (Fr Pr N - Fn Pn R) / den
 //        P_D = Fr Fn Pr Pn / (F_D den),   F_D = Fr Fn / sqrt(sn^2 Fr^2 + sr^2 Fn^2)
@@ -28,10 +19,13 @@
 //      all 0 where max(|Pn|, |Pr|) < eps (decided in FP64; below that floor the
 //      PSF transforms are rounding), inverse columns of each, and sum |P_D|^2 per
 //      tile, which gives sigma_S = F_D ||P_D||_2;
-//   4. row_inv: rows of D + i S (and of P_D when asked for), divided by T^2.
-// The PSF transforms are FP64 so that the floor decisions and the small
+//   4. row_inv_real: rows of D + i S (and of P_D when asked for), divided by T^2.
+// D is small where N and R agree, so the images are separated before the quotient: with
+// D left in one product with Z, its inverse columns carry the larger sum of the images
+// too, and D's error was 1.25 times as large.  S has an inverse column of its own, free of
+// D's rounding.  The PSF transforms are FP64 so that the floor decisions and the small
 // transforms near it are those of an FP64 reference; the images and the
-// filters are FP32.  216 tiles of 512^2 with a PSF pair each: 4.6 ms, against
+// filters are FP32.  216 tiles of 512^2 with a PSF pair each: 3.45 ms, against
 // 12.9 ms with whole FP64 2-D transforms and a combine pass over mirrored pairs.
 #include "argus_internal.cuh"
 #include "fft.cuh"
@@ -45,7 +39,7 @@ struct argus_proper_plan {
     int max_tiles;
     int psf_tiles;          // ZOGY PSF transforms the plan holds: that many tiles', -1 one shared pair, 0 none
     unsigned char* pool;    // pool_bytes() of scratch: see zogy_layout and run_coadd
-    double* psd;            // [max_tiles][T / CB] partial sums of |P_D(k)|^2
+    double* psd;            // [max_tiles][T / (2 CB)] partial sums of |P_D(k)|^2
     float2* tw32;           // [T] e^{-2 pi i m / T}
     double2* tw64;
 };
@@ -170,6 +164,47 @@ __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) row_inv_k
             const long e = base + (long)r * T + lane + m * Rg::LANES;
             out_x[e] = v[m].x * half;
             if (y) out_y[e] = v[m].y * half;
+        }
+    }
+}
+
+// Inverse rows of tiles whose half-inverted columns are those of real images (X(-k) = conj
+// X(k)): TWO, X in the columns 0 < kx < T/2 and Y in their mirrors' places, X + i Y in
+// columns 0 and T/2 (where both are real), and one transform gives both; otherwise X alone in
+// the columns up to T/2.  Grid tiles * T / (CB ROW_ITER).
+template <int T, bool TWO>
+__global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) row_inv_real_kernel(const float2* z, float* out_x, float* out_y,
+                                                                          const float2* twg) {
+    using Rg = fft::Reg<T>;
+    extern __shared__ __align__(16) unsigned char fft_smem[];
+    float2* sm = reinterpret_cast<float2*>(fft_smem);
+    constexpr int PER = T / (Rg::CB * ROW_ITER);
+    const int lane = threadIdx.x % Rg::LANES, seq = threadIdx.x / Rg::LANES;
+    const int t = blockIdx.x / PER, y0 = (blockIdx.x - t * PER) * Rg::CB * ROW_ITER;
+    const long base = (long)t * T * T;
+    z += base;
+    const fft::TwReg<T> tw(twg, lane);
+    float2* b0 = sm + seq * Rg::PT;
+    float2* b1 = sm + (Rg::CB + seq) * Rg::PT;
+    const float scale = 1.0f / ((float)T * (float)T);          // a power of two: exact
+#pragma unroll 1
+    for (int i = 0; i < ROW_ITER; i++) {
+        const int r = y0 + i * Rg::CB + seq;
+        float2 v[8];
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const int k = lane + m * Rg::LANES;                // k < T/2 where m < 4
+            const float2 p = z[blocked<T>(r, k)], n = z[blocked<T>(r, (T - k) & (T - 1))];
+            if (lane == 0 && m % 4 == 0) v[m] = p;
+            else if (TWO) v[m] = m < 4 ? make_float2(p.x - n.y, p.y + n.x) : make_float2(n.x + p.y, p.x - n.y);
+            else v[m] = m < 4 ? p : fft::cconj(n);
+        }
+        fft::fft_reg<T, 1, 1>(v, tw, b0, b1, lane);
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const long e = base + (long)r * T + lane + m * Rg::LANES;
+            out_x[e] = v[m].x * scale;
+            if (TWO) out_y[e] = v[m].y * scale;
         }
     }
 }
@@ -300,53 +335,56 @@ struct ZArgs {
     float lo2, hi2;           // below lo2 certainly under the floor, above hi2 certainly not
     const float4* spec;       // [psf tile][T / 2 + 1][T] (Pn, Pr) at (kx, ky)
     const double* top2;       // [psf tile][T / 2 + 1][T] max(|Pn|^2, |Pr|^2)
-    float2* z;                // rows of N + i R in, half-inverted D out
-    float2* zs;               // half-inverted S
-    float2* zp;               // half-inverted P_D, or null
-    double* psd;              // [tile][T / CB]
+    float2* z;                // rows of N + i R in; half-inverted D, S out (the form row_inv_real takes)
+    float2* zp;               // half-inverted P_D in columns up to T/2, or null
+    double* psd;              // [tile][T / (2 CB)]
     const float2* tw;
     double* sigma_S;
 };
 
-// The filters at one frequency: G = (Fr Pr + i Fn Pn) / den, so that G Z is D^ up to
-// a part whose inverse is imaginary, and P_D; both 0 under the floor (above =
-// false).  Host-callable, so a CPU driver can run the same code.
 __host__ __device__ __forceinline__ float zogy_FD(argus_zogy_tile tp) {
     return tp.Fr * tp.Fn / sqrtf(tp.sn * tp.sn * tp.Fr * tp.Fr + tp.sr * tp.sr * tp.Fn * tp.Fn);
 }
-__host__ __device__ __forceinline__ void zogy_filter(float2 pn, float2 pr, bool above, argus_zogy_tile tp, float FD,
-                                                     float2& G, float2& PD) {
+
+// D, S and P_D at one frequency k from A = Z(k) and B = Z(-k), Z = DFT[N + i R], and the PSFs'
+// transforms there; 0 under the floor (above = false).  Returns |P_D|^2.  Host-callable, so a
+// CPU driver can run the same code.
+__host__ __device__ __forceinline__ double zogy_point(float2 A, float2 B, float2 pn, float2 pr, bool above, argus_zogy_tile tp,
+                                                      float FD, float2& Dh, float2& Sh, float2& PD) {
+    // N = (A + conj B) / 2, R = (A - conj B) / 2i
+    const float2 Nh = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y - B.y));
+    const float2 Rh = make_float2(0.5f * (A.y + B.y), -0.5f * (A.x - B.x));
     const float Fn = tp.Fn, Fr = tp.Fr, sn = tp.sn, sr = tp.sr;
     const float den = sqrtf(sn * sn * Fr * Fr * (pr.x * pr.x + pr.y * pr.y) +
                             sr * sr * Fn * Fn * (pn.x * pn.x + pn.y * pn.y));
-    G = PD = make_float2(0.0f, 0.0f);
+    Dh = PD = make_float2(0.0f, 0.0f);
     if (above && den > 0.0f) {
-        G = make_float2((Fr * pr.x - Fn * pn.y) / den, (Fr * pr.y + Fn * pn.x) / den);
+        // Fr Pr N - Fn Pn R
+        const float2 u = make_float2(Fr * (pr.x * Nh.x - pr.y * Nh.y) - Fn * (pn.x * Rh.x - pn.y * Rh.y),
+                                     Fr * (pr.x * Nh.y + pr.y * Nh.x) - Fn * (pn.x * Rh.y + pn.y * Rh.x));
+        Dh = make_float2(u.x / den, u.y / den);
         const float g = Fr * Fn / (FD * den);
         PD = make_float2(g * (pr.x * pn.x - pr.y * pn.y), g * (pr.x * pn.y + pr.y * pn.x));
     }
+    Sh = make_float2(FD * (Dh.x * PD.x + Dh.y * PD.y), FD * (Dh.y * PD.x - Dh.x * PD.y));
+    return (double)PD.x * PD.x + (double)PD.y * PD.y;
 }
 
-// The same for one frequency pair of separated images: A = z1(k), B = z1(-k), C = z2(k),
-// E = z2(-k) with z1 = DFT[N + i R], z2 = DFT[Pn + i Pr].  Writes W(k) = D + i S and
-// W(-k) = conj D + i conj S, P_D(k) and returns |P_D(k)|^2 (the CPU driver's form).
+// X + i Y, and its value at -k for X, Y the transforms of real images.
+__host__ __device__ __forceinline__ float2 plus_i(float2 X, float2 Y) { return make_float2(X.x - Y.y, X.y + Y.x); }
+__host__ __device__ __forceinline__ float2 plus_i_mirror(float2 X, float2 Y) { return make_float2(X.x + Y.y, Y.x - X.y); }
+
+// The step of one frequency pair on whole transforms, C = z2(k), E = z2(-k) with z2 = DFT[Pn + i
+// Pr]: W(k) = D + i S and W(-k), P_D(k); returns |P_D(k)|^2 (the CPU driver's form).
 [[maybe_unused]] __host__ __device__ __forceinline__ void zogy_pair(float2 A, float2 B, double2 C, double2 E, argus_zogy_tile tp,
                                                    double eps2, float2& Wq, float2& Wp, float2& PD, double& p2) {
     const double2 Pn = make_double2(0.5 * (C.x + E.x), 0.5 * (C.y - E.y));
     const double2 Pr = make_double2(0.5 * (C.y + E.y), -0.5 * (C.x - E.x));
     const double mn = Pn.x * Pn.x + Pn.y * Pn.y, mr = Pr.x * Pr.x + Pr.y * Pr.y;
-    const bool above = mn >= eps2 || mr >= eps2;
-    const float2 pn = f2(Pn), pr = f2(Pr);
-    const float FD = zogy_FD(tp);
-    float2 Gq, Gp, PDp;
-    zogy_filter(pn, pr, above, tp, FD, Gq, PD);
-    zogy_filter(fft::cconj(pn), fft::cconj(pr), above, tp, FD, Gp, PDp);
-    const float2 q = fft::cmul(Gq, A), m = fft::cmul(Gp, B);
-    const float2 Dh = make_float2(0.5f * (q.x + m.x), 0.5f * (q.y - m.y));
-    const float2 Sh = make_float2(FD * (Dh.x * PD.x + Dh.y * PD.y), FD * (Dh.y * PD.x - Dh.x * PD.y));
-    Wq = make_float2(Dh.x - Sh.y, Dh.y + Sh.x);
-    Wp = make_float2(Dh.x + Sh.y, Sh.x - Dh.y);
-    p2 = (double)PD.x * PD.x + (double)PD.y * PD.y;
+    float2 Dh, Sh;
+    p2 = zogy_point(A, B, f2(Pn), f2(Pr), mn >= eps2 || mr >= eps2, tp, zogy_FD(tp), Dh, Sh, PD);
+    Wq = plus_i(Dh, Sh);
+    Wp = plus_i_mirror(Dh, Sh);
 }
 
 // Grid psf_tiles * ceil((T / 2 + 1) / PSEQ).
@@ -385,73 +423,95 @@ __global__ void __launch_bounds__(PSEQ * fft::Reg<T>::LANES) zogy_psf_cols_kerne
     }
 }
 
-// Columns of the tiles: forward, filters, inverse.  Grid n_tiles * T / CB.
+// Columns of the tiles: forward, quotient, inverse.  A thread takes column kx < T/2 and its
+// mirror T - kx (column 0 and column T/2, each its own mirror, go together); after the
+// forward transforms the mirror crosses through shared memory, as Z(-k) lies in it at -ky.
+// Grid n_tiles * T / (2 CB).
 template <int T>
 __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) zogy_col_kernel(ZArgs a) {
     using Rg = fft::Reg<T>;
-    constexpr int CB = Rg::CB, L = Rg::LANES, NB = T / CB, HW = T / 2 + 1;
+    constexpr int CB = Rg::CB, L = Rg::LANES, NB = T / (2 * CB), HW = T / 2 + 1;
     extern __shared__ __align__(16) unsigned char fft_smem[];
     float2* sm = reinterpret_cast<float2*>(fft_smem);
     __shared__ double red[Rg::THREADS / 32];
     const int c = threadIdx.x % CB, lane = threadIdx.x / CB;
     const int t = blockIdx.x / NB, xb = blockIdx.x - t * NB, kx = xb * CB + c;
-    const long blk = ((long)t * NB + xb) * T * CB;
+    const bool self = kx == 0;
+    float2* zk = a.z + (long)t * T * T + blocked<T>(lane, kx);
+    float2* zm = a.z + (long)t * T * T + blocked<T>(lane, self ? T / 2 : T - kx);
     const fft::TwReg<T> tw(a.tw, lane);
     float2* b0 = sm + c;
     float2* b1 = sm + CB * Rg::PT + c;
     const argus_zogy_tile tp = a.tiles[t];
     const float FD = zogy_FD(tp);
-    const bool mir = kx > T / 2;                           // (kx, ky) from the half plane's (-kx, -ky)
-    const long sp = ((a.psf_tiles == 1 ? 0L : (long)t) * HW + (mir ? T - kx : kx)) * T;
-    float2 v[8], xs[8], PD[8];
+    const long sp = ((a.psf_tiles == 1 ? 0L : (long)t) * HW + kx) * T + lane;
+    float2 v[8], w[8], P[8];
 #pragma unroll
-    for (int m = 0; m < 8; m++) v[m] = a.z[blk + (long)(lane + m * L) * CB + c];
-    // the PSF transforms are wanted after this one: on their way to the L2 now (869 -> 830 us
-    // for 247 tiles of 512; registers leave no room to load them ahead)
+    for (int m = 0; m < 8; m++) w[m] = zm[m * L * CB];
+#pragma unroll
+    for (int m = 0; m < 8; m++) v[m] = zk[m * L * CB];
+    // the PSF transforms are wanted after these: on their way to the L2 now (registers leave no
+    // room to load them ahead)
     if (lane % 8 == 0) {
 #pragma unroll
-        for (int m = 0; m < 8; m++) {
-            const int ky = lane + m * L;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.spec + sp + (mir ? (T - ky) & (T - 1) : ky)));
-        }
+        for (int m = 0; m < 8; m++) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.spec + sp + m * L));
     }
+    fft::fft_reg<T, -1, CB>(w, tw, b0, b1, lane);
     fft::fft_reg<T, -1, CB>(v, tw, b0, b1, lane);
-    float s = 0.0f, sl = 0.0f;                             // sum of |P_D|^2 as an unevaluated pair
 #pragma unroll
-    for (int m = 0; m < 8; m++) {
-        const int ky = lane + m * L;
-        const long e = sp + (mir ? (T - ky) & (T - 1) : ky);
-        float4 q = __ldg(a.spec + e);
-        if (mir) { q.y = -q.y; q.w = -q.w; }
+    for (int m = 0; m < 8; m++) b0[fft::pad(lane + m * L) * CB] = w[m];
+    __syncthreads();
+    if (xb == 0) {                                         // the same for every thread
+#pragma unroll
+        for (int m = 0; m < 8; m++) b1[fft::pad(lane + m * L) * CB] = v[m];
+        __syncthreads();
+    }
+    double psd = 0.0;
+    const auto point = [&](float2 A, float2 B, long e, float2& D, float2& S, float2& PD) {
+        const float4 q = __ldg(a.spec + e);
         const float2 pn = make_float2(q.x, q.y), pr = make_float2(q.z, q.w);
         // the floor: FP32 moduli decide except next to it, where the FP64 one does
         const float m2 = fmaxf(pn.x * pn.x + pn.y * pn.y, pr.x * pr.x + pr.y * pr.y);
         bool above = m2 > a.hi2;
         if (!above && !(m2 < a.lo2)) above = __ldg(a.top2 + e) >= a.eps2;
-        float2 G;
-        zogy_filter(pn, pr, above, tp, FD, G, PD[m]);
-        v[m] = fft::cmul(G, v[m]);
-        xs[m] = make_float2(FD * (v[m].x * PD[m].x + v[m].y * PD[m].y), FD * (v[m].y * PD[m].x - v[m].x * PD[m].y));
+        psd += zogy_point(A, B, pn, pr, above, tp, FD, D, S, PD);
+    };
 #pragma unroll
-        for (int i = 0; i < 2; i++) {                      // exact square, two-sum into the pair
-            const float d = i ? PD[m].y : PD[m].x, h = d * d, e2 = fmaf(d, d, -h), n = s + h, b = n - s;
-            sl += e2 + ((s - (n - b)) + (h - b));
-            s = n;
+    for (int m = 0; m < 8; m++) {
+        const int at = fft::pad((T - lane - m * L) & (T - 1)) * CB;
+        const long e = sp + m * L;
+        float2 D, S, PD;
+        if (!self) {
+            point(v[m], b0[at], e, D, S, PD);
+            v[m] = D;
+            w[m] = S;
+            P[m] = PD;
+        } else {                                           // X + i Y of columns 0 and T/2, whose inverses are real
+            float2 PH;
+            point(v[m], b1[at], e, D, S, PD);
+            v[m] = plus_i(D, S);
+            point(w[m], b0[at], e + (long)(T / 2) * T, D, S, PH);
+            w[m] = plus_i(D, S);
+            P[m] = plus_i(PD, PH);
         }
     }
-    double psd = (double)s + (double)sl;
+    if (!self) psd *= 2.0;                                 // k and -k
     for (int o = 16; o > 0; o >>= 1) psd += __shfl_xor_sync(0xffffffffu, psd, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = psd;
-    fft::fft_reg<T, 1, CB>(v, tw, b0, b1, lane);           // (barriers: red is complete after it)
+    if (xb == 0) __syncthreads();                          // b1 is read
+    fft::fft_reg<T, 1, CB>(v, tw, b1, b0, lane);           // (barriers: red is complete after it, b0 read before it is written)
 #pragma unroll
-    for (int m = 0; m < 8; m++) a.z[blk + (long)(lane + m * L) * CB + c] = v[m];
-    fft::fft_reg<T, 1, CB>(xs, tw, b0, b1, lane);
+    for (int m = 0; m < 8; m++) zk[m * L * CB] = v[m];
+    fft::fft_reg<T, 1, CB>(w, tw, b1, b0, lane);
 #pragma unroll
-    for (int m = 0; m < 8; m++) a.zs[blk + (long)(lane + m * L) * CB + c] = xs[m];
+    for (int m = 0; m < 8; m++) zm[m * L * CB] = w[m];
     if (a.zp) {
-        fft::fft_reg<T, 1, CB>(PD, tw, b0, b1, lane);
+        fft::fft_reg<T, 1, CB>(P, tw, b1, b0, lane);
 #pragma unroll
-        for (int m = 0; m < 8; m++) a.zp[blk + (long)(lane + m * L) * CB + c] = PD[m];
+        for (int m = 0; m < 8; m++) {
+            a.zp[zk - a.z + m * L * CB] = self ? make_float2(P[m].x, 0.0f) : P[m];
+            if (self) a.zp[zm - a.z + m * L * CB] = make_float2(P[m].y, 0.0f);
+        }
     }
     if (threadIdx.x == 0) {
         double r = 0.0;
@@ -464,7 +524,7 @@ template <int T>
 __global__ void zogy_sigma_kernel(ZArgs a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.n_tiles) return;
-    constexpr int NB = T / fft::Reg<T>::CB;
+    constexpr int NB = T / (2 * fft::Reg<T>::CB);
     const argus_zogy_tile tp = a.tiles[t];
     const double Fn = tp.Fn, Fr = tp.Fr, sn = tp.sn, sr = tp.sr;
     const double FD = Fr * Fn / sqrt(sn * sn * Fr * Fr + sr * sr * Fn * Fn);
@@ -489,6 +549,14 @@ void launch_inv(const float2* x, const float2* y, float* ox, float* oy, int n, c
     argus_count_launch(1);
 }
 
+template <int T>
+void launch_inv_real(const float2* z, float* ox, float* oy, int n, const float2* tw, cudaStream_t s) {
+    const unsigned gx = (unsigned)((long)n * (T / (fft::Reg<T>::CB * ROW_ITER)));
+    if (oy) row_inv_real_kernel<T, true><<<gx, fft::Reg<T>::THREADS, img_smem<T>(), s>>>(z, ox, oy, tw);
+    else row_inv_real_kernel<T, false><<<gx, fft::Reg<T>::THREADS, img_smem<T>(), s>>>(z, ox, nullptr, tw);
+    argus_count_launch(1);
+}
+
 template <int T> constexpr size_t psf_smem() { return 2 * PSEQ * (size_t)fft::Reg<T>::PT * sizeof(double2); }
 template <int T> constexpr unsigned psf_col_blocks() { return (T / 2 + 1 + PSEQ - 1) / PSEQ; }
 
@@ -496,16 +564,15 @@ template <int T>
 int run(argus_proper_plan* p, ZArgs& a, const RowArgs& rows, const PsfArgs* psf, float* D, float* S, float* PD,
         cudaStream_t s) {
     using Rg = fft::Reg<T>;
-    // the pool, in units of N = max_tiles T^2 pixels: z 8, zs 8, (spec, top2) 16 -- kept for
-    // calls that reuse the PSFs -- and 16 for the PSFs' row transforms, then P_D
+    // the pool, in bytes per pixel of max_tiles tiles: z 8, P_D 8, (spec, top2) 16 -- kept for
+    // calls that reuse the PSFs -- and 16 for the PSFs' row transforms
     const size_t N = (size_t)p->max_tiles * T * T, half = (size_t)(T / 2 + 1) * T;
     a.z = reinterpret_cast<float2*>(p->pool);
-    a.zs = reinterpret_cast<float2*>(p->pool + 8 * N);
+    a.zp = PD ? reinterpret_cast<float2*>(p->pool + 8 * N) : nullptr;
     float4* spec = reinterpret_cast<float4*>(p->pool + 16 * N);
     double* top2 = reinterpret_cast<double*>(spec + half * p->max_tiles);
     a.spec = spec;
     a.top2 = top2;
-    a.zp = PD ? reinterpret_cast<float2*>(p->pool + 32 * N) : nullptr;
     a.psd = p->psd;
     a.tw = p->tw32;
     if (psf) {
@@ -520,10 +587,10 @@ int run(argus_proper_plan* p, ZArgs& a, const RowArgs& rows, const PsfArgs* psf,
     r.tw = p->tw32;
     r.z = a.z;
     launch_rows<T>(r, 1, s);
-    zogy_col_kernel<T><<<(unsigned)a.n_tiles * (T / Rg::CB), Rg::THREADS, img_smem<T>(), s>>>(a);
+    zogy_col_kernel<T><<<(unsigned)a.n_tiles * (T / (2 * Rg::CB)), Rg::THREADS, img_smem<T>(), s>>>(a);
     argus_count_launch(1);
-    launch_inv<T>(a.z, a.zs, D, S, a.n_tiles, p->tw32, s);
-    if (PD) launch_inv<T>(a.zp, nullptr, PD, nullptr, a.n_tiles, p->tw32, s);
+    launch_inv_real<T>(a.z, D, S, a.n_tiles, p->tw32, s);
+    if (PD) launch_inv_real<T>(a.zp, PD, nullptr, a.n_tiles, p->tw32, s);
     if (a.sigma_S) {
         zogy_sigma_kernel<T><<<(a.n_tiles + 127) / 128, 128, 0, s>>>(a);
         argus_count_launch(1);
@@ -533,7 +600,11 @@ int run(argus_proper_plan* p, ZArgs& a, const RowArgs& rows, const PsfArgs* psf,
 
 // ---------------------------------------------------------------------------
 // Proper coaddition (paper Sec. 4.1.3: a per-image matched filter; the
-// statistic of Zackay & Ofek 2017).  With w_j = F_j / s_j^2:
+// statistic of Zackay & Ofek 2017).  The frames of a pair are never separated: with Z =
+// DFT[M_0 + i M_1] and c_0, c_1 transforms of real kernels,
+//   Re IDFT[(c_0 - i c_1) Z] = IDFT[c_0 M_0^ + c_1 M_1^]
+// (the other two products' inverses are imaginary), so a pair costs one complex product per
+// frequency and the real parts are taken by the inverse rows.  With w_j = F_j / s_j^2:
 //   S = sum_j IDFT[w_j conj(P_j) M_j] = Re IDFT[U],
 //   U = sum over frame pairs of (w_0 conj P_0 - i w_1 conj P_1) DFT[M_0 + i M_1]
 // (FP32), den^2 = sum_j F_j^2 / s_j^2 |P_j|^2 and max_j |P_j|^2 in FP64 on the half
@@ -919,7 +990,8 @@ template <typename K> bool dyn_smem(K* kernel, size_t bytes) {
 template <int T>
 bool set_smem() {
     const size_t i = img_smem<T>(), p = psf_smem<T>();
-    return dyn_smem(row_fwd_kernel<T>, i) && dyn_smem(row_inv_kernel<T>, i) && dyn_smem(zogy_col_kernel<T>, i) &&
+    return dyn_smem(row_fwd_kernel<T>, i) && dyn_smem(row_inv_kernel<T>, i) &&
+           dyn_smem(row_inv_real_kernel<T, true>, i) && dyn_smem(row_inv_real_kernel<T, false>, i) && dyn_smem(zogy_col_kernel<T>, i) &&
            dyn_smem(coadd_col_kernel<T>, i) && dyn_smem(psf_rows_kernel<T>, p) && dyn_smem(zogy_psf_cols_kernel<T>, p) &&
            dyn_smem(coadd_psf_cols_kernel<T>, p);
 }
@@ -938,7 +1010,7 @@ extern "C" int argus_proper_plan_create(int device, int tile, int max_tiles, arg
     p->device = device;
     p->tile = tile;
     p->max_tiles = max_tiles;
-    const size_t parts = (size_t)max_tiles * (tile / (tile == 256 ? 8 : 4));
+    const size_t parts = (size_t)max_tiles * (tile / (tile == 256 ? 16 : 8));
     bool ok = cudaMalloc((void**)&p->pool, pool_bytes(tile, max_tiles)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&p->psd, parts * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&p->tw32, (size_t)tile * sizeof(float2)) == cudaSuccess;
