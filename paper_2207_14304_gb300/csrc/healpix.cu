@@ -29,6 +29,7 @@ struct HpArgs {
     double cr, sr, inv_scale, cx, cy;
     float* out;
     uint8_t* cov;
+    long long xmax, ymax;      // the frame's last column and row as positions of the patch path
 };
 
 __host__ __device__ __forceinline__ void hp_sincospi(double t, double* s, double* c) {
@@ -195,6 +196,11 @@ constexpr double HP_FAR = 500000.0;      // positions in fixed point stay below 
 
 __host__ __device__ __forceinline__ int hp_node_row(int j) { return j == 0 ? 0 : (j == 1 ? 10 : (j == 2 ? 21 : 31)); }
 
+// The last position of a frame's axis, or the largest there is where the frame goes on past 2^19.
+__host__ inline long long hp_last(int size) {
+    return size - 1 < 1 << (63 - HP_FRAC) ? (long long)(size - 1) << HP_FRAC : 0x7fffffffffffffffll;
+}
+
 // Lagrange weights of the node columns 0, 21, 42, 63 at each column of a patch, times 2^HP_FRAC.
 struct HpWeights { double w[HP_PATCH][4]; };
 constexpr HpWeights hp_make_weights() {
@@ -345,7 +351,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
                 d[i][3] = f[3];
             }
         }
-        const long long xmax = (long long)(a.w - 1) << HP_FRAC, ymax = (long long)(a.h - 1) << HP_FRAC;
+        const long long xmax = a.xmax, ymax = a.ymax;
         long e = (long)(r0 + grp * (HP_HALF / 4)) * m + c0 + col;
 #pragma unroll 2
         for (int i = 0; i < HP_HALF / 4; i++, e += m) {
@@ -436,6 +442,7 @@ extern "C" int argus_healpix_resample(const float* frame, const uint8_t* flags, 
     HpArgs a;
     a.frame = frame; a.flags = flags; a.pitch = shape.pitch; a.w = shape.w; a.h = shape.h;
     a.segs = segs; a.n_seg = n_seg; a.nside_seg = nside_seg; a.k = k; a.out = out; a.cov = coverage;
+    a.xmax = hp_last(shape.w); a.ymax = hp_last(shape.h);
     hp_fill_wcs(a, wcs);
     if (k >= 6) {                                  // whole 64 x 64 patches
         const long long patches = (long long)n_seg << (2 * (k - 6));

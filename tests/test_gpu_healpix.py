@@ -99,3 +99,35 @@ def test_healpix_patches(ora, nside_seg, k, delta0, step, rot):
             else:
                 assert np.abs(out[i] - o).max() <= tol
         assert not out[-1].any() and not cov[-1].any()      # not a pixel of this NSIDE
+
+
+@pytest.mark.parametrize("cx", [2.9e5, 5.0e5, 5.5e5])
+def test_healpix_frame_wider_than_the_fixed_point(ora, cx):
+    """A frame of more than 2^19 columns, whose last one is past the fixed-point positions' range:
+    segments below the patch path's limit of 5e5 pixels, across it and above, at the bars of the parity test."""
+    from oracle import healpix as hp
+    rng = np.random.default_rng(int(cx))
+    w, h, nside, k, m = 600000, 40, 256, 6, 64
+    scale = math.sqrt(4 * math.pi / (12.0 * (nside << k) ** 2))
+    wcs = (0.9, 0.3, scale, 0.8, cx, 17.25)
+    frame = np.full((h, w), 300.0, np.float32)
+    x0 = int(cx) - 200
+    frame[:, x0:x0 + 400] += rng.normal(0, 10, (h, 400)).astype(np.float32)
+    fl = np.zeros((h, w), np.uint8)
+    fl[:, x0:x0 + 400] = rng.random((h, 400)) < 0.01
+    p = np.arange(12 * nside * nside)
+    ix, iy, f = hp.nest2xyf(p, nside)
+    x, y = hp.gnomonic(hp.xyf2vec(ix, iy, f, nside), *wcs)
+    d = np.where(np.isfinite(x), (x - cx) ** 2 + (y - h / 2) ** 2, np.inf)
+    segs = p[np.argsort(d)[:3]].astype(np.int64)
+    out = torch.full((segs.size, m, m), -7.0, device="cuda")
+    cov = torch.full((segs.size, m, m), 7, dtype=torch.uint8, device="cuda")
+    B.argus_healpix_resample(dev_pitched(frame), dev_pitched(fl), B.argus_shape(w, h, pitch_for(w)), wcs, nside, k,
+                             torch.from_numpy(segs).cuda(), segs.size, out, cov)
+    torch.cuda.synchronize()
+    out, cov = out.cpu().numpy(), cov.cpu().numpy()
+    assert cov.any()
+    for i, s in enumerate(segs):
+        o, oc = hp.resample_segment(frame, fl, int(s), nside, k, wcs)
+        np.testing.assert_array_equal(cov[i], oc)
+        assert np.abs(out[i] - o).max() <= 4 * F32_EPS * float(frame.max())
