@@ -30,6 +30,7 @@ struct HpArgs {
     float* out;
     uint8_t* cov;
     long long xmax, ymax;      // the frame's last column and row as positions of the patch path
+    bool split;                // halves that reach out of the belt are healpix_exact_kernel's
 };
 
 __host__ __device__ __forceinline__ void hp_sincospi(double t, double* s, double* c) {
@@ -41,49 +42,55 @@ __host__ __device__ __forceinline__ void hp_sincospi(double t, double* s, double
 #endif
 }
 
-// Frame position of the centre of segment-image pixel (c, r).  false when the
-// direction is behind the tangent plane.
-__host__ __device__ __forceinline__ bool hp_pixel_xy(const HpArgs& a, long long seg, int c, int r, double& x,
-                                                     double& y) {
-    const long long N = a.nside_seg;
-    const long long face = seg / (N * N);
-    if (seg < 0 || face >= 12) return false;            // not a pixel of this NSIDE
-    const long long ipf = seg - face * N * N;
-    long long X = 0, Y = 0;
+// A segment: its image's first pixel in the face, and that pixel's ring.
+struct HpSeg {
+    long long nside, x, y, jr;
+    int jp;                    // 2 pi / 8 units of the face's first pixel column
+    bool ok;                   // a pixel of this NSIDE
+};
+__host__ __device__ __forceinline__ HpSeg hp_seg(const HpArgs& a, long long seg) {
+    const long long N = a.nside_seg, face = seg / (N * N), ipf = seg - face * N * N;
+    HpSeg g;
+    g.nside = N << a.k;
+    g.ok = seg >= 0 && face < 12;
+    g.x = g.y = 0;
     for (int b = 0; (1LL << b) < N; b++) {
-        X |= ((ipf >> (2 * b)) & 1LL) << b;
-        Y |= ((ipf >> (2 * b + 1)) & 1LL) << b;
+        g.x |= ((ipf >> (2 * b)) & 1LL) << b;
+        g.y |= ((ipf >> (2 * b + 1)) & 1LL) << b;
     }
-    const long long nside = N << a.k;
-    const long long ix = (X << a.k) + c, iy = (Y << a.k) + r;
-    const int jrll[12] = {2, 2, 2, 2, 3, 3, 3, 3, 4, 4, 4, 4};
-    const int jpll[12] = {1, 3, 5, 7, 0, 2, 4, 6, 1, 3, 5, 7};
-    const long long jr = jrll[face] * nside - ix - iy - 1;
-    long long nr, kshift = 0;
-    double z, sin_t;
-    if (jr < nside) {                                    // north polar cap
-        nr = jr;
-        const double cap = (double)nr * (double)nr / (3.0 * (double)nside * (double)nside);
-        z = 1.0 - cap;
-        sin_t = sqrt(cap * (2.0 - cap));
-    } else if (jr > 3 * nside) {                         // south polar cap
-        nr = 4 * nside - jr;
-        const double cap = (double)nr * (double)nr / (3.0 * (double)nside * (double)nside);
-        z = -1.0 + cap;
-        sin_t = sqrt(cap * (2.0 - cap));
-    } else {                                             // equatorial belt
-        nr = nside;
-        z = (double)(2 * nside - jr) * 2.0 / (3.0 * (double)nside);
-        sin_t = sqrt((1.0 - z) * (1.0 + z));
-        kshift = (jr - nside) & 1;
+    g.x <<= a.k;
+    g.y <<= a.k;
+    g.jr = (face < 4 ? 2 : (face < 8 ? 3 : 4)) * g.nside - g.x - g.y - 1;
+    g.jp = (int)(face < 4 ? 2 * face + 1 : (face < 8 ? 2 * (face - 4) : 2 * (face - 8) + 1));
+    return g;
+}
+
+// z and sin(theta) of ring jr.
+__host__ __device__ __forceinline__ double2 hp_ring(long long nside, long long jr) {
+    if (jr >= nside && jr <= 3 * nside) {                // equatorial belt
+        const double z = (double)(2 * nside - jr) * 2.0 / (3.0 * (double)nside);
+        return make_double2(z, sqrt((1.0 - z) * (1.0 + z)));
     }
-    long long jp = (jpll[face] * nr + ix - iy + 1 + kshift) / 2;
+    const long long nr = jr < nside ? jr : 4 * nside - jr;
+    const double cap = (double)nr * (double)nr / (3.0 * (double)nside * (double)nside);
+    return make_double2(jr < nside ? 1.0 - cap : -1.0 + cap, sqrt(cap * (2.0 - cap)));
+}
+
+// Frame position of the centre of pixel (c, r) of a valid segment, `ring` its ring's
+// values.  false when the direction is behind the tangent plane.
+__host__ __device__ __forceinline__ bool hp_on_ring(const HpArgs& a, const HpSeg& g, int c, int r, double2 ring, double& x,
+                                                    double& y) {
+    const long long jr = g.jr - c - r;
+    const bool north = jr < g.nside, south = jr > 3 * g.nside;
+    const long long nr = north ? jr : (south ? 4 * g.nside - jr : g.nside);
+    const long long kshift = north || south ? 0 : (jr - g.nside) & 1;
+    long long jp = (g.jp * nr + (g.x + c) - (g.y + r) + 1 + kshift) / 2;
     if (jp > 4 * nr) jp -= 4 * nr;
     if (jp < 1) jp += 4 * nr;
     // phi = (jp - (kshift + 1) / 2) (pi / 2) / nr
     double sp, cp;
     hp_sincospi(((double)jp - 0.5 * (double)(kshift + 1)) / (2.0 * (double)nr), &sp, &cp);
-    const double v0 = sin_t * cp, v1 = sin_t * sp, v2 = z;
+    const double v0 = ring.y * cp, v1 = ring.y * sp, v2 = ring.x;
     const double d = v0 * a.n[0] + v1 * a.n[1] + v2 * a.n[2];
     if (!(d > 0.0)) return false;
     const double xi = (v0 * a.e[0] + v1 * a.e[1] + v2 * a.e[2]) / d;
@@ -93,19 +100,17 @@ __host__ __device__ __forceinline__ bool hp_pixel_xy(const HpArgs& a, long long 
     return true;
 }
 
-// Whether pixel (c, r) of a valid segment lies in the equatorial belt (ring index in
-// [N, 3N]); the ring index falls with c and with r, so a rectangle whose first and
-// last pixels do lies in it wholly.
-__host__ __device__ __forceinline__ bool hp_pixel_in_belt(const HpArgs& a, long long seg, int c, int r) {
-    const long long N = a.nside_seg, face = seg / (N * N), ipf = seg - face * N * N;
-    long long X = 0, Y = 0;
-    for (int b = 0; (1LL << b) < N; b++) {
-        X |= ((ipf >> (2 * b)) & 1LL) << b;
-        Y |= ((ipf >> (2 * b + 1)) & 1LL) << b;
-    }
-    const long long nside = N << a.k, jrll = face < 4 ? 2 : (face < 8 ? 3 : 4);
-    const long long jr = jrll * nside - ((X << a.k) + c) - ((Y << a.k) + r) - 1;
-    return jr >= nside && jr <= 3 * nside;
+// The same of any segment number; false for one that is no pixel of this NSIDE.
+__host__ __device__ __forceinline__ bool hp_pixel_xy(const HpArgs& a, long long seg, int c, int r, double& x, double& y) {
+    const HpSeg g = hp_seg(a, seg);
+    return g.ok && hp_on_ring(a, g, c, r, hp_ring(g.nside, g.jr - c - r), x, y);
+}
+
+// Whether the w x h pixels from (c, r) on lie wholly in the equatorial belt (ring index in
+// [N, 3N]): the ring index falls with c and with r, so the first and the last pixel tell.
+__host__ __device__ __forceinline__ bool hp_in_belt(const HpSeg& g, int c, int r, int w, int h) {
+    const long long first = g.jr - c - r;
+    return g.ok && first <= 3 * g.nside && first - (w - 1) - (h - 1) >= g.nside;
 }
 
 // Nested-lerp bilinear value of the frame at (x, y); false when not covered
@@ -183,14 +188,15 @@ __host__ __device__ __forceinline__ int hp_node(int j) { return j == 0 ? 0 : (j 
 // position costs three 64-bit additions per coordinate and no FP64: this part does
 // two FP64 operations per clock and SM, and evaluating two FP64 cubics and three
 // FP64 lerps per pixel took 3.80 ms for the 170 segments of a 9576 x 6388 frame; this
-// takes 0.546 ms (the FP64 pipe 46 % busy with nodes and columns, issue slots 61 %).
+// takes 0.521 ms (the FP64 pipe 46 % busy with nodes and columns, issue slots 61 %).
 // The frame pixels under the half (a rectangle around its nodes) are staged in
 // shared memory once, NaN where flagged or not finite: the image axes lie
 // diagonally across the frame, and gathering neighbours from global memory
 // touches about 27 lines per warp load.  The lerps run on unevaluated FP32 pairs
-// (about 2^-44 relative, then one rounding).  Halves not wholly in the belt, with
-// a node behind the tangent plane or beyond HP_FAR pixels take the exact path per
-// pixel; halves whose rectangle exceeds HP_CAP pixels gather from global memory.
+// (about 2^-44 relative, then one rounding).  Halves not wholly in the belt (unless
+// `split` leaves them to healpix_exact_kernel), with a node behind the tangent plane or
+// beyond HP_FAR pixels take the exact path per pixel; halves whose rectangle exceeds
+// HP_CAP pixels gather from global memory.
 constexpr int HP_PATCH = 64, HP_HALF = 32, HP_FRAC = 44, HP_CAP = 10240;
 constexpr double HP_FAR = 500000.0;      // positions in fixed point stay below 2^19
 
@@ -258,7 +264,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
     __shared__ double nd[2][4][4][2];                      // [half][node row][node column][x, y]
     __shared__ long long dif[2][HP_PATCH][4];              // [x, y][column] forward differences of a half
     __shared__ int box[2][4];                              // staged rectangle of a half: x0, y0, x1, y1
-    __shared__ int okh[2];                                 // half interpolated
+    __shared__ int okh[2];                                 // half: 1 interpolated, 0 exact, 2 not this kernel's
     extern __shared__ float hp_smem[];                     // staged frame pixels
     const int tid = threadIdx.x, lane = tid & 31, col = tid & 63, grp = tid >> 6;
     const int ppr = 1 << (a.k - 6);                        // patches per row
@@ -273,8 +279,9 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
         const int hf = lane >> 4, jr = (lane >> 2) & 3, jc = lane & 3;
         double x = 0.0, y = 0.0;
         const int c = c0 + hp_node(jc), r = rp + hf * HP_HALF + hp_node_row(jr);
-        const bool ok = hp_pixel_xy(a, seg, c, r, x, y) && fabs(x) < HP_FAR && fabs(y) < HP_FAR &&
-                        hp_pixel_in_belt(a, seg, c, r);
+        const HpSeg g = hp_seg(a, seg);
+        const bool belt = hp_in_belt(g, c0, rp + hf * HP_HALF, HP_PATCH, HP_HALF);
+        const bool ok = belt && hp_on_ring(a, g, c, r, hp_ring(g.nside, g.jr - c - r), x, y) && fabs(x) < HP_FAR && fabs(y) < HP_FAR;
         nd[hf][jr][jc][0] = x;
         nd[hf][jr][jc][1] = y;
         const unsigned half = hf ? 0xffff0000u : 0x0000ffffu;
@@ -288,7 +295,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
             by1 = max(by1, __shfl_xor_sync(0xffffffffu, by1, o));
         }
         if ((lane & 15) == 0) {
-            okh[hf] = all;
+            okh[hf] = all ? 1 : (a.split && !belt ? 2 : 0);
             box[hf][0] = max(bx0 - 1, 0);
             box[hf][1] = max(by0 - 1, 0);
             box[hf][2] = min(bx1 + 2, a.w - 1);
@@ -298,7 +305,8 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
     __syncthreads();
     for (int hf = 0; hf < 2; hf++) {
         const int r0 = rp + hf * HP_HALF;
-        if (!okh[hf]) {                                    // the same for the whole CTA
+        if (okh[hf] == 2) continue;                        // (the same for the whole CTA)
+        if (!okh[hf]) {
             for (int i = 0; i < HP_HALF / 4; i++) {
                 const int r = r0 + grp * (HP_HALF / 4) + i;
                 double x, y;
@@ -400,6 +408,43 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
     }
 }
 
+// Halves that reach out of the belt, per pixel on the exact path: a CTA takes HX_ROWS rows
+// of up to HX_COLS columns, a warp a row.  A pixel's ring is that of its whole
+// antidiagonal, so the CTA makes the rings' z and sin(theta) (a division and a square root
+// each) once; FP64 bounds the rest.  A 9576 x 6388 frame at a declination of 60 degrees in segments
+// of 512 x 512: 8.22 ms (in the patch kernel's exact branch 10.1, a warp per row without the
+// rings' table 9.69); a 1500 x 1100 frame in segments of 128 x 128, too few patches for the
+// SMs: 50 us (185 and 52).
+constexpr int HX_ROWS = 8, HX_COLS = 512;
+
+__global__ void __launch_bounds__(32 * HX_ROWS) healpix_exact_kernel(HpArgs a) {
+    __shared__ double2 ring[HX_COLS + HX_ROWS - 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long m = 1L << a.k;
+    const int W = (int)min(m, (long)HX_COLS), per_row = (int)(m / W);
+    const long per_seg = m / HX_ROWS * per_row;
+    for (long unit = blockIdx.x; unit < a.n_seg * per_seg; unit += gridDim.x) {
+        const long s = unit / per_seg;
+        const int q = (int)(unit - s * per_seg), c0 = q % per_row * W, r0 = q / per_row * HX_ROWS, rh = r0 & -HP_HALF;
+        const HpSeg g = hp_seg(a, a.segs[s]);
+        if (hp_in_belt(g, c0, rh, W, HP_HALF)) continue;   // the same for the whole CTA
+        __syncthreads();                                   // the last unit's rings are done with
+        if (g.ok)
+            for (int e = threadIdx.x; e < W + HX_ROWS - 1; e += blockDim.x) ring[e] = hp_ring(g.nside, g.jr - c0 - r0 - e);
+        __syncthreads();
+        const int r = r0 + warp;
+        const long row = (s * m + r) * m;
+        for (int c = c0 + lane; c < c0 + W; c += 32) {
+            if (hp_in_belt(g, c & -HP_PATCH, rh, HP_PATCH, HP_HALF)) continue;       // the patch kernel's
+            double x, y;
+            float v = 0.0f;
+            const bool ok = g.ok && hp_on_ring(a, g, c, r, ring[c - c0 + warp], x, y) && hp_bilinear(a, x, y, v);
+            a.out[row + c] = ok ? v : 0.0f;
+            if (a.cov) a.cov[row + c] = ok ? 1 : 0;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) healpix_resample_kernel(HpArgs a) {
     const long m = 1L << a.k;
     const long total = (long)a.n_seg * m * m;
@@ -428,6 +473,13 @@ __host__ inline void hp_fill_wcs(HpArgs& a, const argus_wcs& w) {
     a.cy = w.cy;
 }
 
+// Whether every pixel of the frame lies in the equatorial belt, |sin(dec)| <= 2/3: the farthest
+// corner's distance from the tangent point bounds every pixel's.
+__host__ inline bool hp_frame_in_belt(const HpArgs& a) {
+    const double dx = std::fmax(std::fabs(a.cx), std::fabs(a.w - 1 - a.cx)), dy = std::fmax(std::fabs(a.cy), std::fabs(a.h - 1 - a.cy));
+    return std::asin(std::fabs(a.n[2])) + std::atan(std::hypot(dx, dy) / a.inv_scale) < std::asin(2.0 / 3.0);
+}
+
 }  // namespace
 
 extern "C" int argus_healpix_resample(const float* frame, const uint8_t* flags, argus_shape shape, argus_wcs wcs,
@@ -448,7 +500,16 @@ extern "C" int argus_healpix_resample(const float* frame, const uint8_t* flags, 
         const long long patches = (long long)n_seg << (2 * (k - 6));
         if (patches > 0x7fffffffLL) return ARGUS_ERR_ARG;
         const size_t smem = HP_CAP * sizeof(float);
+        // a frame inside the belt has next to no pixel of a half that reaches out of it: one kernel takes
+        // them all (a second launch would add 3 us or so to calls of 31); any other frame's halves go to a
+        // kernel of their own (at declinations 45 to 80 1.2 to 3.7 times as fast)
+        a.split = !hp_frame_in_belt(a);
         healpix_patch_kernel<<<(unsigned)patches, 256, smem, (cudaStream_t)stream>>>(a);
+        if (a.split) {
+            const long m = 1L << k, units = (long)n_seg * (m / HX_ROWS) * (m < HX_COLS ? 1 : m / HX_COLS);
+            healpix_exact_kernel<<<(unsigned)(units < 152L * 32 ? units : 152L * 32), 32 * HX_ROWS, 0, (cudaStream_t)stream>>>(a);
+            argus_count_launch(1);
+        }
     } else {
         const long total = (long)n_seg << (2 * k);
         long blocks = (total + 255) / 256;

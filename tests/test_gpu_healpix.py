@@ -131,3 +131,40 @@ def test_healpix_frame_wider_than_the_fixed_point(ora, cx):
         o, oc = hp.resample_segment(frame, fl, int(s), nside, k, wcs)
         np.testing.assert_array_equal(cov[i], oc)
         assert np.abs(out[i] - o).max() <= 4 * F32_EPS * float(frame.max())
+
+
+@pytest.mark.parametrize("nside_seg,k,delta0", [(64, 10, 0.85),       # caps only, images wider than a row piece
+                                               (256, 6, 0.7297),     # the belt's edge inside the frame
+                                               (512, 7, -0.735),
+                                               (256, 6, 0.69),       # a frame inside the belt, segments beyond it
+                                               (128, 8, 1.52)])      # next to the pole
+def test_healpix_halves_out_of_the_belt(ora, nside_seg, k, delta0):
+    """Each half patch is taken by exactly one kernel, whatever part of the frame and of the segments
+    lies in the belt, at the bars of the parity test."""
+    from oracle import healpix as hp
+    rng = np.random.default_rng(nside_seg + k)
+    w, h = 700, 500
+    scale = math.sqrt(4 * math.pi / (12.0 * (nside_seg << k) ** 2))
+    wcs = (2.1, delta0, scale, -0.4, (w - 1) / 2, (h - 1) / 2)
+    frame = (300 + rng.normal(0, 10, (h, w))).astype(np.float32)
+    frame.flat[11::701] = np.nan
+    fl = (rng.random((h, w)) < 0.01).astype(np.uint8)
+    p = np.arange(12 * nside_seg * nside_seg)
+    ix, iy, f = hp.nest2xyf(p, nside_seg)
+    x, y = hp.gnomonic(hp.xyf2vec(ix, iy, f, nside_seg), *wcs)
+    d = np.where(np.isfinite(x), (x - w / 2) ** 2 + (y - h / 2) ** 2, np.inf)
+    near = p[np.argsort(d)[:1 if k == 10 else 60]]
+    segs = np.concatenate([near[:1], rng.choice(near, size=min(7, near.size - 1), replace=False), [-1]]).astype(np.int64)
+    m = 1 << k
+    out = torch.full((segs.size, m, m), -7.0, device="cuda")
+    cov = torch.full((segs.size, m, m), 7, dtype=torch.uint8, device="cuda")
+    B.argus_healpix_resample(dev_pitched(frame), dev_pitched(fl), B.argus_shape(w, h, pitch_for(w)), wcs,
+                             nside_seg, k, torch.from_numpy(segs).cuda(), segs.size, out, cov)
+    torch.cuda.synchronize()
+    out, cov = out.cpu().numpy(), cov.cpu().numpy()
+    assert cov[0].any()
+    for i, s in enumerate(segs[:-1]):
+        o, oc = hp.resample_segment(frame, fl, int(s), nside_seg, k, wcs)
+        np.testing.assert_array_equal(cov[i], oc)
+        assert np.abs(out[i] - o).max() <= 4 * F32_EPS * float(np.nanmax(frame))
+    assert not out[-1].any() and not cov[-1].any()
