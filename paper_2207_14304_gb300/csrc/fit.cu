@@ -1670,10 +1670,13 @@ __global__ void select_ring_kernel(const float* R, const uint8_t* flags, const u
 // pixels no fainter than the least of those stars, and without one it is done after one
 // read of its own pixels: steps 2 and 3 were most of the time (barriers and shared memory),
 // and their maxima can't win there.  9576 x 6388 in 20 x 20 cells: 319 -> 170 us, of which
-// one read of R is 36; a frame whose tiles all run at once gains nothing (1024 x 1024:
-// 17 -> 19 us, the extra read).
+// one read of R is 36; 4096 x 4096 106 -> 87 (with the launches around it).  Tiles that start
+// before any has finished find no star and would only pay for the read, so frames of up to
+// SEL_ROUNDS rounds of tiles go without step 0 (1024 x 1024: 23.6 us, with it 25.6; 2048 x
+// 2048 42.0 and 44.0; 3000 x 2000, 2.5 rounds, 50.2 either way).
 constexpr int SEL_TX = 128, SEL_TY = 64, SEL_QR = 3, SEL_MAX_ISO = 32, SEL_THREADS = 512;
 constexpr int SEL_LIST = SEL_TX * SEL_TY / 4;
+constexpr double SEL_ROUNDS = 2.5;      // of two tiles an SM
 
 struct SelGeom {
     int qr, ox, rw, rh, mw, mh;
@@ -1761,7 +1764,7 @@ __device__ __forceinline__ void sel_tile(int b, int w, int h, int gx, int gy, in
 template <int QR>
 __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float* R, const uint8_t* flags, long pitch,
                                                                     int w, int h, int gx, int gy, int m,
-                                                                    float max_peak, int iso, float iso_frac,
+                                                                    float max_peak, int iso, float iso_frac, bool early,
                                                                     unsigned long long* cell_key) {
     constexpr int MW = SEL_TX + 2 * QR, MH = SEL_TY + 2 * QR;
     constexpr int MOFF = (4 - QR % 4) % 4;                       // r column of mv column 0 is cx = -QR mod 4
@@ -1786,45 +1789,48 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float
     //    pixel wins in none of them.  Where few pixels are as bright, they are taken as the
     //    candidates themselves (their isolation is then tested from the first ring on), and
     //    where none is the tile is done
-    float4 own[SEL_TX * SEL_TY / 4 / SEL_THREADS];
-    constexpr int NOWN = sizeof(own) / sizeof(own[0]);
-#pragma unroll
-    for (int k = 0; k < NOWN; k++) {
-        const int e = tid + k * SEL_THREADS, Y = min(y0 + e / (SEL_TX / 4), h - 1);
-        own[k] = __ldg(reinterpret_cast<const float4*>(R + (long)Y * pitch + min(x0 + 4 * (e % (SEL_TX / 4)), (w - 1) & ~3)));
-    }
-    if (wid == 0) {
-        const int cx0 = sel_cell(x0, gx, w), ncx = sel_cell(min(x0 + SEL_TX, w) - 1, gx, w) - cx0 + 1;
-        const int cy0 = sel_cell(y0, gy, h), ncy = sel_cell(min(y0 + SEL_TY, h) - 1, gy, h) - cy0 + 1;
-        float best = INF;
-        for (int i = lane; i < ncx * ncy; i += 32) {
-            const unsigned long long key = __ldcg(cell_key + (cy0 + i / ncx) * gx + cx0 + i % ncx);
-            const unsigned ord = (unsigned)(key >> 32);
-            best = fminf(best, key ? __uint_as_float((ord & 0x80000000u) ? ord ^ 0x80000000u : ~ord) : NEG);
-        }
-        for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-        if (lane == 0) least = best;
-    }
-    __syncthreads();
-    const float lst = least;
-    const bool few = lst > NEG;                                  // every cell has a star
-    if (few) {
+    bool few = false;                                            // every cell has a star
+    if (early) {                                                 // the same for the whole grid
+        float4 own[SEL_TX * SEL_TY / 4 / SEL_THREADS];
+        constexpr int NOWN = sizeof(own) / sizeof(own[0]);
 #pragma unroll
         for (int k = 0; k < NOWN; k++) {
-            if (!(fmaxf(fmaxf(own[k].x, own[k].y), fmaxf(own[k].z, own[k].w)) >= lst)) continue;
-            const int e = tid + k * SEL_THREADS, y = e / (SEL_TX / 4), x = 4 * (e % (SEL_TX / 4)), Y = y0 + y;
-            const float v[4] = {own[k].x, own[k].y, own[k].z, own[k].w};
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const int X = x0 + x + c;
-                if (v[c] >= lst && v[c] < max_peak && v[c] < INF && X - m >= 0 && X + m <= w - 1 && Y - m >= 0 && Y + m <= h - 1) {
-                    const int at = atomicAdd(&n_fin, 1);
-                    if (at < SEL_FEW) cand[at] = (unsigned short)(y * SEL_TX + x + c);
-                }
+            const int e = tid + k * SEL_THREADS, Y = min(y0 + e / (SEL_TX / 4), h - 1);
+            own[k] = __ldg(reinterpret_cast<const float4*>(R + (long)Y * pitch + min(x0 + 4 * (e % (SEL_TX / 4)), (w - 1) & ~3)));
+        }
+        if (wid == 0) {
+            const int cx0 = sel_cell(x0, gx, w), ncx = sel_cell(min(x0 + SEL_TX, w) - 1, gx, w) - cx0 + 1;
+            const int cy0 = sel_cell(y0, gy, h), ncy = sel_cell(min(y0 + SEL_TY, h) - 1, gy, h) - cy0 + 1;
+            float best = INF;
+            for (int i = lane; i < ncx * ncy; i += 32) {
+                const unsigned long long key = __ldcg(cell_key + (cy0 + i / ncx) * gx + cx0 + i % ncx);
+                const unsigned ord = (unsigned)(key >> 32);
+                best = fminf(best, key ? __uint_as_float((ord & 0x80000000u) ? ord ^ 0x80000000u : ~ord) : NEG);
             }
+            for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+            if (lane == 0) least = best;
         }
         __syncthreads();
-        if (n_fin == 0) return;
+        const float lst = least;
+        few = lst > NEG;
+        if (few) {
+#pragma unroll
+            for (int k = 0; k < NOWN; k++) {
+                if (!(fmaxf(fmaxf(own[k].x, own[k].y), fmaxf(own[k].z, own[k].w)) >= lst)) continue;
+                const int e = tid + k * SEL_THREADS, y = e / (SEL_TX / 4), x = 4 * (e % (SEL_TX / 4)), Y = y0 + y;
+                const float v[4] = {own[k].x, own[k].y, own[k].z, own[k].w};
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const int X = x0 + x + c;
+                    if (v[c] >= lst && v[c] < max_peak && v[c] < INF && X - m >= 0 && X + m <= w - 1 && Y - m >= 0 && Y + m <= h - 1) {
+                        const int at = atomicAdd(&n_fin, 1);
+                        if (at < SEL_FEW) cand[at] = (unsigned short)(y * SEL_TX + x + c);
+                    }
+                }
+            }
+            __syncthreads();
+            if (n_fin == 0) return;
+        }
     }
     const bool direct = few && n_fin <= SEL_FEW;                 // the same for the whole CTA
     // 1. stage R in 16-byte chunks; XS is a multiple of 4, so a chunk is inside or
@@ -2013,16 +2019,18 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) select_tile_kernel(const float
 
 template <int QR>
 int launch_select_tile(const float* ref, const uint8_t* flags, const argus_shape& shape, int grid_x, int grid_y,
-                       int m, float max_peak, int iso, float iso_frac, unsigned long long* keys, cudaStream_t st) {
+                       int m, float max_peak, int iso, float iso_frac, int num_sms, unsigned long long* keys,
+                       cudaStream_t st) {
     const size_t smem = select_tile_smem(iso);
     if (cudaFuncSetAttribute(select_tile_kernel<QR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return ARGUS_ERR_CUDA;
     const SelOrder o = sel_order(shape.w, shape.h, grid_x, grid_y);
-    const long tiles = (long)o.sx * o.sy * o.nx * o.ny;
+    const long tiles = (long)o.sx * o.sy * o.nx * o.ny;      // with those that lie outside the frame
+    const long inside = (long)((shape.w + SEL_TX - 1) / SEL_TX) * ((shape.h + SEL_TY - 1) / SEL_TY);
     select_tile_kernel<QR><<<(unsigned)tiles, SEL_THREADS, smem, st>>>(ref, flags, shape.pitch, shape.w, shape.h,
                                                                        grid_x, grid_y, m, max_peak, iso, iso_frac,
-                                                                       keys);
+                                                                       inside > (long)(2 * SEL_ROUNDS * num_sms), keys);
     argus_count_launch(1);
     return ARGUS_OK;
 }
@@ -2356,10 +2364,10 @@ extern "C" int argus_select_stamps(argus_ctx* ctx, const float* ref, const uint8
     if (blocks > (long)ctx->num_sms * 16) blocks = (long)ctx->num_sms * 16;
     if (iso <= SEL_MAX_ISO) {
         const int m = stamp / 2 + khalf;
-        rc = iso == 0   ? launch_select_tile<0>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->cell_key, st)
-             : iso == 1 ? launch_select_tile<1>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->cell_key, st)
-             : iso == 2 ? launch_select_tile<2>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->cell_key, st)
-                        : launch_select_tile<3>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->cell_key, st);
+        rc = iso == 0   ? launch_select_tile<0>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->num_sms, ctx->cell_key, st)
+             : iso == 1 ? launch_select_tile<1>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->num_sms, ctx->cell_key, st)
+             : iso == 2 ? launch_select_tile<2>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->num_sms, ctx->cell_key, st)
+                        : launch_select_tile<3>(ref, flags, shape, grid_x, grid_y, m, max_peak, iso, iso_frac, ctx->num_sms, ctx->cell_key, st);
         if (rc) return rc;
     } else {
         uint8_t* lmax = reinterpret_cast<uint8_t*>(ctx->label);   // the label scratch, one byte per pixel

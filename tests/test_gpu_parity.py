@@ -422,6 +422,36 @@ def test_select_stamps_of_many_tiles(gx, gy, iso, iso_frac, max_peak):
         B.argus_destroy(ctx)
 
 
+@pytest.mark.parametrize("more", [0, 1])
+@pytest.mark.parametrize("gx,gy,iso", [(4, 3, 10), (1, 1, 3), (40, 19, 0)])
+def test_select_stamps_on_either_side_of_the_early_end(gx, gy, iso, more):
+    """Frames of the most tiles whose kernel tests every pixel, and of one row of tiles more, whose later
+    tiles end early: the same stamps as the per-pixel kernel's."""
+    w = 128 * 40 - 3
+    h = 64 * (int(2.5 * 2 * torch.cuda.get_device_properties(0).multi_processor_count) // 40 + more) - 1
+    rng = np.random.default_rng(gx + iso)
+    R = np.rint(rng.normal(300, 20, (h, w))).astype(np.float32)
+    y, x = rng.integers(0, h, 3000), rng.integers(0, w, 3000)
+    R[y, x] = np.rint(rng.uniform(0, 4e4, 3000) / 500) * 500
+    R[rng.random((h, w)) < 1e-5] = np.nan
+    fl = (rng.random((h, w)) < 2e-4).astype(np.uint8)
+    dR, dfl, shape = dev_pitched(R), dev_pitched(fl), B.argus_shape(w, h, pitch_for(w))
+    ctx = ctx_for(w, h)
+    try:
+        out = []
+        for f in (lambda *a: B.argus_select_stamps(ctx, *a), B.argus_select_stamps_noalloc):
+            cen = torch.full((gx * gy, 2), -1, dtype=torch.int32, device="cuda")
+            ns = torch.zeros(4, dtype=torch.int32, device="cuda")
+            f(dR, dfl, shape, gx, gy, 21, 5, 3e4, iso, 0.1, cen, ns)
+            torch.cuda.synchronize()
+            out.append((int(ns[0].item()), cen))
+        n = out[0][0]
+        assert n == out[1][0] and n > 0
+        assert torch.equal(out[0][1][:n], out[1][1][:n])
+    finally:
+        B.argus_destroy(ctx)
+
+
 # --------------------------------------------------------------------------- fit + expand
 def _fit_field(w, h, seed, sdeg):
     cat = synth.star_catalog(w * h // 80, w, h, seed=seed, flux_min=1e2, flux_max=1e6)
