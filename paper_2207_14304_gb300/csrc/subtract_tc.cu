@@ -83,6 +83,11 @@ namespace {
 using namespace argus_sub;
 
 constexpr int TCX = 128;                     // output columns per CTA (MMA M)
+// source rows per block: the variance's narrow MMAs leave the tensor pipe idle, so its
+// blocks are larger (fewer barrier rounds per row); the difference image's MMA width
+// grows with G (N = (KS - 1 + G) NK), so it keeps four
+template <bool VAR>
+__host__ __device__ constexpr int gsz() { return VAR ? 8 : 4; }
 // Output rows per band, chosen per call.  A CTA is held for the longest share of bands
 // any SM gets, ceil(bands / CTAs) of them, and a band costs its rows, the 2r halo rows and
 // a start (BAND_COST rows' worth): small frames want bands enough for every SM, large ones
@@ -97,6 +102,8 @@ constexpr int TCX = 128;                     // output columns per CTA (MMA M)
 constexpr int BAND_MIN = 16, BAND_COST = 16;
 template <bool VAR>
 inline int band_rows(int w, int h, int r, int ctas) {
+    constexpr int G = gsz<VAR>();
+    static_assert(!VAR || (BAND_MIN % G == 0 && VAR_TILE % BAND_MIN == 0), "bands start on block boundaries and divide a tile");
     const int gx = (w + TCX - 1) / TCX;
     int best = VAR ? VAR_TILE : 256;
     long cost = -1;
@@ -111,15 +118,10 @@ inline int band_rows(int w, int h, int r, int ctas) {
         for (int rows = VAR_TILE; rows >= BAND_MIN; rows /= 2) consider(rows);
     } else {
         const int most = (h + BAND_MIN - 1) / BAND_MIN;
-        for (int n = most < 256 ? most : 256; n >= 1; n--) consider(((h + n - 1) / n + 3) / 4 * 4);
+        for (int n = most < 256 ? most : 256; n >= 1; n--) consider(((h + n - 1) / n + G - 1) / G * G);
     }
     return best;
 }
-// source rows per block: the variance's narrow MMAs leave the tensor pipe idle, so its
-// blocks are larger (fewer barrier rounds per row); the difference image's MMA width
-// grows with G (N = (KS - 1 + G) NK), so it keeps four
-template <bool VAR>
-__host__ __device__ constexpr int gsz() { return VAR ? 8 : 4; }
 // blocks staged ahead (24 source rows either way) and staging slots per warp (> LA)
 template <bool VAR>
 __host__ __device__ constexpr int lahead() { return VAR ? 3 : 6; }
@@ -257,7 +259,6 @@ __global__ void __launch_bounds__(TC_THREADS, VAR ? 2 : 1)
     constexpr int P = VAR ? 1 : 3;               // products per K slice: hi*hi (+ hi*lo + lo*hi)
     static_assert(!VAR || NK == 1, "the variance convolution has one term");
     static_assert(!VAR || TCX == VAR_TILE, "one variance tile per strip");
-    static_assert(BAND_MIN % G == 0 && VAR_TILE % BAND_MIN == 0, "bands start on block boundaries");
     float* outp = VAR ? a.diff_var : a.diff;
     constexpr int R = (KS - 1) / 2;
     constexpr int SOFF = (4 - R % 4) % 4;        // wsrc[.][SOFF + c] = R(x0 - R + c); x0 - R - SOFF is a multiple of 4

@@ -157,3 +157,14 @@ def psf_matching_field(ks, W, H, sig_ref=1.2, s0=1.3, s1=0.9, n=25):
     A = _terms(X.ravel(), Y.ravel(), 2)
     coef, *_ = np.linalg.lstsq(A, G.reshape(n * n, -1), rcond=None)
     return coef.reshape(6, ks, ks)
+
+
+def band_rows(w, h, r, sms, variance):
+    """Output rows of a band as the subtraction chooses them (csrc/subtract_tc.cu, band_rows): the least of
+    rounds of bands over the CTAs times a band's rows, halo rows and start."""
+    ctas, gx = (2 if variance else 1) * sms, -(-w // 128)
+    if variance:
+        rows = [128, 64, 32, 16]
+    else:
+        rows = [-(--(-h // n) // 4) * 4 for n in range(min(-(-h // 16), 256), 0, -1)]
+    return min(rows, key=lambda b: -(-(gx * -(-h // b)) // ctas) * (b + 2 * r + 16))

@@ -704,3 +704,36 @@ def test_subtract_does_not_depend_on_bands(ora, w, h, ks, deg):
         assert_rel(Dg, Do, scale, 1e-4, "D")
     finally:
         B.argus_destroy(ctx)
+
+
+@pytest.mark.parametrize("w,h,ks,deg", [(4000, 700, 21, 2), (9576, 300, 11, 1)])
+def test_subtract_of_other_bands_is_the_same(w, h, ks, deg):
+    """A frame and the frame without its first 128 rows, at heights whose bands differ for the difference
+    and for the variance: the same bits away from the cut."""
+    from tests.gpu_helpers import band_rows
+    rng = np.random.default_rng(w + h)
+    nk, r, top = (deg + 1) * (deg + 2) // 2, ks // 2, 128
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for v in (False, True):
+        assert band_rows(w, h, r, sms, v) != band_rows(w, h - top, r, sms, v)
+    I, R = (rng.normal(300, 20, (h, w)).astype(np.float32) for _ in range(2))
+    V, Vr = (rng.uniform(200, 400, (h, w)).astype(np.float32) for _ in range(2))
+    fl = (rng.random((h, w)) < 0.01).astype(np.uint8)
+    K = (rng.normal(0, 1, (nk, ks, ks)) / ks ** 2).astype(np.float32)
+    pitch = pitch_for(w)
+    dI, dV, dR, dVr, dfl = (dev_pitched(a) for a in (I, V, R, Vr, fl))
+    dK, dbg = torch.from_numpy(K.reshape(-1)).cuda(), torch.from_numpy(rng.normal(0, 2, nk)).cuda()
+    ctx = ctx_for(w, h)
+    try:
+        out = []
+        for y0 in (0, top):
+            D, VD = (torch.zeros((h - y0, pitch), device="cuda") for _ in range(2))
+            B.argus_subtract(ctx, dI[y0:], dV[y0:], dR[y0:], dVr[y0:], dfl[y0:], B.argus_shape(w, h - y0, pitch), w, h, 0,
+                             y0, ks, deg, dK, deg, dbg, D, VD)
+            torch.cuda.synchronize()
+            assert B.argus_sync_status(ctx) == 0
+            out.append((D, VD))
+        for a, b in zip(*out):
+            assert a.any() and torch.equal(a[top + r:], b[r:])
+    finally:
+        B.argus_destroy(ctx)

@@ -59,3 +59,21 @@ def test_coadd_shifts_stay_in_range(driver, size):
     assert (np.abs(first) <= size + 32).all()
     span = np.abs(first[:, None] - first[None, :])
     np.testing.assert_array_equal(fits, ((span + 32) * 9 <= 512) & ((span + 9) * 32 <= 512))
+
+
+# --------------------------------------------------------------------------- subtraction
+def test_subtraction_bands(driver):
+    """Bands start on block boundaries (whole blocks of 4 and 8 source rows), a variance band divides a
+    128-row tile, and the choice is that of tests/gpu_helpers.band_rows."""
+    from tests.gpu_helpers import band_rows
+    exe = driver("host_bands")
+    rng = np.random.default_rng(3)
+    w = np.exp(rng.uniform(0, np.log(20000), 400)).astype(np.int32)
+    h = np.exp(rng.uniform(0, np.log(20000), 400)).astype(np.int32)
+    c = np.stack([w, h, rng.choice([5, 10], 400), rng.choice([1, 16, 148, 152, 160], 400)], 1).astype(np.int32)
+    c.tofile(exe.parent / "bands.bin")
+    _run(exe, "bands.bin", "bands.out")
+    rows = np.fromfile(exe.parent / "bands.out", np.int32).reshape(-1, 2)
+    assert (rows > 0).all() and (rows[:, 0] % 4 == 0).all() and np.isin(rows[:, 1], [16, 32, 64, 128]).all()
+    want = [[band_rows(*map(int, q), v) for v in (False, True)] for q in c]
+    np.testing.assert_array_equal(rows, want)
