@@ -541,6 +541,20 @@ void launch_box_medians(const BgArgs& a, cudaStream_t s) {
     box_median_kernel<NPL><<<a.nx * a.ny, BOX_THREADS, 0, s>>>(a);
 }
 
+// Where a call's scratch lies (bytes from its start): the raw mesh first, then the fill
+// value, the mesh in FP32 and the count of cells to fill.
+struct BgScratch {
+    size_t fill, meshf, missing, bytes;
+};
+__host__ inline BgScratch bg_scratch(size_t ncell) {
+    BgScratch s;
+    s.fill = ncell * sizeof(double);
+    s.meshf = s.fill + sizeof(double);
+    s.missing = s.meshf + ncell * sizeof(float);
+    s.bytes = s.missing + sizeof(int);
+    return s;
+}
+
 }  // namespace
 
 extern "C" int argus_background(argus_ctx* ctx, const float* img, const uint8_t* flags, argus_shape shape,
@@ -554,18 +568,20 @@ extern "C" int argus_background(argus_ctx* ctx, const float* img, const uint8_t*
         ((uintptr_t)mesh & 7u))
         return ARGUS_ERR_ALIGN;
     const int nx = (shape.w + box - 1) / box, ny = (shape.h + box - 1) / box;
-    if (ny > 65535 || ((size_t)nx * ny + 1) * sizeof(double) > ctx->max_pixels * sizeof(int)) return ARGUS_ERR_ARG;
+    // scratch in the detection label buffer: a frame that fits the context leaves room (pitch >= 8 nx and
+    // h >= ny, so at least 32 bytes for each box's 12)
+    const BgScratch sc = bg_scratch((size_t)nx * ny);
+    if (ny > 65535 || sc.bytes > ctx->max_pixels * sizeof(int)) return ARGUS_ERR_ARG;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return ARGUS_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     BgArgs a;
     a.img = img; a.flags = flags; a.mesh = mesh; a.map = map; a.pitch = shape.pitch;
     a.w = shape.w; a.h = shape.h; a.box = box; a.filt = filt; a.nx = nx; a.ny = ny; a.min_frac = min_frac;
-    // scratch in the detection label buffer: the raw mesh, the fill value, the mesh in FP32 and
-    // the count of cells to fill, 12 bytes per box and 12 (max_pixels ints are 256 bytes per 8 x 8 box)
-    a.raw = reinterpret_cast<double*>(ctx->label);
-    a.fill = a.raw + (long)nx * ny;
-    a.meshf = reinterpret_cast<float*>(a.fill + 1);
-    a.missing = reinterpret_cast<int*>(a.meshf + (long)nx * ny);
+    char* scratch = reinterpret_cast<char*>(ctx->label);
+    a.raw = reinterpret_cast<double*>(scratch);
+    a.fill = reinterpret_cast<double*>(scratch + sc.fill);
+    a.meshf = reinterpret_cast<float*>(scratch + sc.meshf);
+    a.missing = reinterpret_cast<int*>(scratch + sc.missing);
     if (cudaMemsetAsync(a.missing, 0, sizeof(int), s) != cudaSuccess) return ARGUS_ERR_CUDA;
     const int npl = (box * box + BOX_THREADS - 1) / BOX_THREADS;   // keys per thread: the smallest compiled bound
     if (npl <= 2) launch_box_medians<2>(a, s);

@@ -77,3 +77,17 @@ def test_subtraction_bands(driver):
     assert (rows > 0).all() and (rows[:, 0] % 4 == 0).all() and np.isin(rows[:, 1], [16, 32, 64, 128]).all()
     want = [[band_rows(*map(int, q), v) for v in (False, True)] for q in c]
     np.testing.assert_array_equal(rows, want)
+
+
+# --------------------------------------------------------------------------- background map
+def test_background_scratch_holds_every_part(driver):
+    """The parts of a call's scratch lie apart and aligned, and a frame's own pixels (an int each, a pitch
+    of a multiple of 16) leave room for them at the smallest box and the most ragged sizes."""
+    sizes = [(w, h) for w in (1, 7, 8, 9, 16, 17, 130, 9576) for h in (1, 8, 9, 65, 6388)]
+    cells = [-(-w // 8) * -(-h // 8) for w, h in sizes]
+    out = subprocess.check_output([str(driver("host_bg_scratch")), *map(str, cells)]).decode().split("\n")
+    for (w, h), n, line in zip(sizes, cells, out):
+        fill, meshf, missing, size = map(int, line.split())
+        parts = [(0, 8 * n, 8), (fill, 8, 8), (meshf, 4 * n, 4), (missing, 4, 4)]     # start, bytes, alignment
+        assert all(a + b <= c for (a, b, _), (c, _, _) in zip(parts, parts[1:]))
+        assert all(a % k == 0 for a, _, k in parts) and missing + 4 <= size <= 4 * h * (-(-w // 16) * 16)
