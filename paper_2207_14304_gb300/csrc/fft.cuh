@@ -3,8 +3,9 @@
 // e^{-2 pi i m / T} built in double precision on the host.  Forward transforms
 // are unnormalised, inverse transforms are unscaled (the caller divides by T^2),
 // as in numpy.  The real type is float (image data) or double (PSF transforms).
-// The first half states the butterflies and a pass over a sequence in memory
-// (what the CPU tests run); the second half is the register form the kernels run.
+// The first half states the butterflies and a pass over a sequence in memory (the form
+// of whole transforms on the CPU); the second half is the register form the kernels
+// run, whose steps and lane maps are host-callable too.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -156,53 +157,77 @@ template <int T> struct TwReg {
 #pragma unroll
         for (int i = 0; i < Reg<T>::NTW; i++) w[i] = __ldg(tab + tw_index<T>(i, lane));
     }
-    __device__ __forceinline__ float2 get(int i) const { return w[i]; }
+    FFT_HD float2 get(int i) const { return w[i]; }
 };
 template <int T> struct TwTab {
     const double2* tab;
     int lane;
-    __device__ __forceinline__ double2 get(int i) const { return __ldg(tab + tw_index<T>(i, lane)); }
+    FFT_HD double2 get(int i) const {
+#ifdef __CUDA_ARCH__
+        return __ldg(tab + tw_index<T>(i, lane));
+#else
+        return tab[tw_index<T>(i, lane)];
+#endif
+    }
 };
 
-// Lane values of a pass of radix RAD with Ns points done, to the next pass's
-// lane values; ST the element stride of the sequence in shared memory.  FEW: only
-// values 0, 1, 6 and 7 are used next.
-template <int T, int RAD, int Ns, int ST, bool FEW = false, typename C>
+// Where value i of a lane goes in the padded row between pass STEP and the next (passes are
+// counted from 0; the first two are of radix 8, then 8 or 4): butterfly j's output r to
+// (j / Ns) Ns RAD + j mod Ns + r Ns.
+template <int T, int STEP> FFT_HD int cross_to(int lane, int i) {
+    constexpr int RAD = STEP < 2 ? 8 : 4, Ns = STEP == 0 ? 1 : (STEP == 1 ? 8 : 64), NB = 8 / RAD;
+    const int j = lane + i % NB * (T / 8);
+    return pad((j / Ns) * Ns * RAD + (j & (Ns - 1)) + i / NB * Ns);
+}
+
+// Lane values of pass STEP to the next pass's; ST the element stride of the sequence in
+// shared memory.  FEW: only values 0, 1, 6 and 7 are used next.
+template <int T, int STEP, int ST, bool FEW = false, typename C>
 __device__ __forceinline__ void cross(C (&v)[8], C*& s0, C*& s1, int lane) {
-    constexpr int L = T / 8, NB = 8 / RAD;
 #pragma unroll
-    for (int b = 0; b < NB; b++) {
-        const int j = lane + b * L;
-        const int d = (j / Ns) * Ns * RAD + (j & (Ns - 1));
-#pragma unroll
-        for (int r = 0; r < RAD; r++) {
-            const int p = d + r * Ns;
-            s0[pad(p) * ST] = v[b + NB * r];
-        }
-    }
+    for (int i = 0; i < 8; i++) s0[cross_to<T, STEP>(lane, i) * ST] = v[i];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 8; m++) {
         if (FEW && m >= 2 && m < 6) continue;
-        const int p = lane + m * L;
-        v[m] = s0[pad(p) * ST];
+        v[m] = s0[pad(lane + m * (T / 8)) * ST];
     }
     C* t = s0;
     s0 = s1;
     s1 = t;
 }
 
-template <int S, typename C> __device__ __forceinline__ C tmul(C v, C w) { return cmul(v, S < 0 ? w : cconj(w)); }
+template <int S, typename C> FFT_HD C tmul(C v, C w) { return cmul(v, S < 0 ? w : cconj(w)); }
 
 // One radix-4 pass: butterflies b = 0, 1 on v[b], v[b + 2], v[b + 4], v[b + 6],
 // twiddle slots i0 + (PER ? 3 b : 0) + r - 1.
 template <int S, bool PER, typename C, typename TW>
-__device__ __forceinline__ void radix4(C (&v)[8], const TW& tw, int i0) {
+FFT_HD void radix4(C (&v)[8], const TW& tw, int i0) {
 #pragma unroll
     for (int b = 0; b < 2; b++) {
 #pragma unroll
         for (int r = 1; r < 4; r++) v[b + 2 * r] = tmul<S>(v[b + 2 * r], tw.get(i0 + (PER ? 3 * b : 0) + r - 1));
         dft4<S>(v[b], v[b + 2], v[b + 4], v[b + 6]);
+    }
+}
+
+// The butterflies of pass STEP > 0 on a lane's values.  FEW (pass 1): values 2 .. 5 are zero.
+template <int T, int S, int STEP, bool FEW = false, typename C, typename TW>
+FFT_HD void pass(C (&v)[8], const TW& tw) {
+    if constexpr (STEP == 1) {
+#pragma unroll
+        for (int r = 1; r < 8; r++)
+            if (!FEW || r < 2 || r > 5) v[r] = tmul<S>(v[r], tw.get(r - 1));
+        if (FEW) dft8_few<S>(v);
+        else dft8<S>(v);
+    } else if constexpr (T == 512) {
+#pragma unroll
+        for (int r = 1; r < 8; r++) v[r] = tmul<S>(v[r], tw.get(6 + r));
+        dft8<S>(v);
+    } else if constexpr (T == 256) {
+        radix4<S, true>(v, tw, 7);
+    } else {
+        radix4<S, STEP == 3>(v, tw, STEP == 3 ? 10 : 7);
     }
 }
 
@@ -212,23 +237,13 @@ __device__ __forceinline__ void radix4(C (&v)[8], const TW& tw, int i0) {
 // second pass meets as its elements 0, 1, 6 and 7.
 template <int T, int S, int ST, bool FEW = false, typename C, typename TW>
 __device__ __forceinline__ void fft_tail(C (&v)[8], const TW& tw, C*& s0, C*& s1, int lane) {
-    cross<T, 8, 1, ST, FEW>(v, s0, s1, lane);
-#pragma unroll
-    for (int r = 1; r < 8; r++)
-        if (!FEW || r < 2 || r > 5) v[r] = tmul<S>(v[r], tw.get(r - 1));
-    if (FEW) dft8_few<S>(v);
-    else dft8<S>(v);
-    cross<T, 8, 8, ST>(v, s0, s1, lane);
-    if constexpr (T == 512) {
-#pragma unroll
-        for (int r = 1; r < 8; r++) v[r] = tmul<S>(v[r], tw.get(6 + r));
-        dft8<S>(v);
-    } else if constexpr (T == 256) {
-        radix4<S, true>(v, tw, 7);
-    } else {
-        radix4<S, false>(v, tw, 7);
-        cross<T, 4, 64, ST>(v, s0, s1, lane);
-        radix4<S, true>(v, tw, 10);
+    cross<T, 0, ST, FEW>(v, s0, s1, lane);
+    pass<T, S, 1, FEW>(v, tw);
+    cross<T, 1, ST>(v, s0, s1, lane);
+    pass<T, S, 2>(v, tw);
+    if constexpr (T == 1024) {
+        cross<T, 2, ST>(v, s0, s1, lane);
+        pass<T, S, 3>(v, tw);
     }
 }
 

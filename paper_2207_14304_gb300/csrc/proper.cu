@@ -227,12 +227,13 @@ struct PsfArgs {
     double2* rows;          // [tile][pair][2][ps][T / 2 + 1]
 };
 
-// First pass of a sequence with values only at positions lane (v0, has0) and
-// lane + 7 T/8 (v7, has7).  Most warps hold values of one kind at most, which need no sums
-// (column transforms of 31 x 31 stamps in 247 tiles of 512: 2.45 -> 2.25 ms).
-__device__ __forceinline__ void psf_first(double2 (&v)[8], double2 v0, double2 v7, bool has0, bool has7) {
+// First pass of a sequence with values only at positions lane (v0; none in any lane of the
+// warp unless any0) and lane + 7 T/8 (v7, any7).  Most warps hold values of one kind at
+// most, which need no sums (column transforms of 31 x 31 stamps in 216 tiles of 512: 2.45 ->
+// 2.25 ms).
+__host__ __device__ __forceinline__ void psf_first(double2 (&v)[8], double2 v0, double2 v7, bool any0, bool any7) {
     const double r = 0.70710678118654752440;
-    if (!__any_sync(0xffffffffu, has7)) {
+    if (!any7) {
 #pragma unroll
         for (int m = 0; m < 8; m++) v[m] = v0;
         return;
@@ -240,7 +241,7 @@ __device__ __forceinline__ void psf_first(double2 (&v)[8], double2 v0, double2 v
     const double2 d1 = make_double2(r * (v7.x - v7.y), r * (v7.x + v7.y));    // v7 e^{i pi / 4}
     const double2 d3 = make_double2(-d1.y, d1.x);                             // v7 e^{3 i pi / 4}
     const double2 d2 = make_double2(-v7.y, v7.x);
-    if (!__any_sync(0xffffffffu, has0)) {
+    if (!any0) {
         v[0] = v7; v[4] = make_double2(-v7.x, -v7.y);
         v[1] = d1; v[5] = make_double2(-d1.x, -d1.y);
         v[2] = d2; v[6] = make_double2(-d2.x, -d2.y);
@@ -253,15 +254,24 @@ __device__ __forceinline__ void psf_first(double2 (&v)[8], double2 v0, double2 v
     v[3] = fft::cadd(v0, d3); v[7] = fft::csub(v0, d3);
 }
 
+// The stamp pixels at positions lane and lane - T/8 of a sequence, its centre at 0; none where
+// not in [0, ps).
+template <int T> __host__ __device__ __forceinline__ int psf_at(int ps, int lane, bool wrapped) {
+    return ps / 2 + lane - (wrapped ? T / 8 : 0);
+}
+
 constexpr int PSEQ = 2;       // FP64 sequences per CTA
 
 // The other passes of a stamp's sequence.  A stamp of half-side below T/32 leaves half of
 // the second pass's values zero too: FP64 arithmetic bounds these kernels, and its radix-8
 // butterflies then take 52 operations instead of 84 (column transforms of 31 x 31 stamps
-// in 247 tiles of 512: 2.87 -> 2.45 ms).
+// in 216 tiles of 512: 2.87 -> 2.45 ms).
+template <int T> __host__ __device__ __forceinline__ bool psf_few(int ps) {
+    return T == 1024 || ps / 2 < T / 32;                   // (a side is at most 63)
+}
 template <int T, int ST>
 __device__ __forceinline__ void psf_tail(double2 (&v)[8], int ps, const fft::TwTab<T>& tw, double2*& b0, double2*& b1, int lane) {
-    if (T == 1024 || ps / 2 < T / 32) fft::fft_tail<T, -1, ST, true>(v, tw, b0, b1, lane);   // a side is at most 63
+    if (psf_few<T>(ps)) fft::fft_tail<T, -1, ST, true>(v, tw, b0, b1, lane);
     else fft::fft_tail<T, -1, ST>(v, tw, b0, b1, lane);
 }
 
@@ -281,18 +291,17 @@ __global__ void __launch_bounds__(PSEQ * fft::Reg<T>::LANES) psf_rows_kernel(Psf
     const bool live = row < a.ps;
     const long o = t * a.tile_stride + p * a.pair_stride + (long)row * a.ps;
     const bool two = p < a.n_second;
-    const int hh = a.ps / 2;
+    const int q = psf_at<T>(a.ps, lane, false), u = psf_at<T>(a.ps, lane, true);
     double2 v0 = make_double2(0.0, 0.0), v7 = v0, v[8];
-    if (live && lane + hh < a.ps) {
-        v0.x = a.p0[o + lane + hh];
-        if (two) v0.y = a.p1[o + lane + hh];
+    if (live && q < a.ps) {
+        v0.x = a.p0[o + q];
+        if (two) v0.y = a.p1[o + q];
     }
-    const int u = hh - Rg::LANES + lane;                    // column of the stamp at position lane - T/8 < 0
     if (live && u >= 0) {
         v7.x = a.p0[o + u];
         if (two) v7.y = a.p1[o + u];
     }
-    psf_first(v, v0, v7, lane + hh < a.ps, u >= 0);
+    psf_first(v, v0, v7, __any_sync(0xffffffffu, q < a.ps), __any_sync(0xffffffffu, u >= 0));
     double2* b0 = sm + seq * Rg::PT;
     double2* b1 = sm + (PSEQ + seq) * Rg::PT;
     const fft::TwTab<T> tw{a.tw, lane};
@@ -315,12 +324,12 @@ __global__ void __launch_bounds__(PSEQ * fft::Reg<T>::LANES) psf_rows_kernel(Psf
 template <int T>
 __device__ __forceinline__ void psf_column(double2 (&v)[8], const double2* rows, int ps, int kx, const fft::TwTab<T>& tw,
                                            double2*& b0, double2*& b1, int lane) {
-    constexpr int HW = T / 2 + 1, L = T / 8;
-    const int hh = ps / 2, u = hh - L + lane;
+    constexpr int HW = T / 2 + 1;
+    const int q = psf_at<T>(ps, lane, false), u = psf_at<T>(ps, lane, true);
     double2 v0 = make_double2(0.0, 0.0), v7 = v0;
-    if (kx < HW && lane + hh < ps) v0 = rows[(long)(lane + hh) * HW + kx];
+    if (kx < HW && q < ps) v0 = rows[(long)q * HW + kx];
     if (kx < HW && u >= 0) v7 = rows[(long)u * HW + kx];
-    psf_first(v, v0, v7, lane + hh < ps, u >= 0);
+    psf_first(v, v0, v7, __any_sync(0xffffffffu, q < ps), __any_sync(0xffffffffu, u >= 0));
     psf_tail<T, PSEQ>(v, ps, tw, b0, b1, lane);
 }
 

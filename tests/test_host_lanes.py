@@ -91,3 +91,42 @@ def test_background_scratch_holds_every_part(driver):
         parts = [(0, 8 * n, 8), (fill, 8, 8), (meshf, 4 * n, 4), (missing, 4, 4)]     # start, bytes, alignment
         assert all(a + b <= c for (a, b, _), (c, _, _) in zip(parts, parts[1:]))
         assert all(a % k == 0 for a, _, k in parts) and missing + 4 <= size <= 4 * h * (-(-w // 16) * 16)
+
+
+# --------------------------------------------------------------------------- transforms
+@pytest.mark.parametrize("T", [256, 512, 1024])
+@pytest.mark.parametrize("dbl", [0, 1])
+def test_register_transforms_match_numpy(driver, T, dbl):
+    """The register passes, lane by lane, against numpy, at the bar of the whole transforms' test (a few
+    ulps times log2 of the points), and unit impulses at every position of a lane's eight values."""
+    exe = driver("host_fft_lanes")
+    rng = np.random.default_rng(T + dbl)
+    x = rng.normal(size=(40, T)) + 1j * rng.normal(size=(40, T))
+    x[8:] = np.eye(T)[(np.arange(32) * (T // 32) + np.arange(32) % 7) % T]
+    x = x.astype(np.complex128 if dbl else np.complex64)
+    x.tofile(exe.parent / "seq.bin")
+    for sign in (-1, 1):
+        _run(exe, "full", T, dbl, sign, "seq.bin", "seq.out")
+        y = np.fromfile(exe.parent / "seq.out", x.dtype).reshape(x.shape)
+        x64 = x.astype(np.complex128)
+        ref = np.fft.fft(x64) if sign < 0 else np.fft.ifft(x64) * T
+        err = (np.abs(y - ref).max(1) / np.abs(ref).max(1)).max()
+        assert err < 8 * (2.0 ** -53 if dbl else 2.0 ** -24) * np.log2(T), (sign, err)
+
+
+@pytest.mark.parametrize("T", [256, 512, 1024])
+@pytest.mark.parametrize("ps", [1, 3, 13, 15, 17, 31, 33, 63])
+def test_psf_transforms_leave_out_only_zeros(driver, T, ps):
+    """A stamp's sequence with its centre at position 0: the passes that leave out zeros against numpy, and
+    equal to the passes that don't (a value that is left out is NaN in the driver)."""
+    exe = driver("host_fft_lanes")
+    rng = np.random.default_rng(T + ps)
+    p = rng.normal(size=(5, ps))
+    p.tofile(exe.parent / "psf.bin")
+    _run(exe, "psf", T, ps, "psf.bin", "psf.out")
+    y, whole = np.fromfile(exe.parent / "psf.out", np.complex128).reshape(2, 5, T)
+    x = np.zeros((5, T))
+    x[:, (np.arange(ps) - ps // 2) % T] = p
+    ref = np.fft.fft(x)
+    assert np.abs(y - ref).max() < 8 * 2.0 ** -53 * np.log2(T) * np.abs(ref).max()
+    np.testing.assert_array_equal(y, whole)
