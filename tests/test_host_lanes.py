@@ -130,3 +130,20 @@ def test_psf_transforms_leave_out_only_zeros(driver, T, ps):
     ref = np.fft.fft(x)
     assert np.abs(y - ref).max() < 8 * 2.0 ** -53 * np.log2(T) * np.abs(ref).max()
     np.testing.assert_array_equal(y, whole)
+
+
+def test_coadd_cuts_fit_the_pool(driver):
+    """Every cut holds at least a pair of a tile, all pairs where a chunk has several tiles, no more than was
+    asked for, and stays inside the plan's pool."""
+    exe = driver("host_cut")
+    rng = np.random.default_rng(8)
+    n = 4000
+    most = np.exp(rng.uniform(0, np.log(400), n)).astype(np.int32)
+    c = np.stack([rng.choice([256, 512, 1024], n), most, 1 + (rng.random(n) * most).astype(np.int32), rng.integers(1, 33, n),
+                  rng.choice([1, 3, 31, 63], n), rng.integers(0, 2, n), rng.integers(0, 2, n)], 1).astype(np.int32)
+    c.tofile(exe.parent / "cuts.bin")
+    _run(exe, "cuts.bin", "cuts.out")
+    tiles, group, used, pool = np.fromfile(exe.parent / "cuts.out", np.int64).reshape(-1, 4).T
+    assert (group >= 1).all() and (tiles >= 1).all() and (tiles <= c[:, 2]).all() and (group <= c[:, 3]).all()
+    assert (group[tiles > 1] == c[tiles > 1, 3]).all()
+    assert (used <= pool).all()
