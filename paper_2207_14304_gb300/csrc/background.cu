@@ -216,6 +216,59 @@ __device__ __forceinline__ int pick_bin(const int* hist, int& k, int* sh) {
 // needed 200 of them and waited on its loads eight warps to an SM.
 constexpr int BOX_THREADS = 128, BOX_WARPS = BOX_THREADS / 32, CAREFUL = 10;
 
+// The bracket and its next thresholds, the same for every thread; host-callable, so a CPU
+// driver can run the same selection.
+constexpr unsigned BOX_NONE = 0xffffffffu;                 // above every valid key
+struct BoxBracket {
+    unsigned lo, hi;         // the ranks r1, r2 lie in (lo, hi], or at the cut
+    int clo, chi, r1, r2;    // ranks clo .. chi - 1 are in it
+    unsigned t, u;           // thresholds of the next pass, t <= u
+    bool split;              // r1 is the last key <= cut, r2 the first above
+    unsigned cut;
+    // of n valid keys; s0 <= s1 the first thresholds
+    __host__ __device__ __forceinline__ void init(int n, unsigned s0, unsigned s1) {
+        r1 = (n - 1) / 2;
+        r2 = n / 2;
+        lo = 0u;             // no valid key is 0 or above hi
+        hi = BOX_NONE - 1u;
+        clo = 0;
+        chi = n;
+        t = s0;
+        u = s1;
+        split = false;
+        cut = 0u;
+    }
+    __host__ __device__ __forceinline__ bool useful() const { return t > lo && t < hi && u > lo && u < hi; }
+    // the counts of keys <= t and <= u
+    __host__ __device__ __forceinline__ void narrow(int ct, int cu) {
+        if (ct <= r1) { lo = t; clo = ct; }
+        else if (ct > r2) { hi = t; chi = ct; }
+        else { split = true; cut = t; }
+        if (cu <= r1) { if (u > lo) { lo = u; clo = cu; } }
+        else if (cu > r2) { if (u < hi) { hi = u; chi = cu; } }
+        else { split = true; cut = u; }
+    }
+    __host__ __device__ __forceinline__ bool done() const { return split || chi - clo <= 32 || hi - lo == 1u; }
+    // thresholds after pass it
+    __host__ __device__ __forceinline__ void next(int it) {
+        const unsigned span = hi - lo;
+        if (it >= CAREFUL) {
+            t = u = lo + span / 2;
+        } else {
+            const float c = (float)(chi - clo), per = (float)span / c;
+            const float g = ((float)(r1 - clo) + 0.75f) * per, m = fmaxf(8.0f, 1.5f * sqrtf(c)) * per;
+            // (2^32 as a float at most: one below it at the most where the cast is asked for)
+            const float top = fminf((float)(span - 1u), 4294967040.0f);
+            t = lo + umin_(umax_(1u, (unsigned)fminf(fmaxf(g - m, 1.0f), top)), span - 1u);
+            u = lo + umin_(umax_(1u, (unsigned)fminf(g + m, top)), span - 1u);
+        }
+    }
+    // whether a key is left in the bracket
+    __host__ __device__ __forceinline__ bool holds(unsigned key) const { return key - lo - 1u < hi - lo; }
+    static __host__ __device__ __forceinline__ unsigned umin_(unsigned a, unsigned b) { return a < b ? a : b; }
+    static __host__ __device__ __forceinline__ unsigned umax_(unsigned a, unsigned b) { return a > b ? a : b; }
+};
+
 // The lanes' values in ascending order over the lanes (bitonic).
 __device__ __forceinline__ unsigned warp_sort(unsigned v, int lane) {
 #pragma unroll
@@ -279,7 +332,7 @@ __global__ void __launch_bounds__(BOX_THREADS) box_median_kernel(BgArgs a) {
 #pragma unroll
             for (int j = 0; j < LB; j++) {
                 const bool ok = (f[j] == 0u) & (fabsf(v[j]) <= 3.402823466e38f);     // finite
-                key[j0 + j] = ok ? key32(v[j]) : 0xffffffffu;
+                key[j0 + j] = ok ? key32(v[j]) : BOX_NONE;
                 nv += ok ? 1 : 0;
             }
         }
@@ -295,47 +348,27 @@ __global__ void __launch_bounds__(BOX_THREADS) box_median_kernel(BgArgs a) {
         if (tid == 0) a.raw[b] = __longlong_as_double(0x7ff8000000000000ll);     // NaN: no value
         return;
     }
-    const int r1 = (n - 1) / 2, r2 = n / 2;
-    unsigned lo = 0u, hi = 0xfffffffeu;                    // no valid key is 0 or above hi
-    int clo = 0, chi = n;
-    unsigned t = smp[0], u = smp[1];
-    bool split = false;
-    unsigned cut = 0u;                                     // split: r1 is the last key <= cut, r2 the first above
+    BoxBracket q;
+    q.init(n, smp[0], smp[1]);
     for (int it = 0;; it++) {                              // the same for every thread
-        if (t > lo && t < hi && u > lo && u < hi) {
+        if (q.useful()) {
             int c = 0, d = 0;
 #pragma unroll
             for (int j = 0; j < NPL; j++) {
-                c += key[j] <= t ? 1 : 0;
-                d += key[j] <= u ? 1 : 0;
+                c += key[j] <= q.t ? 1 : 0;
+                d += key[j] <= q.u ? 1 : 0;
             }
             const int2 s = box_sum2(c, d, part, slot);
-            if (s.x <= r1) { lo = t; clo = s.x; }
-            else if (s.x > r2) { hi = t; chi = s.x; }
-            else { split = true; cut = t; }
-            if (s.y <= r1) { if (u > lo) { lo = u; clo = s.y; } }
-            else if (s.y > r2) { if (u < hi) { hi = u; chi = s.y; } }
-            else { split = true; cut = u; }
+            q.narrow(s.x, s.y);
         }
-        if (split || chi - clo <= 32 || hi - lo == 1u) break;
-        const unsigned span = hi - lo;
-        if (it >= CAREFUL) {
-            t = u = lo + span / 2;
-        } else {
-            const float c = (float)(chi - clo), per = (float)span / c;
-            const float g = ((float)(r1 - clo) + 0.75f) * per, m = fmaxf(8.0f, 1.5f * sqrtf(c)) * per;
-            const float top = (float)(span - 1u);
-            t = lo + max(1u, (unsigned)fminf(fmaxf(g - m, 1.0f), top));
-            u = lo + max(1u, (unsigned)fminf(g + m, top));
-            t = min(t, hi - 1u);
-            u = min(u, hi - 1u);
-        }
+        if (q.done()) break;
+        q.next(it);
     }
-    if (split) {
-        unsigned m1 = 0u, m2 = 0xffffffffu;
+    if (q.split) {
+        unsigned m1 = 0u, m2 = BOX_NONE;
 #pragma unroll
         for (int j = 0; j < NPL; j++) {
-            if (key[j] <= cut) m1 = max(m1, key[j]);
+            if (key[j] <= q.cut) m1 = max(m1, key[j]);
             else m2 = min(m2, key[j]);
         }
         m1 = __reduce_max_sync(0xffffffffu, m1);
@@ -352,16 +385,16 @@ __global__ void __launch_bounds__(BOX_THREADS) box_median_kernel(BgArgs a) {
             }
             a.raw[b] = median_of_keys(m1, m2);
         }
-    } else if (hi - lo == 1u) {
-        if (tid == 0) a.raw[b] = median_of_keys(hi, hi);   // every key left is hi
+    } else if (q.hi - q.lo == 1u) {
+        if (tid == 0) a.raw[b] = median_of_keys(q.hi, q.hi);   // every key left is hi
     } else {
 #pragma unroll
         for (int j = 0; j < NPL; j++)
-            if (key[j] - lo - 1u < hi - lo) cand[atomicAdd(&at, 1)] = key[j];     // lo < key <= hi: at most 32
+            if (q.holds(key[j])) cand[atomicAdd(&at, 1)] = key[j];     // at most 32
         __syncthreads();
         if (warp == 0) {
-            const unsigned v = warp_sort(lane < at ? cand[lane] : 0xffffffffu, lane);
-            const unsigned k1 = __shfl_sync(0xffffffffu, v, r1 - clo), k2 = __shfl_sync(0xffffffffu, v, r2 - clo);
+            const unsigned v = warp_sort(lane < at ? cand[lane] : BOX_NONE, lane);
+            const unsigned k1 = __shfl_sync(0xffffffffu, v, q.r1 - q.clo), k2 = __shfl_sync(0xffffffffu, v, q.r2 - q.clo);
             if (lane == 0) a.raw[b] = median_of_keys(k1, k2);
         }
     }

@@ -147,3 +147,27 @@ def test_coadd_cuts_fit_the_pool(driver):
     assert (group >= 1).all() and (tiles >= 1).all() and (tiles <= c[:, 2]).all() and (group <= c[:, 3]).all()
     assert (group[tiles > 1] == c[tiles > 1, 3]).all()
     assert (used <= pool).all()
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 64, 2304, 4096])
+def test_box_selection_ends_at_the_median(driver, n):
+    """The bracketing selection's median equals numpy's exactly, on noise, ties, wide ranges, two values,
+    extremes of the type, denormals, signed zeros and boxes with invalid pixels, within the interpolated passes plus one
+    per bit of a key."""
+    exe = driver("host_box_median")
+    rng = np.random.default_rng(n)
+    big = np.finfo(np.float32).max
+    x = [rng.normal(300, 15, n), np.rint(rng.normal(5, 2, n)), np.full(n, 7.5), np.exp(rng.normal(0, 40, n)),
+         rng.choice([-1.0, 1.0], n), rng.choice([-big, big], n), rng.choice([0.0, -0.0, 1e-45, -1e-45], n), rng.choice([1e-40, -3.0], n),
+         np.where(rng.random(n) < 0.5, big, rng.normal(0, 1, n)), np.sort(rng.normal(0, 1, n)), -np.sort(-rng.normal(0, 1, n)),
+         np.r_[np.full(n // 2, -big), rng.normal(1e30, 1e28, n - n // 2)]]
+    x += [np.where(rng.random(n) < p, np.nan, rng.normal(300, 15, n)) for p in (0.01, 0.5, 0.97)]
+    with np.errstate(over="ignore"):
+        x = np.stack(x).astype(np.float32)                  # (the wide range reaches infinity, which is no valid pixel)
+    x[:, 0] = np.where(np.isnan(x[:, 0]), 1.0, x[:, 0])     # a valid pixel at least
+    x.tofile(exe.parent / "boxes.bin")
+    _run(exe, n, "boxes.bin", "boxes.out")
+    raw = (exe.parent / "boxes.out").read_bytes()
+    med, passes = np.frombuffer(raw, np.float64, len(x)), np.frombuffer(raw, np.int32, len(x), 8 * len(x))
+    np.testing.assert_array_equal(med, np.nanmedian(np.where(np.isfinite(x), x, np.nan).astype(np.float64), axis=1))
+    assert passes.max() <= 11 + 32
