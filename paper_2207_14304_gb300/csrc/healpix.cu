@@ -225,6 +225,11 @@ constexpr HpWeights hp_make_weights() {
 }
 __device__ const HpWeights hp_weights = hp_make_weights();
 
+// A column's coordinate at a node row from the node columns' (in units of 2^-HP_FRAC).
+__host__ __device__ __forceinline__ double hp_column(const double* w, double n0, double n1, double n2, double n3) {
+    return ((w[0] * n0 + w[1] * n1) + w[2] * n2) + w[3] * n3;
+}
+
 // Forward differences at row 0 (unit steps) of the cubic through v[] at the node
 // rows 0, 10, 21, 31: from its divided differences c1, c2, c3,
 // p(r) = v0 + c1 r + c2 r (r - 10) + c3 r (r - 10) (r - 21).
@@ -239,6 +244,20 @@ __host__ __device__ __forceinline__ void hp_differences(const double* v, long lo
     d[3] = (long long)(6.0 * c3);
 }
 
+// The differences q rows on from those at row 0.
+__host__ __device__ __forceinline__ void hp_advance(const long long* f, int q, long long* d) {
+    const int q2 = q * (q - 1) / 2, q3 = q * (q - 1) * (q - 2) / 6;
+    d[0] = f[0] + q * f[1] + q2 * f[2] + q3 * f[3];
+    d[1] = f[1] + q * f[2] + q2 * f[3];
+    d[2] = f[2] + q * f[3];
+    d[3] = f[3];
+}
+__host__ __device__ __forceinline__ void hp_step(long long* d) {
+    d[0] += d[1];
+    d[1] += d[2];
+    d[2] += d[3];
+}
+
 // a + t (b - a) with t = th + tl, a = ah + al, b = bh + bl as unevaluated pairs.
 struct F2p { float h, l; };
 __host__ __device__ __forceinline__ F2p hp_lerp(F2p a, F2p b, float th, float tl) {
@@ -248,6 +267,16 @@ __host__ __device__ __forceinline__ F2p hp_lerp(F2p a, F2p b, float th, float tl
     const float s = a.h + p, q = s - a.h;                  // s + r = a.h + p exactly
     const float r = (a.h - (s - q)) + (p - q) + (pl + a.l);
     return {s, r};
+}
+
+// The frame between the pixels q00 (x0, y0), q01 (x0 + 1, y0), q10, q11 at the fractions fx, fy
+// (fixed point; 24 + 20 bits as a pair).
+__host__ __device__ __forceinline__ float hp_fixed_bilinear(float q00, float q01, float q10, float q11, long long fx, long long fy) {
+    const float xh = (float)(int)(fx >> 20) * 0x1p-24f, xl = (float)(int)(fx & 0xfffff) * 0x1p-44f;
+    const float yh = (float)(int)(fy >> 20) * 0x1p-24f, yl = (float)(int)(fy & 0xfffff) * 0x1p-44f;
+    const F2p top = hp_lerp({q00, 0.0f}, {q01, 0.0f}, xh, xl), bot = hp_lerp({q10, 0.0f}, {q11, 0.0f}, xh, xl);
+    const F2p r = hp_lerp(top, bot, yh, yl);
+    return r.h + r.l;
 }
 
 __device__ __forceinline__ float hp_nan() { return __int_as_float(0x7fffffff); }
@@ -320,10 +349,8 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
         }
         if (tid < 2 * HP_PATCH) {                          // grp 0: x, grp 1: y
             double v[4];
-            for (int j = 0; j < 4; j++) {
-                v[j] = 0.0;
-                for (int i = 0; i < 4; i++) v[j] += hp_weights.w[col][i] * nd[hf][j][i][grp];
-            }
+            for (int j = 0; j < 4; j++)
+                v[j] = hp_column(hp_weights.w[col], nd[hf][j][0][grp], nd[hf][j][1][grp], nd[hf][j][2][grp], nd[hf][j][3][grp]);
             long long d[4];
             hp_differences(v, d);
             for (int i = 0; i < 4; i++) dif[grp][col][i] = d[i];
@@ -347,29 +374,15 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
         }
         __syncthreads();
         long long d[2][4];
-        {
-            const int q = grp * (HP_HALF / 4);             // first row: differences there from those at row 0
-            const int q2 = q * (q - 1) / 2, q3 = q * (q - 1) * (q - 2) / 6;
-#pragma unroll
-            for (int i = 0; i < 2; i++) {
-                const long long* f = dif[i][col];
-                d[i][0] = f[0] + q * f[1] + q2 * f[2] + q3 * f[3];
-                d[i][1] = f[1] + q * f[2] + q2 * f[3];
-                d[i][2] = f[2] + q * f[3];
-                d[i][3] = f[3];
-            }
-        }
+        hp_advance(dif[0][col], grp * (HP_HALF / 4), d[0]);        // the group's first row
+        hp_advance(dif[1][col], grp * (HP_HALF / 4), d[1]);
         const long long xmax = a.xmax, ymax = a.ymax;
         long e = (long)(r0 + grp * (HP_HALF / 4)) * m + c0 + col;
 #pragma unroll 2
         for (int i = 0; i < HP_HALF / 4; i++, e += m) {
             const long long X = d[0][0], Y = d[1][0];
-#pragma unroll
-            for (int j = 0; j < 2; j++) {
-                d[j][0] += d[j][1];
-                d[j][1] += d[j][2];
-                d[j][2] += d[j][3];
-            }
+            hp_step(d[0]);
+            hp_step(d[1]);
             float v = 0.0f;
             bool ok = X >= 0 && Y >= 0 && X <= xmax && Y <= ymax;
             if (ok) {
@@ -391,12 +404,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
                     q10 = hp_fetch(a, x0, y0 + sy);
                     q11 = hp_fetch(a, x0 + sx, y0 + sy);
                 }
-                // the fraction as 24 + 20 bits
-                const float xh = (float)(int)(fx >> 20) * 0x1p-24f, xl = (float)(int)(fx & 0xfffff) * 0x1p-44f;
-                const float yh = (float)(int)(fy >> 20) * 0x1p-24f, yl = (float)(int)(fy & 0xfffff) * 0x1p-44f;
-                const F2p top = hp_lerp({q00, 0.0f}, {q01, 0.0f}, xh, xl), bot = hp_lerp({q10, 0.0f}, {q11, 0.0f}, xh, xl);
-                const F2p r = hp_lerp(top, bot, yh, yl);
-                v = r.h + r.l;
+                v = hp_fixed_bilinear(q00, q01, q10, q11, fx, fy);
                 ok = q00 == q00 && q01 == q01 && q10 == q10 && q11 == q11;
                 if (ok && !isfinite(v))                    // differences beyond FP32: lerps in FP64
                     hp_bilinear(a, (double)X * 0x1p-44, (double)Y * 0x1p-44, v);

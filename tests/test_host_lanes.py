@@ -171,3 +171,46 @@ def test_box_selection_ends_at_the_median(driver, n):
     med, passes = np.frombuffer(raw, np.float64, len(x)), np.frombuffer(raw, np.int32, len(x), 8 * len(x))
     np.testing.assert_array_equal(med, np.nanmedian(np.where(np.isfinite(x), x, np.nan).astype(np.float64), axis=1))
     assert passes.max() <= 11 + 32
+
+
+# --------------------------------------------------------------------------- HEALPix patches
+@pytest.mark.parametrize("nside_seg,k,delta0,rot", [(256, 6, 0.3, 0.8), (256, 9, -0.2, -2.0), (64, 7, 0.0, 0.0), (128, 8, 0.7, 0.3)])
+def test_patch_positions_follow_the_exact_ones(driver, nside_seg, k, delta0, rot):
+    """The fixed-point positions of halves in the belt against the exact path's.  A cubic through the
+    columns 0, 21, 42, 63 is off by at most 21^4 / 24 times the fourth derivative, which for a map of
+    one frame pixel per image pixel is F delta^3 (delta the pixel's angle, F <= 20 within 10 degrees of the tangent
+    point); the rows' nodes are half as far apart; the differences and the fixed point add less than 1e-9."""
+    from oracle import healpix as hp
+    exe = driver("host_hp_patch")
+    delta = np.sqrt(4 * np.pi / (12.0 * (nside_seg << k) ** 2))
+    wcs = np.array([0.9, delta0, delta, rot, 400.0, 300.0])
+    p = np.arange(12 * nside_seg * nside_seg)
+    ix, iy, f = hp.nest2xyf(p, nside_seg)
+    x, y = hp.gnomonic(hp.xyf2vec(ix, iy, f, nside_seg), *wcs)
+    near = p[np.argsort(np.where(np.isfinite(x), np.hypot(x - 400, y - 300), np.inf))[:3]]
+    wcs.tofile(exe.parent / "wcs.bin")
+    near.astype(np.int64).tofile(exe.parent / "segs.bin")
+    _run(exe, "pos", nside_seg, k, "wcs.bin", "segs.bin", "pos.out")
+    o = np.fromfile(exe.parent / "pos.out").reshape(-1, 4)
+    assert len(o) >= 2 * 64 * 32
+    assert np.abs(o[:, :2] - o[:, 2:]).max() <= 20 * delta ** 3 * 21 ** 4 / 24 * (1 + 1 / 16) + 1e-9
+
+
+def test_fixed_point_interpolation(driver):
+    """Four values and fractions of 2^-44 against FP64: one rounding (half an ulp of the result) and the pairs'
+    2^-44 of the largest value, over ten decades, of either sign, ties of values and the ends of a pixel."""
+    exe = driver("host_hp_patch")
+    rng = np.random.default_rng(1)
+    n = 200000
+    q = (rng.normal(size=(n, 4)) * 10.0 ** rng.uniform(-5, 5, (n, 1))).astype(np.float32)
+    q[::5] = (300 + rng.normal(size=(len(q[::5]), 4))).astype(np.float32)
+    q[::7, 1] = q[::7, 0]
+    t = np.floor(rng.random((n, 2)) * 2.0 ** 44) / 2.0 ** 44
+    t[::11, 0], t[::13, 1], t[::17] = 0.0, 0.0, (2.0 ** 44 - 1) / 2.0 ** 44
+    (exe.parent / "lerp.bin").write_bytes(q.tobytes() + t.tobytes())
+    _run(exe, "lerp", "lerp.bin", "lerp.out")
+    v = np.fromfile(exe.parent / "lerp.out", np.float32).astype(np.float64)
+    d = q.astype(np.float64)
+    top, bot = d[:, 0] + t[:, 0] * (d[:, 1] - d[:, 0]), d[:, 2] + t[:, 0] * (d[:, 3] - d[:, 2])
+    ref = top + t[:, 1] * (bot - top)
+    assert (np.abs(v - ref) <= 2.0 ** -24 * np.abs(ref) * 1.0001 + 16 * 2.0 ** -44 * np.abs(d).max(1)).all()
