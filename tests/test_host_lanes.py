@@ -40,19 +40,22 @@ def test_coadd_shifts_stay_in_range(driver, size):
     """Shifts inside the frame split exactly; any other, and any that is not finite, gives a
     window that no tile of the frame finds a pixel in, with coordinates and a union in range."""
     exe = driver("host_coadd_shift")
-    v = np.array([0, -0.25, 0.5, 1, -1, size - 1, -size, size, size + 0.5, -size - 40, 46341, -46341, 65536, 1e9, -1e9, 2147483520,
+    v = np.array([0, -0.25, 0.5, 1, -1, 0.1, -0.3, 0.7123, -1e-9, size - 1, -size, size, size + 0.5, -size - 40, 46341, -46341, 65536, 1e9, -1e9, 2147483520,
                   -2147483648, 3e9, -3e9, 3e38, -3e38, np.inf, -np.inf, np.nan], np.float32)
     v.tofile(exe.parent / "shifts.bin")
     _run(exe, size, "shifts.bin", "shifts.out")
     raw = (exe.parent / "shifts.out").read_bytes()
     n = v.size
     whole, frac = np.frombuffer(raw, np.int32, n), np.frombuffer(raw, np.float32, n, 4 * n)
-    fits = np.frombuffer(raw, np.uint8, n * n, 8 * n).reshape(n, n)
+    weights = np.frombuffer(raw, np.float32, 2 * n, 8 * n).reshape(2, n)
+    fits = np.frombuffer(raw, np.uint8, n * n, 16 * n).reshape(n, n)
     inside = np.abs(v) <= size
     d = v[np.isfinite(v)].astype(np.float64)
     np.testing.assert_array_equal(whole[inside], np.floor(v[inside]))
     np.testing.assert_array_equal(frac[np.isfinite(v)], (d - np.floor(d)).astype(np.float32))
     assert np.isnan(frac[~np.isfinite(v)]).all()
+    f = frac[np.isfinite(v)].astype(np.float64)             # the variances' weights: squares rounded once
+    np.testing.assert_array_equal(weights[:, np.isfinite(v)], np.stack([(1 - f) ** 2, f ** 2]).astype(np.float32))
     # a tile starts in [0, size); its window reaches 32 pixels on
     first, last = whole.astype(np.int64), whole.astype(np.int64) + size - 1 + 31
     assert ((first[~inside] >= size) | (last[~inside] < 0)).all()
