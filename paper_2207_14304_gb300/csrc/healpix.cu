@@ -31,6 +31,7 @@ struct HpArgs {
     uint8_t* cov;
     long long xmax, ymax;      // the frame's last column and row as positions of the patch path
     bool split;                // halves that reach out of the belt are healpix_exact_kernel's
+    double far;                // a half with every node's direction below this along n lies off the frame
 };
 
 __host__ __device__ __forceinline__ void hp_sincospi(double t, double* s, double* c) {
@@ -77,9 +78,9 @@ __host__ __device__ __forceinline__ double2 hp_ring(long long nside, long long j
 }
 
 // Frame position of the centre of pixel (c, r) of a valid segment, `ring` its ring's
-// values.  false when the direction is behind the tangent plane.
+// values, and its direction along n.  false when that is behind the tangent plane.
 __host__ __device__ __forceinline__ bool hp_on_ring(const HpArgs& a, const HpSeg& g, int c, int r, double2 ring, double& x,
-                                                    double& y) {
+                                                    double& y, double& d) {
     const long long jr = g.jr - c - r;
     const bool north = jr < g.nside, south = jr > 3 * g.nside;
     const long long nr = north ? jr : (south ? 4 * g.nside - jr : g.nside);
@@ -91,13 +92,19 @@ __host__ __device__ __forceinline__ bool hp_on_ring(const HpArgs& a, const HpSeg
     double sp, cp;
     hp_sincospi(((double)jp - 0.5 * (double)(kshift + 1)) / (2.0 * (double)nr), &sp, &cp);
     const double v0 = ring.y * cp, v1 = ring.y * sp, v2 = ring.x;
-    const double d = v0 * a.n[0] + v1 * a.n[1] + v2 * a.n[2];
+    d = v0 * a.n[0] + v1 * a.n[1] + v2 * a.n[2];
     if (!(d > 0.0)) return false;
     const double xi = (v0 * a.e[0] + v1 * a.e[1] + v2 * a.e[2]) / d;
     const double eta = (v0 * a.u[0] + v1 * a.u[1] + v2 * a.u[2]) / d;
     x = a.cx + (a.cr * xi + a.sr * eta) * a.inv_scale;
     y = a.cy + (-a.sr * xi + a.cr * eta) * a.inv_scale;
     return true;
+}
+
+__host__ __device__ __forceinline__ bool hp_on_ring(const HpArgs& a, const HpSeg& g, int c, int r, double2 ring, double& x,
+                                                    double& y) {
+    double d;
+    return hp_on_ring(a, g, c, r, ring, x, y, d);
 }
 
 // The same of any segment number; false for one that is no pixel of this NSIDE.
@@ -188,7 +195,7 @@ __host__ __device__ __forceinline__ int hp_node(int j) { return j == 0 ? 0 : (j 
 // position costs three 64-bit additions per coordinate and no FP64: this part does
 // two FP64 operations per clock and SM, and evaluating two FP64 cubics and three
 // FP64 lerps per pixel took 3.80 ms for the 170 segments of a 9576 x 6388 frame; this
-// takes 0.521 ms (the FP64 pipe 46 % busy with nodes and columns, issue slots 61 %).
+// takes 0.525 ms (the FP64 pipe 46 % busy with nodes and columns, issue slots 61 %).
 // The frame pixels under the half (a rectangle around its nodes) are staged in
 // shared memory once, NaN where flagged or not finite: the image axes lie
 // diagonally across the frame, and gathering neighbours from global memory
@@ -196,7 +203,10 @@ __host__ __device__ __forceinline__ int hp_node(int j) { return j == 0 ? 0 : (j 
 // (about 2^-44 relative, then one rounding).  Halves not wholly in the belt (unless
 // `split` leaves them to healpix_exact_kernel), with a node behind the tangent plane or
 // beyond HP_FAR pixels take the exact path per pixel; halves whose rectangle exceeds
-// HP_CAP pixels gather from global memory.
+// HP_CAP pixels gather from global memory.  Halves whose nodes all lie farther from the
+// tangent point than any frame pixel and the patch allow for (HpArgs::far) are zero
+// throughout: segments of the whole sky, most of them behind the plane or far off, cost the
+// exact path otherwise (4 segments of 1024 x 1024: 307 to 442 us, 649 to 807 without).
 constexpr int HP_PATCH = 64, HP_HALF = 32, HP_FRAC = 44, HP_CAP = 10240;
 constexpr double HP_FAR = 500000.0;      // positions in fixed point stay below 2^19
 
@@ -293,7 +303,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
     __shared__ double nd[2][4][4][2];                      // [half][node row][node column][x, y]
     __shared__ long long dif[2][HP_PATCH][4];              // [x, y][column] forward differences of a half
     __shared__ int box[2][4];                              // staged rectangle of a half: x0, y0, x1, y1
-    __shared__ int okh[2];                                 // half: 1 interpolated, 0 exact, 2 not this kernel's
+    __shared__ int okh[2];                                 // half: 1 interpolated, 0 exact, 2 not this kernel's, 3 off the frame
     extern __shared__ float hp_smem[];                     // staged frame pixels
     const int tid = threadIdx.x, lane = tid & 31, col = tid & 63, grp = tid >> 6;
     const int ppr = 1 << (a.k - 6);                        // patches per row
@@ -310,11 +320,13 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
         const int c = c0 + hp_node(jc), r = rp + hf * HP_HALF + hp_node_row(jr);
         const HpSeg g = hp_seg(a, seg);
         const bool belt = hp_in_belt(g, c0, rp + hf * HP_HALF, HP_PATCH, HP_HALF);
-        const bool ok = belt && hp_on_ring(a, g, c, r, hp_ring(g.nside, g.jr - c - r), x, y) && fabs(x) < HP_FAR && fabs(y) < HP_FAR;
+        double d = 1.0;
+        const bool ok = belt && hp_on_ring(a, g, c, r, hp_ring(g.nside, g.jr - c - r), x, y, d) && fabs(x) < HP_FAR && fabs(y) < HP_FAR;
         nd[hf][jr][jc][0] = x;
         nd[hf][jr][jc][1] = y;
         const unsigned half = hf ? 0xffff0000u : 0x0000ffffu;
         const bool all = (__ballot_sync(0xffffffffu, ok) & half) == half;
+        const bool off = (__ballot_sync(0xffffffffu, d < a.far) & half) == half;
         const int xi = ok ? (int)floor(x) : 0, yi = ok ? (int)floor(y) : 0;
         int bx0 = xi, bx1 = xi, by0 = yi, by1 = yi;
         for (int o = 8; o > 0; o >>= 1) {                  // over the half's 16 lanes
@@ -324,7 +336,7 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
             by1 = max(by1, __shfl_xor_sync(0xffffffffu, by1, o));
         }
         if ((lane & 15) == 0) {
-            okh[hf] = all ? 1 : (a.split && !belt ? 2 : 0);
+            okh[hf] = off ? 3 : (all ? 1 : (a.split && !belt ? 2 : 0));
             box[hf][0] = max(bx0 - 1, 0);
             box[hf][1] = max(by0 - 1, 0);
             box[hf][2] = min(bx1 + 2, a.w - 1);
@@ -335,6 +347,14 @@ __global__ void __launch_bounds__(256, 4) healpix_patch_kernel(HpArgs a) {
     for (int hf = 0; hf < 2; hf++) {
         const int r0 = rp + hf * HP_HALF;
         if (okh[hf] == 2) continue;                        // (the same for the whole CTA)
+        if (okh[hf] == 3) {
+            for (int i = 0; i < HP_HALF / 4; i++) {
+                const long e = (long)(r0 + grp * (HP_HALF / 4) + i) * m + c0 + col;
+                out[e] = 0.0f;
+                if (cov) cov[e] = 0;
+            }
+            continue;
+        }
         if (!okh[hf]) {
             for (int i = 0; i < HP_HALF / 4; i++) {
                 const int r = r0 + grp * (HP_HALF / 4) + i;
@@ -481,11 +501,22 @@ __host__ inline void hp_fill_wcs(HpArgs& a, const argus_wcs& w) {
     a.cy = w.cy;
 }
 
-// Whether every pixel of the frame lies in the equatorial belt, |sin(dec)| <= 2/3: the farthest
-// corner's distance from the tangent point bounds every pixel's.
-__host__ inline bool hp_frame_in_belt(const HpArgs& a) {
+// The farthest frame pixel's angle from the tangent point: its farthest corner's.
+__host__ inline double hp_frame_radius(const HpArgs& a) {
     const double dx = std::fmax(std::fabs(a.cx), std::fabs(a.w - 1 - a.cx)), dy = std::fmax(std::fabs(a.cy), std::fabs(a.h - 1 - a.cy));
-    return std::asin(std::fabs(a.n[2])) + std::atan(std::hypot(dx, dy) / a.inv_scale) < std::asin(2.0 / 3.0);
+    return std::atan(std::hypot(dx, dy) / a.inv_scale);
+}
+
+// Whether every pixel of the frame lies in the equatorial belt, |sin(dec)| <= 2/3.
+__host__ inline bool hp_frame_in_belt(const HpArgs& a) {
+    return std::asin(std::fabs(a.n[2])) + hp_frame_radius(a) < std::asin(2.0 / 3.0);
+}
+
+// Where the directions begin that are off the frame with a whole half patch around them: a pixel
+// of a half lies at most 11 columns and 5 rows from a node, steps of at most 1.07 / NSIDE each
+// in the belt.
+__host__ inline double hp_far(const HpArgs& a) {
+    return std::cos(std::fmin(hp_frame_radius(a) + 32.0 / ((double)a.nside_seg * (1 << a.k)), M_PI));
 }
 
 }  // namespace
@@ -512,6 +543,7 @@ extern "C" int argus_healpix_resample(const float* frame, const uint8_t* flags, 
         // them all (a second launch would add 3 us or so to calls of 31); any other frame's halves go to a
         // kernel of their own (at declinations 45 to 80 1.2 to 3.7 times as fast)
         a.split = !hp_frame_in_belt(a);
+        a.far = hp_far(a);
         healpix_patch_kernel<<<(unsigned)patches, 256, smem, (cudaStream_t)stream>>>(a);
         if (a.split) {
             const long m = 1L << k, units = (long)n_seg * (m / HX_ROWS) * (m < HX_COLS ? 1 : m / HX_COLS);

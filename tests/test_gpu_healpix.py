@@ -168,3 +168,34 @@ def test_healpix_halves_out_of_the_belt(ora, nside_seg, k, delta0):
         np.testing.assert_array_equal(cov[i], oc)
         assert np.abs(out[i] - o).max() <= 4 * F32_EPS * float(np.nanmax(frame))
     assert not out[-1].any() and not cov[-1].any()
+
+
+@pytest.mark.parametrize("radius,delta0", [(0.02, 0.3), (0.02, -1.1), (0.3, 0.7), (0.9, -0.2)])
+def test_healpix_segments_of_the_whole_sky(ora, radius, delta0):
+    """All segments of the sky on frames of 1 to 52 degrees' radius: those behind the tangent plane, off the
+    frame, across its edge and on it.  An image pixel is 0.23 degrees (delta) here, and a cubic is off by up to
+    21^4 / 24 times the fourth derivative: that of tan(theta) / scale is at most 24 sec^5, on theta up to a piece (0.25)
+    past the frame's radius, and the HEALPix map's own curvature is given a factor of 4.  Coverage may differ
+    from the oracle's only for pixels nearer than that to the frame's edge."""
+    from oracle import healpix as hp
+    nside, k, w, h = 4, 6, 300, 200
+    scale = math.tan(radius) / math.hypot((w - 1) / 2, (h - 1) / 2)
+    delta = math.sqrt(math.pi / 3) / (nside << k)
+    near = 4 * 24 / math.cos(radius + 0.25) ** 5 * delta ** 4 * 21 ** 4 / 24 / scale
+    assert near < 10
+    wcs = (2.1, delta0, scale, -0.4, (w - 1) / 2, (h - 1) / 2)
+    frame = np.full((h, w), 7.0, np.float32)
+    segs = np.arange(12 * nside * nside, dtype=np.int64)
+    m = 1 << k
+    out = torch.full((segs.size, m, m), -7.0, device="cuda")
+    cov = torch.full((segs.size, m, m), 7, dtype=torch.uint8, device="cuda")
+    B.argus_healpix_resample(dev_pitched(frame), None, B.argus_shape(w, h, pitch_for(w)), wcs, nside, k,
+                             torch.from_numpy(segs).cuda(), segs.size, out, cov)
+    torch.cuda.synchronize()
+    out, cov = out.cpu().numpy(), cov.cpu().numpy()
+    assert cov.any() and (out == np.float32(7.0) * cov).all()
+    for i, s in enumerate(segs):
+        x, y = hp.gnomonic(hp.segment_vectors(int(s), nside, k), *wcs)
+        inside = np.minimum(np.minimum(x, w - 1 - x), np.minimum(y, h - 1 - y))     # > 0: so far inside the frame
+        inside = np.where(np.isfinite(inside), inside, -np.inf)
+        assert cov[i][inside > near].all() and not cov[i][inside < -near].any()
