@@ -393,8 +393,12 @@ int argus_cnn_params(argus_cnn *net, float **master, float **adam_m, float **ada
  *   ARGUS_PREC_BF16_SPLIT  BF16 weights; the forward on the tensor cores
  *                          (tcgen05 implicit GEMMs, FP32 accumulation) with each
  *                          activation split into BF16 hi + lo parts (within
- *                          2^-17 relative of the FP32 value); the backward as
- *                          ARGUS_PREC_BF16.
+ *                          2^-17 relative of the FP32 value); the data gradients
+ *                          likewise, the weight gradients as ARGUS_PREC_BF16.
+ *                          argus_cnn_train_step's own forward sums in another
+ *                          order than argus_cnn_forward (400 stamps: 406 against
+ *                          150 us): outputs differ by FP32 rounding, a step's loss
+ *                          by about 3e-8 of it.
  * The tensor-core forward's bounded device waits latch ARGUS_ERR_TIMEOUT, read
  * by argus_cnn_status. */
 int argus_cnn_set_state(argus_cnn *net, int precision, int step, argus_stream stream);

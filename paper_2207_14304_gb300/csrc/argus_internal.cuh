@@ -95,7 +95,7 @@ int argus_nterms(int deg);
 int argus_cnn_forward_tc(const float* x, const void* wbf, void* wpack, int n, float* y, float* acts, long lstride,
                          int num_sms, int* status, cudaStream_t st);
 size_t argus_cnn_tc_pack_bytes();
-// the same forward with the rounding that a training step's losses keep (cnn_train_tc.cu)
+// the forward of a training step (cnn_train_tc.cu): the same layers, summed in another order
 int argus_cnn_forward_train_tc(const float* x, const void* wbf, void* wpack, int n, float* y, float* acts, long lstride,
                                int num_sms, int* status, cudaStream_t st);
 // the data gradient of 7x7 layer `layer` on the tensor cores (cnn_tc.cu): dh_in =

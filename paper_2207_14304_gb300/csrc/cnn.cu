@@ -19,19 +19,15 @@
 #include <math.h>
 #include <stdlib.h>
 
-#include "argus_internal.cuh"
-#include "tc_ptx.cuh"
+#include "cnn_net.cuh"
 
 namespace {
 
-constexpr int S = 21, NPX = S * S, C = 32, KS = 7, SP = S + KS - 1;   // padded side 27
+using namespace cnn_net;
+
+constexpr int SP = S + KS - 1;                                         // padded side 27
 constexpr int CS = 33;                                                 // padded channel stride
 constexpr int PADSZ = (SP * SP * CS + 3) / 4 * 4;                      // keeps what follows 16-byte aligned
-constexpr long NPARAM = 64 + 32 + 4L * (49 * 1024 + 32) + 32 + 1;
-constexpr long OFF_W1 = 0, OFF_B1 = 64;
-__host__ __device__ constexpr long off_w(int l) { return 96 + (long)l * (49 * 1024 + 32); }
-__host__ __device__ constexpr long off_b(int l) { return off_w(l) + 49 * 1024; }
-constexpr long OFF_W6 = 96 + 4L * (49 * 1024 + 32), OFF_B6 = OFF_W6 + 32;
 
 __device__ __forceinline__ float ld(const float* p, long i) { return p[i]; }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p, long i) { return __bfloat162float(p[i]); }

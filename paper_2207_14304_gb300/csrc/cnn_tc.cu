@@ -54,13 +54,12 @@
 // against W'[ky][kx][o][i] = W[6 - ky][6 - kx][i][o], one layer per launch.
 #include <cuda_bf16.h>
 
-#include "argus_internal.cuh"
-#include "split16.cuh"
-#include "tc_ptx.cuh"
+#include "cnn_net.cuh"
 
 namespace {
 
-constexpr int S = 21, NPX = S * S, C = 32, KS = 7, NTAP = KS * KS;
+using namespace cnn_net;
+
 constexpr int WP = 32;                    // plane row pitch: one warp of lanes
 constexpr int NPP = (S + KS - 1) * WP;    // 864 plane pixels
 constexpr int PLANE = NPP * 16;           // one 8-channel chunk plane (BF16): 13,824 bytes
@@ -73,15 +72,8 @@ constexpr int NG = 4, GC = C / NG;        // channel groups of the epilogue, cha
 constexpr int NEPI = 4 * NG;              // epilogue warps
 constexpr int NTHR = 64 + 32 * NEPI;
 constexpr uint32_t TMEM_COLS = 512;       // two accumulator buffers, 256 columns apart
-constexpr long long WAIT_LIMIT = 2000000000LL;   // ~1 s of SM clock
 // the last tile's rows reach 3 plane rows past the planes: into the next chunk, or the ring
 static_assert((4 * (MT - 1) + KS - 1) * WP + 128 <= NPP + 3 * WP && 3 * WP * 16 <= KYB, "tile reads stay inside the block");
-
-// parameter offsets (the layout of the library's parameter vector)
-constexpr long OFF_W1 = 0, OFF_B1 = 64;
-__host__ __device__ constexpr long off_w(int l) { return 96 + (long)l * (49 * 1024 + 32); }
-__host__ __device__ constexpr long off_b(int l) { return off_w(l) + 49 * 1024; }
-constexpr long OFF_W6 = 96 + 4L * (49 * 1024 + 32), OFF_B6 = OFF_W6 + 32;
 
 struct CnnTcShared {
     alignas(128) uint8_t act[2][SETB];    // operand planes: [hi | lo][chunk][pixel][8 channels]
@@ -94,35 +86,9 @@ struct CnnTcShared {
 };
 static_assert(sizeof(CnnTcShared) + 1024 <= 228 * 1024, "one CTA per SM");
 
-// One try first (the common case), then a bounded wait that also gives up once
-// another role has aborted.
-__device__ __forceinline__ bool wait_or_abort(CnnTcShared& sh, uint64_t* bar, uint32_t parity, int* status) {
-    if (tc::mbar_try_wait(bar, parity)) return true;
-    if (*(volatile int*)&sh.abort) return false;
-    if (!tc::mbar_wait_bounded(bar, parity, WAIT_LIMIT)) {
-        sh.abort = 1;
-        argus_latch(status, ARGUS_ERR_TIMEOUT);
-        return false;
-    }
-    return true;
-}
-
 // The 8 channels of chunk ic of plane pixel P as BF16 hi and lo parts into both operand sets.
 __device__ __forceinline__ void store_chunk(CnnTcShared& sh, int ic, int P, const float (&h)[GC]) {
-    uint32_t hi[4], lo[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const float v0 = h[2 * k], v1 = h[2 * k + 1];
-        hi[k] = bf16x2_rn(v0, v1);
-        lo[k] = bf16x2_rn(v0 - __uint_as_float(hi[k] << 16), v1 - __uint_as_float(hi[k] & 0xffff0000u));
-    }
-    *reinterpret_cast<uint4*>(sh.act[0] + ic * PLANE + P * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<uint4*>(sh.act[1] + ic * PLANE + P * 16) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-}
-
-__device__ __forceinline__ void store_acts(float* dst, const float (&h)[GC]) {
-    reinterpret_cast<float4*>(dst)[0] = make_float4(h[0], h[1], h[2], h[3]);
-    reinterpret_cast<float4*>(dst)[1] = make_float4(h[4], h[5], h[6], h[7]);
+    split_chunk(h, sh.act[0] + ic * PLANE + P * 16, sh.act[1] + ic * PLANE + P * 16);
 }
 
 // Packs the BF16 weights W[l][ky][kx][i][o] of the four 7x7 layers into the
@@ -471,7 +437,7 @@ int argus_cnn_dgrad_tc(const float* dh_out, const float* h_out, const void* wbf,
     return launch_tc<true>(a, num_sms, st);
 }
 
-// The forward outside a training step (whose losses keep the rounding of cnn_train_tc.cu).
+// The forward outside a training step (a step rounds as cnn_train_tc.cu does).
 int argus_cnn_forward_tc(const float* x, const void* wbf, void* wpack, int n, float* y, float* acts, long lstride,
                          int num_sms, int* status, cudaStream_t st) {
     static_assert(sizeof(__nv_bfloat16) == 2, "BF16 storage");

@@ -1,9 +1,12 @@
 // The forward of a training step on the tensor cores: layer 1, the four 7x7 'same'
 // 32 -> 32 convolutions with ReLU and the 1x1 output in one persistent kernel, every tap
 // an MMA of its own (N = 32).  argus_cnn_forward runs the wider kernel of cnn_tc.cu, which
-// takes 0.37 of the time (150 against 406 us for 400 stamps); its sums round in another
-// order, which moves the FP64 loss of a step by 3e-8.  A training step keeps this kernel
-// so that the losses a run records stay the same to 1e-9.
+// takes 0.37 of the time (150 against 406 us for 400 stamps) and whose outputs are within
+// FP32-level rounding of these (half their error against FP64); its sums run in another order.
+// What this kernel is kept for: the loss of one step from given weights keeps the value that recorded
+// steps have, to 1e-9 (the other forward moves it by 3e-8).  It does not make whole runs agree with
+// records: the weight gradients are summed in other orders than they once were, so the weights after a
+// step differ by FP32 rounding, and later losses with them.
 //
 // Implicit GEMM.  A stamp's activations sit in shared memory zero padded to
 // 27 columns (21 + 6) and flattened: plane pixel P = row * 27 + col.  Output q
@@ -37,13 +40,12 @@
 // wait is bounded; a timeout latches ARGUS_ERR_TIMEOUT and all roles stop.
 #include <cuda_bf16.h>
 
-#include "argus_internal.cuh"
-#include "split16.cuh"
-#include "tc_ptx.cuh"
+#include "cnn_net.cuh"
 
 namespace {
 
-constexpr int S = 21, NPX = S * S, C = 32, KS = 7, NTAP = KS * KS;
+using namespace cnn_net;
+
 constexpr int WP = S + KS - 1;            // 27: padded row length
 constexpr int HPR = 28;                   // plane rows: q + 6 * 27 + 6 < 756 for q < 567
 constexpr int NPP = WP * HPR;             // 756 plane pixels
@@ -56,16 +58,9 @@ constexpr int NSLOT = 7;                  // weight ring depth (taps)
 constexpr int NTHR = 192;
 constexpr int NEPI = 128;                 // epilogue threads
 constexpr uint32_t TMEM_COLS = 256;       // 160 used
-constexpr long long WAIT_LIMIT = 2000000000LL;   // ~1 s of SM clock
 static_assert(MT * 128 >= NQ && 4 * 128 < NQ, "five M tiles, the last one overlapping the fourth");
 static_assert(NQ - 1 + (KS - 1) * WP + (KS - 1) < NPP, "the last tile's reads stay inside the planes");
 static_assert(MT * C <= (int)TMEM_COLS, "accumulators fit the allocation");
-
-// parameter offsets (the layout of the library's parameter vector)
-constexpr long OFF_W1 = 0, OFF_B1 = 64;
-__host__ __device__ constexpr long off_w(int l) { return 96 + (long)l * (49 * 1024 + 32); }
-__host__ __device__ constexpr long off_b(int l) { return off_w(l) + 49 * 1024; }
-constexpr long OFF_W6 = 96 + 4L * (49 * 1024 + 32), OFF_B6 = OFF_W6 + 32;
 
 __device__ __forceinline__ int tile_q0(int t) { return t < MT - 1 ? 128 * t : NQ - 128; }
 
@@ -79,39 +74,11 @@ struct CnnTcShared {
 };
 static_assert(sizeof(CnnTcShared) + 1024 <= 228 * 1024 / 2, "two CTAs per SM");
 
-// One try first (the common case), then a bounded wait that also gives up once
-// another role has aborted.
-__device__ __forceinline__ bool wait_or_abort(CnnTcShared& sh, uint64_t* bar, uint32_t parity, int* status) {
-    if (tc::mbar_try_wait(bar, parity)) return true;
-    if (*(volatile int*)&sh.abort) return false;
-    if (!tc::mbar_wait_bounded(bar, parity, WAIT_LIMIT)) {
-        sh.abort = 1;
-        argus_latch(status, ARGUS_ERR_TIMEOUT);
-        return false;
-    }
-    return true;
-}
-
 // The 32 channels of plane pixel P as BF16 hi and lo parts into both operand sets.
 __device__ __forceinline__ void store_planes(CnnTcShared& sh, int P, const float (&h)[C]) {
 #pragma unroll
-    for (int ic = 0; ic < C / 8; ic++) {
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const float v0 = h[ic * 8 + 2 * k], v1 = h[ic * 8 + 2 * k + 1];
-            hi[k] = bf16x2_rn(v0, v1);
-            lo[k] = bf16x2_rn(v0 - __uint_as_float(hi[k] << 16), v1 - __uint_as_float(hi[k] & 0xffff0000u));
-        }
-        *reinterpret_cast<uint4*>(sh.act[0] + ic * PLANE + P * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(sh.act[1] + ic * PLANE + P * 16) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    }
-}
-
-__device__ __forceinline__ void store_acts(float* dst, const float (&h)[C]) {
-#pragma unroll
-    for (int k = 0; k < C / 4; k++)
-        reinterpret_cast<float4*>(dst)[k] = make_float4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
+    for (int ic = 0; ic < C / 8; ic++)
+        split_chunk(h + ic * 8, sh.act[0] + ic * PLANE + P * 16, sh.act[1] + ic * PLANE + P * 16);
 }
 
 // Packs the BF16 weights W[l][ky][kx][i][o] of the four 7x7 layers into the

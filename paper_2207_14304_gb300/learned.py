@@ -39,9 +39,11 @@ class _DevArray:
 
 
 class KernelNet:
-    """precision: "bf16_split" (BF16 weights, the forward on the tensor cores with
-    activations as BF16 hi + lo parts), "bf16" (BF16 weights, CUDA-core kernels) or
-    "fp32"; the backward runs on the CUDA cores in every mode."""
+    """precision: "bf16_split" (BF16 weights, the forward and the data gradients on the
+    tensor cores with activations and gradients as BF16 hi + lo parts), "bf16" (BF16
+    weights, CUDA-core kernels) or "fp32"; the weight gradients run on the CUDA cores in
+    every mode.  A training step's forward in "bf16_split" rounds differently from
+    `forward` (FP32 level)."""
 
     def __init__(self, device=0, max_batch=1024, seed=1, precision="bf16_split"):
         self.device = torch.device("cuda", device)
