@@ -47,10 +47,10 @@ BYTES_PER_PX = 2 + 4 + 4 + 1 + 4 + 4 + 4 + 4 + 1
 # launch, scaled by pixels to the frame (the kernel streams its bands once, so traffic
 # grows in proportion).  It holds only for the kernel sources it was taken on (None
 # until a capture of these sources is recorded here).
-SUBTRACT_TRAFFIC = {"bytes_per_px": 11.4422, "sources_sha1": "b88d70334bc10c960f3a5630a72c35fb9f6525bc",
+SUBTRACT_TRAFFIC = {"bytes_per_px": 11.5500, "sources_sha1": "2e6be4e336cc858fb6620a756ca01ed275aa8c5d",
                     "sources": ("subtract_tc.cu", "subtract_tile.cuh", "tc_ptx.cuh")}
 # the same for the difference-variance kernel (V_I, V_ref and flags in, V_D out)
-VARIANCE_TRAFFIC = {"bytes_per_px": 11.4747, "sources_sha1": "9332ad8c9b092988cc87fafc1738f66d06951598",
+VARIANCE_TRAFFIC = {"bytes_per_px": 11.4757, "sources_sha1": "8b8b219e3c24f56c325e89b1aca15c3f92e57c87",
                     "sources": ("subtract_tc.cu", "subtract_tile.cuh", "tc_ptx.cuh", "subtract.cu")}
 
 
