@@ -247,6 +247,47 @@ __device__ __forceinline__ void fft_tail(C (&v)[8], const TW& tw, C*& s0, C*& s1
     }
 }
 
+// Two sequences of a lane side by side: one barrier serves both crossings, and each one's
+// arithmetic hides the other's latency.
+template <int T, int STEP, int ST, typename C>
+__device__ __forceinline__ void cross2(C (&v)[8], C (&w)[8], C*& v0, C*& v1, C*& w0, C*& w1, int lane) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const int to = cross_to<T, STEP>(lane, i) * ST;
+        v0[to] = v[i];
+        w0[to] = w[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 8; m++) {
+        const int from = pad(lane + m * (T / 8)) * ST;
+        v[m] = v0[from];
+        w[m] = w0[from];
+    }
+    C* t = v0;
+    v0 = v1;
+    v1 = t;
+    t = w0;
+    w0 = w1;
+    w1 = t;
+}
+template <int T, int S, int ST, typename C, typename TW>
+__device__ __forceinline__ void fft_reg2(C (&v)[8], C (&w)[8], const TW& tw, C*& v0, C*& v1, C*& w0, C*& w1, int lane) {
+    dft8<S>(v);
+    dft8<S>(w);
+    cross2<T, 0, ST>(v, w, v0, v1, w0, w1, lane);
+    pass<T, S, 1>(v, tw);
+    pass<T, S, 1>(w, tw);
+    cross2<T, 1, ST>(v, w, v0, v1, w0, w1, lane);
+    pass<T, S, 2>(v, tw);
+    pass<T, S, 2>(w, tw);
+    if constexpr (T == 1024) {
+        cross2<T, 2, ST>(v, w, v0, v1, w0, w1, lane);
+        pass<T, S, 3>(v, tw);
+        pass<T, S, 3>(w, tw);
+    }
+}
+
 template <int T, int S, int ST, typename C, typename TW>
 __device__ __forceinline__ void fft_reg(C (&v)[8], const TW& tw, C*& s0, C*& s1, int lane) {
     dft8<S>(v);

@@ -25,7 +25,7 @@
 // too, and D's error was 1.25 times as large.  S has an inverse column of its own, free of
 // D's rounding.  The PSF transforms are FP64 so that the floor decisions and the small
 // transforms near it are those of an FP64 reference; the images and the
-// filters are FP32.  216 tiles of 512^2 with a PSF pair each: 3.45 ms, against
+// filters are FP32.  216 tiles of 512^2 with a PSF pair each: 3.35 ms, against
 // 12.9 ms with whole FP64 2-D transforms and a combine pass over mirrored pairs.
 #include "argus_internal.cuh"
 #include "fft.cuh"
@@ -39,7 +39,7 @@ struct argus_proper_plan {
     int max_tiles;
     int psf_tiles;          // ZOGY PSF transforms the plan holds: that many tiles', -1 one shared pair, 0 none
     unsigned char* pool;    // pool_bytes() of scratch: see zogy_layout and run_coadd
-    double* psd;            // [max_tiles][T / (2 CB)] partial sums of |P_D(k)|^2
+    double* psd;            // [max_tiles][zogy_blocks] partial sums of |P_D(k)|^2
     float2* tw32;           // [T] e^{-2 pi i m / T}
     double2* tw64;
 };
@@ -346,7 +346,7 @@ struct ZArgs {
     const double* top2;       // [psf tile][T / 2 + 1][T] max(|Pn|^2, |Pr|^2)
     float2* z;                // rows of N + i R in; half-inverted D, S out (the form row_inv_real takes)
     float2* zp;               // half-inverted P_D in columns up to T/2, or null
-    double* psd;              // [tile][T / (2 CB)]
+    double* psd;              // [tile][zogy_blocks]
     const float2* tw;
     double* sigma_S;
 };
@@ -356,9 +356,9 @@ __host__ __device__ __forceinline__ float zogy_FD(argus_zogy_tile tp) {
 }
 
 // D, S and P_D at one frequency k from A = Z(k) and B = Z(-k), Z = DFT[N + i R], and the PSFs'
-// transforms there; 0 under the floor (above = false).  Returns |P_D|^2.  Host-callable, so a
-// CPU driver can run the same code.
-__host__ __device__ __forceinline__ double zogy_point(float2 A, float2 B, float2 pn, float2 pr, bool above, argus_zogy_tile tp,
+// transforms there; 0 under the floor (above = false).  Host-callable, so a CPU driver can run
+// the same code.
+__host__ __device__ __forceinline__ void zogy_point(float2 A, float2 B, float2 pn, float2 pr, bool above, argus_zogy_tile tp,
                                                       float FD, float2& Dh, float2& Sh, float2& PD) {
     // N = (A + conj B) / 2, R = (A - conj B) / 2i
     const float2 Nh = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y - B.y));
@@ -376,7 +376,6 @@ __host__ __device__ __forceinline__ double zogy_point(float2 A, float2 B, float2
         PD = make_float2(g * (pr.x * pn.x - pr.y * pn.y), g * (pr.x * pn.y + pr.y * pn.x));
     }
     Sh = make_float2(FD * (Dh.x * PD.x + Dh.y * PD.y), FD * (Dh.y * PD.x - Dh.x * PD.y));
-    return (double)PD.x * PD.x + (double)PD.y * PD.y;
 }
 
 // X + i Y, and its value at -k for X, Y the transforms of real images.
@@ -391,7 +390,8 @@ __host__ __device__ __forceinline__ float2 plus_i_mirror(float2 X, float2 Y) { r
     const double2 Pr = make_double2(0.5 * (C.y + E.y), -0.5 * (C.x - E.x));
     const double mn = Pn.x * Pn.x + Pn.y * Pn.y, mr = Pr.x * Pr.x + Pr.y * Pr.y;
     float2 Dh, Sh;
-    p2 = zogy_point(A, B, f2(Pn), f2(Pr), mn >= eps2 || mr >= eps2, tp, zogy_FD(tp), Dh, Sh, PD);
+    zogy_point(A, B, f2(Pn), f2(Pr), mn >= eps2 || mr >= eps2, tp, zogy_FD(tp), Dh, Sh, PD);
+    p2 = (double)PD.x * PD.x + (double)PD.y * PD.y;
     Wq = plus_i(Dh, Sh);
     Wp = plus_i_mirror(Dh, Sh);
 }
@@ -432,97 +432,86 @@ __global__ void __launch_bounds__(PSEQ * fft::Reg<T>::LANES) zogy_psf_cols_kerne
     }
 }
 
-// Columns of the tiles: forward, quotient, inverse.  A thread takes column kx < T/2 and its
-// mirror T - kx (column 0 and column T/2, each its own mirror, go together); after the
-// forward transforms the mirror crosses through shared memory, as Z(-k) lies in it at -ky.
-// Its loads bound it with the 16 warps an SM that 128 registers leave (216 tiles of 512: 597
-// us; a column per thread, with twice as many inverse transforms and stores, 830).
-// Grid n_tiles * T / (2 CB).
+// Columns of the tiles: forward, quotient, inverse.  A thread takes column kx and its mirror
+// T - kx (columns 0 and T/2, each its own mirror, alone); after the forward transforms the
+// mirror crosses through shared memory, as Z(-k) lies in it at -ky.  The two sequences go
+// through a transform side by side.  sum |P_D|^2: a thread's 16 exact squares as an unevaluated
+// FP32 pair (at most 2^-44 of it off), FP64 over the threads; sigma_S's error against 64 bits, 3e-8 to
+// 6e-8 from P_D in FP32, is that of FP64 sums, which cost 0.1 ms (two operations per clock and
+// SM).  Its loads bound it with the 16 warps an SM that 128 registers leave.  216 tiles of
+// 512 with kept PSFs, the whole call: 0.91 ms; with a column per thread, twice as many inverse
+// transforms and stores, 1.39.  Grid n_tiles * zogy_blocks<T>().
+template <int T> __host__ __device__ constexpr int zogy_blocks() { return T / (2 * fft::Reg<T>::CB) + 1; }
+
 template <int T>
 __global__ void __launch_bounds__(fft::Reg<T>::THREADS, min_ctas<T>()) zogy_col_kernel(ZArgs a) {
     using Rg = fft::Reg<T>;
-    constexpr int CB = Rg::CB, L = Rg::LANES, NB = T / (2 * CB), HW = T / 2 + 1;
+    constexpr int CB = Rg::CB, L = Rg::LANES, NB = zogy_blocks<T>(), HW = T / 2 + 1;
     extern __shared__ __align__(16) unsigned char fft_smem[];
     float2* sm = reinterpret_cast<float2*>(fft_smem);
     __shared__ double red[Rg::THREADS / 32];
     const int c = threadIdx.x % CB, lane = threadIdx.x / CB;
     const int t = blockIdx.x / NB, xb = blockIdx.x - t * NB, kx = xb * CB + c;
-    const bool self = kx == 0;
-    float2* zk = a.z + (long)t * T * T + blocked<T>(lane, kx);
-    float2* zm = a.z + (long)t * T * T + blocked<T>(lane, self ? T / 2 : T - kx);
+    const bool live = kx <= T / 2, self = kx == 0 || kx == T / 2;
+    float2* zk = a.z + (long)t * T * T + blocked<T>(lane, live ? kx : 0);
+    float2* zm = a.z + (long)t * T * T + blocked<T>(lane, live && !self ? T - kx : 0);
     const fft::TwReg<T> tw(a.tw, lane);
-    float2* b0 = sm + c;
-    float2* b1 = sm + CB * Rg::PT + c;
+    float2* v0 = sm + c;                                   // two buffers for each of the two sequences
+    float2* v1 = v0 + CB * Rg::PT;
+    float2* w0 = v1 + CB * Rg::PT;
+    float2* w1 = w0 + CB * Rg::PT;
     const argus_zogy_tile tp = a.tiles[t];
     const float FD = zogy_FD(tp);
-    const long sp = ((a.psf_tiles == 1 ? 0L : (long)t) * HW + kx) * T + lane;
+    const long sp = ((a.psf_tiles == 1 ? 0L : (long)t) * HW + (live ? kx : 0)) * T + lane;
     float2 v[8], w[8], P[8];
 #pragma unroll
-    for (int m = 0; m < 8; m++) w[m] = zm[m * L * CB];
+    for (int m = 0; m < 8; m++) w[m] = live && !self ? zm[m * L * CB] : make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int m = 0; m < 8; m++) v[m] = zk[m * L * CB];
+    for (int m = 0; m < 8; m++) v[m] = live ? zk[m * L * CB] : make_float2(0.0f, 0.0f);
     // the PSF transforms are wanted after these: on their way to the L2 now (registers leave no
     // room to load them ahead)
     if (lane % 8 == 0) {
 #pragma unroll
         for (int m = 0; m < 8; m++) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.spec + sp + m * L));
     }
-    fft::fft_reg<T, -1, CB>(w, tw, b0, b1, lane);
-    fft::fft_reg<T, -1, CB>(v, tw, b0, b1, lane);
+    fft::fft_reg2<T, -1, CB>(v, w, tw, v0, v1, w0, w1, lane);
 #pragma unroll
-    for (int m = 0; m < 8; m++) b0[fft::pad(lane + m * L) * CB] = w[m];
+    for (int m = 0; m < 8; m++) w0[fft::pad(lane + m * L) * CB] = self ? v[m] : w[m];
     __syncthreads();
-    if (xb == 0) {                                         // the same for every thread
+    float hs = 0.0f, ls = 0.0f;
 #pragma unroll
-        for (int m = 0; m < 8; m++) b1[fft::pad(lane + m * L) * CB] = v[m];
-        __syncthreads();
-    }
-    double psd = 0.0;
-    const auto point = [&](float2 A, float2 B, long e, float2& D, float2& S, float2& PD) {
-        const float4 q = __ldg(a.spec + e);
+    for (int m = 0; m < 8; m++) {
+        const float4 q = __ldg(a.spec + sp + m * L);
         const float2 pn = make_float2(q.x, q.y), pr = make_float2(q.z, q.w);
         // the floor: FP32 moduli decide except next to it, where the FP64 one does
         const float m2 = fmaxf(pn.x * pn.x + pn.y * pn.y, pr.x * pr.x + pr.y * pr.y);
         bool above = m2 > a.hi2;
-        if (!above && !(m2 < a.lo2)) above = __ldg(a.top2 + e) >= a.eps2;
-        psd += zogy_point(A, B, pn, pr, above, tp, FD, D, S, PD);
-    };
+        if (!above && !(m2 < a.lo2)) above = __ldg(a.top2 + sp + m * L) >= a.eps2;
+        float2 D;
+        zogy_point(v[m], w0[fft::pad((T - lane - m * L) & (T - 1)) * CB], pn, pr, above, tp, FD, D, w[m], P[m]);
+        v[m] = self ? plus_i(D, w[m]) : D;                 // columns 0 and T/2: X + i Y, whose inverse is real and real
 #pragma unroll
-    for (int m = 0; m < 8; m++) {
-        const int at = fft::pad((T - lane - m * L) & (T - 1)) * CB;
-        const long e = sp + m * L;
-        float2 D, S, PD;
-        if (!self) {
-            point(v[m], b0[at], e, D, S, PD);
-            v[m] = D;
-            w[m] = S;
-            P[m] = PD;
-        } else {                                           // X + i Y of columns 0 and T/2, whose inverses are real
-            float2 PH;
-            point(v[m], b1[at], e, D, S, PD);
-            v[m] = plus_i(D, S);
-            point(w[m], b0[at], e + (long)(T / 2) * T, D, S, PH);
-            w[m] = plus_i(D, S);
-            P[m] = plus_i(PD, PH);
+        for (int i = 0; i < 2; i++) {                      // exact square, two-sum into the pair
+            const float d = i ? P[m].y : P[m].x, h = d * d, e2 = fmaf(d, d, -h), n = hs + h, b = n - hs;
+            ls += e2 + ((hs - (n - b)) + (h - b));
+            hs = n;
         }
     }
-    if (!self) psd *= 2.0;                                 // k and -k
+    double psd = live ? ((double)hs + (double)ls) * (self ? 1.0 : 2.0) : 0.0;      // k and -k
     for (int o = 16; o > 0; o >>= 1) psd += __shfl_xor_sync(0xffffffffu, psd, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = psd;
-    if (xb == 0) __syncthreads();                          // b1 is read
-    fft::fft_reg<T, 1, CB>(v, tw, b1, b0, lane);           // (barriers: red is complete after it, b0 read before it is written)
+    // (barriers: red is complete after it, and w0 is read before it is written)
+    fft::fft_reg2<T, 1, CB>(v, w, tw, v1, v0, w1, w0, lane);
 #pragma unroll
-    for (int m = 0; m < 8; m++) zk[m * L * CB] = v[m];
-    fft::fft_reg<T, 1, CB>(w, tw, b1, b0, lane);
-#pragma unroll
-    for (int m = 0; m < 8; m++) zm[m * L * CB] = w[m];
+    for (int m = 0; m < 8; m++) {
+        if (live) zk[m * L * CB] = v[m];
+        if (live && !self) zm[m * L * CB] = w[m];
+    }
     if (a.zp) {
-        fft::fft_reg<T, 1, CB>(P, tw, b1, b0, lane);
+        fft::fft_reg<T, 1, CB>(P, tw, v1, v0, lane);
 #pragma unroll
-        for (int m = 0; m < 8; m++) {
-            a.zp[zk - a.z + m * L * CB] = self ? make_float2(P[m].x, 0.0f) : P[m];
-            if (self) a.zp[zm - a.z + m * L * CB] = make_float2(P[m].y, 0.0f);
-        }
+        for (int m = 0; m < 8; m++)
+            if (live) a.zp[zk - a.z + m * L * CB] = P[m];
     }
     if (threadIdx.x == 0) {
         double r = 0.0;
@@ -535,7 +524,7 @@ template <int T>
 __global__ void zogy_sigma_kernel(ZArgs a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.n_tiles) return;
-    constexpr int NB = T / (2 * fft::Reg<T>::CB);
+    constexpr int NB = zogy_blocks<T>();
     const argus_zogy_tile tp = a.tiles[t];
     const double Fn = tp.Fn, Fr = tp.Fr, sn = tp.sn, sr = tp.sr;
     const double FD = Fr * Fn / sqrt(sn * sn * Fr * Fr + sr * sr * Fn * Fn);
@@ -598,7 +587,7 @@ int run(argus_proper_plan* p, ZArgs& a, const RowArgs& rows, const PsfArgs* psf,
     r.tw = p->tw32;
     r.z = a.z;
     launch_rows<T>(r, 1, s);
-    zogy_col_kernel<T><<<(unsigned)a.n_tiles * (T / (2 * Rg::CB)), Rg::THREADS, img_smem<T>(), s>>>(a);
+    zogy_col_kernel<T><<<(unsigned)a.n_tiles * zogy_blocks<T>(), Rg::THREADS, 2 * img_smem<T>(), s>>>(a);
     argus_count_launch(1);
     launch_inv_real<T>(a.z, D, S, a.n_tiles, p->tw32, s);
     if (PD) launch_inv_real<T>(a.zp, PD, nullptr, a.n_tiles, p->tw32, s);
@@ -1002,7 +991,7 @@ template <int T>
 bool set_smem() {
     const size_t i = img_smem<T>(), p = psf_smem<T>();
     return dyn_smem(row_fwd_kernel<T>, i) && dyn_smem(row_inv_kernel<T>, i) &&
-           dyn_smem(row_inv_real_kernel<T, true>, i) && dyn_smem(row_inv_real_kernel<T, false>, i) && dyn_smem(zogy_col_kernel<T>, i) &&
+           dyn_smem(row_inv_real_kernel<T, true>, i) && dyn_smem(row_inv_real_kernel<T, false>, i) && dyn_smem(zogy_col_kernel<T>, 2 * i) &&
            dyn_smem(coadd_col_kernel<T>, i) && dyn_smem(psf_rows_kernel<T>, p) && dyn_smem(zogy_psf_cols_kernel<T>, p) &&
            dyn_smem(coadd_psf_cols_kernel<T>, p);
 }
@@ -1021,7 +1010,7 @@ extern "C" int argus_proper_plan_create(int device, int tile, int max_tiles, arg
     p->device = device;
     p->tile = tile;
     p->max_tiles = max_tiles;
-    const size_t parts = (size_t)max_tiles * (tile / (tile == 256 ? 16 : 8));
+    const size_t parts = (size_t)max_tiles * (tile == 256 ? zogy_blocks<256>() : tile == 512 ? zogy_blocks<512>() : zogy_blocks<1024>());
     bool ok = cudaMalloc((void**)&p->pool, pool_bytes(tile, max_tiles)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&p->psd, parts * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&p->tw32, (size_t)tile * sizeof(float2)) == cudaSuccess;
